@@ -842,7 +842,9 @@ int64_t batch_size(wm_hier_t h, WorkSpace& ws, const wm_sample_desc* d, int64_t 
     maxsys = std::max<int64_t>(WM_LANES, (int64_t)(budget / per) / WM_LANES * WM_LANES);
   }
   int64_t per_batch = std::min<int64_t>(nsys, maxsys);
-  if (per_batch > WM_LANES) per_batch = per_batch / WM_LANES * WM_LANES;
+  // whole tiles where a pass takes several batches (one batch takes every system: a
+  // remainder of a few systems would cost a second solve's launches and waits)
+  if (per_batch < nsys && per_batch > WM_LANES) per_batch = per_batch / WM_LANES * WM_LANES;
   return std::max<int64_t>(1, per_batch);
 }
 
