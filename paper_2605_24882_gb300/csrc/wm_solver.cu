@@ -1297,8 +1297,13 @@ int Batch::chunks_for(int N) const {
 
 // row chunks per tile inside the V-cycle (no partial sums there): at least
 // vcycle_rows (16) rows each (two per warp), so that the small coarse levels
-// still spread over the SMs instead of running a few long, latency-bound warps
-int Batch::vcycle_chunks(int N) const { return std::max(1, std::min(64, (N + vcycle_rows - 1) / vcycle_rows)); }
+// still spread over the SMs instead of running a few long, latency-bound warps;
+// 64, or with few tiles as many as give every SM some 32 blocks
+int Batch::vcycle_chunks(int N) const {
+  const int groups = (tiles + kTPW - 1) / kTPW;
+  const int most = std::max(64, 32 * 152 / std::max(1, groups));
+  return std::max(1, std::min(most, (N + vcycle_rows - 1) / vcycle_rows));
+}
 
 // the one-shift tiles of the current batch
 static UniTiles uni_of(const WorkSpace& ws) {
