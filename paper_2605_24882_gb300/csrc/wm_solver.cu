@@ -883,6 +883,10 @@ constexpr int kTailMax = 6;    // smoothing levels of a fused tail
 #define WM_TAIL_WARPS 32
 #endif
 constexpr int kTailWarps = WM_TAIL_WARPS;
+// At most so many tiles: blocks of eight systems.  One block of 32 systems takes 126 us
+// (spheres, p = 2) and 415 us (p = 3) on its SM, one of eight 55 and 131 us; with 4 x 114
+// blocks every SM has three.
+constexpr int kTailSplitTiles = 114;
 struct TailLv {
   int N = 0, W = 0, nu = 0;
   int oz0 = 0, oz1 = 0, orr = -1;   // rows of the two iterates and of r (orr < 0: r in global memory)
@@ -914,20 +918,26 @@ __device__ __forceinline__ void tail_copy(char* dst, const E* src, int n, int ti
   for (int w = tid; w < n * NW; w += nt) d[w] = __ldg(s + w);
 }
 
-template <bool STAGED>
+// LN systems of a tile per block (32, or 8 where there are too few tiles to give every
+// SM one): with LN = 8 a warp works on four rows at once, lane = (row, system).
+template <bool STAGED, int LN>
 __global__ void __launch_bounds__(WM_LANES * kTailWarps, 1)
     k_vcycle_tail(const TailDesc D, const double* __restrict__ sigma, const int* __restrict__ sid,
                   const float* __restrict__ rin, float* __restrict__ zout, const int* __restrict__ tile_active) {
   extern __shared__ __align__(16) float sh[];
-  const int t = blockIdx.x;
+  constexpr int SPL = WM_LANES / LN;      // rows of a warp at once
+  constexpr int RST = kTailWarps * SPL;   // rows of the block at once
+  const int t = blockIdx.x / SPL;
   if (!tile_active[t]) return;  // the whole block
-  const int lane = threadIdx.x, wy = threadIdx.y;
-  const int g = t * WM_LANES + lane;
+  const int lane = threadIdx.x % LN;      // system of the block
+  const int row0_ = threadIdx.y * SPL + threadIdx.x / LN;  // first row of this thread
+  const int gl = (int)(blockIdx.x % SPL) * LN + lane;      // system of the tile
+  const int g = t * WM_LANES + gl;
   const float sg = (float)sigma[g];
   const int sd = sid[g];
   char* const tb = reinterpret_cast<char*>(sh) + D.tab0;
   if constexpr (STAGED) {
-    const int tid = wy * WM_LANES + lane, nt = WM_LANES * kTailWarps;
+    const int tid = threadIdx.y * WM_LANES + threadIdx.x, nt = WM_LANES * kTailWarps;
     for (int l = 0; l < D.nl; ++l) {
       const TailLv& L = D.lv[l];
       tail_copy(tb + L.opk, L.pk, L.npk, tid, nt);
@@ -983,8 +993,8 @@ __global__ void __launch_bounds__(WM_LANES * kTailWarps, 1)
       return ld_tr(gp + j);
     }
   };
-  const float* rg = rin + (size_t)t * D.lv[0].N * WM_LANES + lane;
-  auto V = [&](int row0, int i) -> float& { return sh[(row0 + i) * WM_LANES + lane]; };
+  const float* rg = rin + (size_t)t * D.lv[0].N * WM_LANES + gl;
+  auto V = [&](int row0, int i) -> float& { return sh[(row0 + i) * LN + lane]; };
   auto rval = [&](const TailLv& L, int i) { return L.orr < 0 ? rg[(size_t)i * WM_LANES] : V(L.orr, i); };
   // (the entries of a row are loaded UR at a time, then summed in order: one
   // block works a row at a time per warp, so the loads must overlap)
@@ -1017,7 +1027,7 @@ __global__ void __launch_bounds__(WM_LANES * kTailWarps, 1)
   auto cheb = [&](const TailLv& L, int k, int zin, int prev, int out) {
     const float2 cf = L.ctab[sd * WM_MAX_CHEB + k];
     const float c1 = k > 0 ? cf.x : 0.f, c2 = cf.y;
-    for (int i = wy; i < L.N; i += kTailWarps) {
+    for (int i = row0_; i < L.N; i += RST) {
       float aS, aM;
       apply_row(L, zin, i, aS, aM);
       const float ds = dS_at(L, i), dm = dM_at(L, i);
@@ -1030,7 +1040,7 @@ __global__ void __launch_bounds__(WM_LANES * kTailWarps, 1)
   };
   auto transfer = [&](const int32_t* ptr, int optr, const PkTr32* ent, int oent, int nout, int in, int out,
                       bool add) {
-    for (int i = wy; i < nout; i += kTailWarps) {
+    for (int i = row0_; i < nout; i += RST) {
       float acc = 0.f;
       const int j1 = ptr_at(ptr, optr, i + 1);
       int j = ptr_at(ptr, optr, i);
@@ -1061,7 +1071,7 @@ __global__ void __launch_bounds__(WM_LANES * kTailWarps, 1)
     const TailLv& L = D.lv[l];
     {
       const float c2 = L.ctab[sd * WM_MAX_CHEB].y;
-      for (int i = wy; i < L.N; i += kTailWarps) {
+      for (int i = row0_; i < L.N; i += RST) {
         const float ds = dS_at(L, i), dm = dM_at(L, i);
         V(L.oz0, i) = c2 * rval(L, i) / (ds + sg * dm);
       }
@@ -1074,7 +1084,7 @@ __global__ void __launch_bounds__(WM_LANES * kTailWarps, 1)
       c = o;
       o = x;
     }
-    for (int i = wy; i < L.N; i += kTailWarps) {
+    for (int i = row0_; i < L.N; i += RST) {
       float aS, aM;
       apply_row(L, c, i, aS, aM);
       V(D.ores, i) = rval(L, i) - (aS + sg * aM);
@@ -1088,7 +1098,7 @@ __global__ void __launch_bounds__(WM_LANES * kTailWarps, 1)
   // dense coarse solve in float64 with the inverse of the system's shift
   {
     const double* A = D.ainv + (size_t)sd * D.Nc * D.Nc;
-    for (int i = wy; i < D.Nc; i += kTailWarps) {
+    for (int i = row0_; i < D.Nc; i += RST) {
       const double* Ai = A + (size_t)i * D.Nc;
       double acc = 0.0;
       int j = 0;
@@ -1121,8 +1131,8 @@ __global__ void __launch_bounds__(WM_LANES * kTailWarps, 1)
     }
     cur[l] = c;
   }
-  float* zg = zout + (size_t)t * D.lv[0].N * WM_LANES + lane;
-  for (int i = wy; i < D.lv[0].N; i += kTailWarps) zg[(size_t)i * WM_LANES] = V(cur[0], i);
+  float* zg = zout + (size_t)t * D.lv[0].N * WM_LANES + gl;
+  for (int i = row0_; i < D.lv[0].N; i += RST) zg[(size_t)i * WM_LANES] = V(cur[0], i);
 }
 
 // inverse of S_c + sigma M_c for each shift by in-place Gauss–Jordan
@@ -1561,7 +1571,10 @@ static int vcycle_tail(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, 
   D.ozc = row + Cv.N;
   row += 2 * Cv.N;
   D.ainv = ws.ainv.p;
-  const size_t vec = (size_t)row * WM_LANES * sizeof(float);
+  // few tiles: four blocks of eight systems per tile (a block's time is the shared-memory
+  // reads of its rows, about a quarter then)
+  const bool split = bt.tiles <= kTailSplitTiles;
+  const size_t vec = (size_t)row * (split ? 8 : WM_LANES) * sizeof(float);
   // the table area: every array at a 16-byte boundary
   size_t tab = 0;
   auto put = [&](int& off, size_t bytes) {
@@ -1597,17 +1610,17 @@ static int vcycle_tail(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, 
   const int pct = (int)std::min<size_t>(100, (smem + 1024 + per_sm - 1) * 100 / std::max(per_sm, 1));
   const dim3 blk(WM_LANES, kTailWarps);
   float* zo = vb<float>(ws.lvl[l].za);
-  if (staged) {
-    WM_CUDA(cudaFuncSetAttribute(k_vcycle_tail<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    WM_CUDA(cudaFuncSetAttribute(k_vcycle_tail<true>, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
-    WM_LAUNCH(WM_PC_VTAIL, s, k_vcycle_tail<true><<<bt.tiles, blk, smem, s>>>(D, ws.sigma.p, ws.sid.p, rin, zo,
-                                                                                ws.tile_active.p));
-  } else {
-    WM_CUDA(cudaFuncSetAttribute(k_vcycle_tail<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    WM_CUDA(cudaFuncSetAttribute(k_vcycle_tail<false>, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
-    WM_LAUNCH(WM_PC_VTAIL, s, k_vcycle_tail<false><<<bt.tiles, blk, smem, s>>>(D, ws.sigma.p, ws.sid.p, rin, zo,
-                                                                                 ws.tile_active.p));
-  }
+  auto launch = [&](auto* kernel) -> int {
+    WM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    WM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
+    WM_LAUNCH(WM_PC_VTAIL, s, kernel<<<bt.tiles * (split ? 4 : 1), blk, smem, s>>>(D, ws.sigma.p, ws.sid.p, rin, zo,
+                                                                                     ws.tile_active.p));
+    return WM_OK;
+  };
+  if (split)
+    WM_TRY(staged ? launch(k_vcycle_tail<true, 8>) : launch(k_vcycle_tail<false, 8>));
+  else
+    WM_TRY(staged ? launch(k_vcycle_tail<true, WM_LANES>) : launch(k_vcycle_tail<false, WM_LANES>));
   WM_CUDA(cudaGetLastError());
   double fl = 2.0 * Cv.N * Cv.N;
   for (int k = 0; k < nl; ++k) {

@@ -213,3 +213,16 @@ def test_coarse_smoother_degree(wm):
         assert st["n_not_converged"] == 0
         d = u1 - u0
         assert float(torch.sqrt((d * hier.apply_mass(d)).sum() / (u0 * hier.apply_mass(u0)).sum())) < 1e-8
+
+
+def test_fused_coarse_tail_of_many_tiles(wm):
+    # with more than 114 tiles the fused coarse end works on 32 systems per block, not
+    # on eight: the same z as the per-level launches, bound as above
+    hier = wm.Hierarchy(wm.Geometry("sphere", 2, 4), 3)
+    nv = 120 * 32 - 5
+    sg = np.geomspace(0.05, 1e5, nv)
+    r = torch.tensor(random_vectors(22, nv, hier.num_dofs(0)), device="cuda")
+    z1 = hier.vcycle(r, sg, precision="mixed", smoother_degree=2).cpu().numpy()
+    hier.set_schedule(tail_fused=0)
+    z0 = hier.vcycle(r, sg, precision="mixed", smoother_degree=2).cpu().numpy()
+    np.testing.assert_allclose(z1, z0, rtol=0, atol=2e-6 * np.abs(z0).max())
