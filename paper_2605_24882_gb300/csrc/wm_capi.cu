@@ -179,7 +179,8 @@ static void release_level(wm_level& L) {
   L.d_ng_ptr.release(); L.d_ng_idx.release(); L.d_Sdense.release(); L.d_Mdense.release(); L.d_noise_w.release();
   L.d_pk32.release(); L.d_pk64.release(); L.d_P32.release(); L.d_R32.release(); L.d_P64.release();
   L.d_R64.release();
-  L.d_ext.release(); L.d_own.release(); L.d_csm32.release(); L.d_csm64.release(); L.d_csmdf.release();
+  L.d_ext.release(); L.d_own.release(); L.d_csm64.release(); L.d_csmdf.release();
+  L.d_st_ext.release(); L.d_st_done.release(); L.d_st_dext.release(); L.d_st_cols.release();
 }
 
 extern "C" void wm_destroy_hier(wm_hier_t h) {
@@ -647,6 +648,12 @@ static int set_batch_meta(WorkSpace& ws, const wm_schedule& sc, int tiles, const
     }
     grp.push_back(make_int2(t, 1));
   }
+  std::vector<int> tshift(tiles);
+  for (int t = 0; t < tiles; ++t) tshift[t] = si[(size_t)t * WM_LANES];
+  std::vector<int2> sgrp;
+  wm_stream_groups(uni, tshift, sgrp, ws.st_n);
+  WM_TRY(ws.st_groups.alloc(sgrp.size()));
+  WM_CUDA(cudaMemcpyAsync(ws.st_groups.p, sgrp.data(), sgrp.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
   ws.n_uni_groups = (int)grp.size();
   ws.uni_waves = sc.uni_waves;
   if (!grp.empty()) {

@@ -144,8 +144,12 @@ struct wm_level {
   bool sten = false;
   int ELU = 0, ELV = 0, nbu = 0, nbv = 0;
   DevBuf<int32_t> d_ext, d_own;
-  DevBuf<float2> d_csm32;
   DevBuf<double2> d_csm64;
+  // the streaming kernels' form (wm_stream.cu): padded id tables, coefficients
+  // by window row in the order of their use, diagonals by the padded tables
+  DevBuf<int32_t> d_st_ext, d_st_done;
+  DevBuf<float2> d_st_dext;
+  DevBuf<unsigned char> d_st_cols;
   // the same coefficients as float pairs (S_hi, S_lo, M_hi, M_lo) for the
   // double-float residual
   DevBuf<float4> d_csmdf;

@@ -1326,6 +1326,30 @@ static UniTiles uni_of(const WorkSpace& ws) {
   return u;
 }
 
+// the batch's tiles as the streaming kernels take them
+static StreamTiles stream_tiles(const WorkSpace& ws, int tiles) {
+  StreamTiles t;
+  t.tiles = tiles;
+  t.groups = ws.st_groups.p;
+  for (int k = 0; k < 2; ++k) t.n[k] = ws.st_n[k];
+  return t;
+}
+// what every step of the streaming kernels on a level takes
+static StreamArgs stream_args(const wm_hier* h, const WorkSpace& ws, const Batch& bt, const wm_level& L,
+                              const float2* ctab, int cat, cudaStream_t s) {
+  StreamArgs a;
+  a.L = &L;
+  a.np = h->np;
+  a.st = stream_tiles(ws, bt.tiles);
+  a.sigma = ws.sigma.p;
+  a.ctab = ctab;
+  a.sid = ws.sid.p;
+  a.tile_active = ws.tile_active.p;
+  a.cat = cat;
+  a.s = s;
+  return a;
+}
+
 template <typename T>
 static T* vb(VBuf& b);
 template <>
@@ -1371,6 +1395,7 @@ int WorkSpace::reserve(const wm_hier* h, int tiles, int nshift, bool dbl) {
   WM_TRY(rr_ref.alloc(ns));
   size_t nch = (size_t)std::max(64, wm_sten_chunks(h->lv[0], h->np));
   size_t np = (size_t)std::max(tiles, (nshift + WM_LANES - 1) / WM_LANES) * nch * WM_LANES;
+  np = std::max(np, wm_stream_part_max(h->lv[0], h->np, tiles) * WM_LANES);
   for (int k = 0; k < 3; ++k) WM_TRY(part[k].alloc(np));
   WM_TRY(flags.alloc(4));
   WM_TRY(counters.alloc(8));
@@ -1397,6 +1422,7 @@ void WorkSpace::release() {
   lvl.clear();
   sigma.release(); sid.release(); src_of.release(); active.release(); rep.release(); restart.release();
   tile_active.release(); tile_rep.release(); tile_uni.release(); uni_groups.release();
+  st_groups.release();
   rho.release(); alpha.release(); beta.release(); bb.release(); rr.release(); rr_ref.release();
   for (auto& pp : part) pp.release();
   flags.release(); counters.release(); lmax.release(); ainv.release(); shifts.release(); statd.release();
@@ -1683,6 +1709,7 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
       }
     }
   }
+  constexpr bool STREAM = std::is_same<T, float>::value;  // the float steps of stencil levels
   T* res = vb<T>(B.res);
   const int nu = bt.degree_of(l);
   int step_rc = WM_OK;
@@ -1691,11 +1718,28 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
   auto cheb_step = [&](int k, const T* zin, T* zo, bool has_prev, VDots<T>* dd) {
     const T* prev = has_prev ? zo : nullptr;
     if (Lv.sten) {
-      const bool fuse = dd && ws.n_uni_tiles > 0;
-      int e = wm_sten_cheb_step<T>(Lv, h->np, h->p, tiles, k, ws.sigma.p, ctab, ws.sid.p, rin, zin, prev, zo, ta,
-                                   uni_of(ws), csm, s, fuse ? dd->q : nullptr,
-                                   fuse ? dd->prz : nullptr, fuse ? dd->pzq : nullptr);
-      if (fuse) dd->fused = true;
+      int e = WM_OK;
+      if constexpr (STREAM) {
+        StreamArgs a = stream_args(h, ws, bt, Lv, ctab, csm, s);
+        a.kstep = k;
+        a.z = zin;
+        a.r = rin;
+        a.prev = prev;
+        a.out = zo;
+        if (dd) {
+          a.q = dd->q;
+          a.part = dd->prz;
+          a.part2 = dd->pzq;
+          dd->fused = true;
+        }
+        e = wm_stream(h->p, dd ? ST_CHEBDOT : ST_CHEB, a);
+      } else {
+        const bool fuse = dd && ws.n_uni_tiles > 0;
+        e = wm_sten_cheb_step(Lv, h->np, h->p, tiles, k, ws.sigma.p, ctab, ws.sid.p, rin, zin, prev, zo, ta,
+                              uni_of(ws), csm, s, fuse ? dd->q : nullptr, fuse ? dd->prz : nullptr,
+                              fuse ? dd->pzq : nullptr);
+        if (fuse) dd->fused = true;
+      }
       if (e != WM_OK) step_rc = e;
     } else {
       WM_LAUNCH(csm, s, k_cheb_step<T><<<ggrid, kBlk, 0, s>>>(Lv.N, Lv.W, ch, tiles, k, pk, dS, dM, ws.sigma.p,
@@ -1703,21 +1747,30 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
     }
     units(csm, bt, (has_prev ? 4.0 : 3.0) * Tb * Lv.N, 2.0 * Lv.nnz + 8.0 * Lv.N);
   };
-  // pre-smoothing from z = 0; with a stencil form the one-shift tiles do the
-  // first two steps in one pass over r (z1 in za, z2 in zb)
+  // pre-smoothing from z = 0; with a stencil form the float solves (float64: the
+  // one-shift tiles) do the first two steps in one pass over r (z1 in za, z2 in zb)
   T* cur = za;
   T* oth = zb;
   int k1 = 1;
-  if (Lv.sten && ws.n_uni_tiles > 0 && nu >= 2) {
-    WM_TRY(wm_sten_cheb_first2<T>(Lv, h->np, h->p, tiles, ws.sigma.p, ctab, ws.sid.p, rin, za, zb, ta, uni_of(ws),
-                                  csm, s));
-    units(csm, bt, 3.0 * Tb * Lv.N, 2.0 * Lv.nnz + 8.0 * Lv.N);
-    if (ws.n_uni_tiles < tiles) {
-      WM_LAUNCH(csm, s, k_cheb_first<T><<<ggrid, kBlk, 0, s>>>(Lv.N, ch, tiles, rin, dS, dM, ws.sigma.p, ctab,
-                                                               ws.sid.p, za, ta, ws.tile_uni.p));
-      int e = wm_sten_cheb_step<T>(Lv, h->np, h->p, tiles, 1, ws.sigma.p, ctab, ws.sid.p, rin, za, nullptr, zb, ta,
-                                   uni_of(ws), csm, s, nullptr, nullptr, nullptr, true);
-      if (e != WM_OK) return e;
+  if (Lv.sten && (STREAM || ws.n_uni_tiles > 0) && nu >= 2) {
+    if constexpr (STREAM) {
+      StreamArgs a = stream_args(h, ws, bt, Lv, ctab, csm, s);
+      a.z = rin;
+      a.out1 = za;
+      a.out = zb;
+      WM_TRY(wm_stream(h->p, ST_CHEB1, a));
+      units(csm, bt, 3.0 * Tb * Lv.N, 2.0 * Lv.nnz + 8.0 * Lv.N);
+    } else {
+      WM_TRY(wm_sten_cheb_first2(Lv, h->np, h->p, tiles, ws.sigma.p, ctab, ws.sid.p, rin, za, zb, ta, uni_of(ws),
+                                 csm, s));
+      units(csm, bt, 3.0 * Tb * Lv.N, 2.0 * Lv.nnz + 8.0 * Lv.N);
+      if (ws.n_uni_tiles < tiles) {
+        WM_LAUNCH(csm, s, k_cheb_first<T><<<ggrid, kBlk, 0, s>>>(Lv.N, ch, tiles, rin, dS, dM, ws.sigma.p, ctab,
+                                                                 ws.sid.p, za, ta, ws.tile_uni.p));
+        int e = wm_sten_cheb_step(Lv, h->np, h->p, tiles, 1, ws.sigma.p, ctab, ws.sid.p, rin, za, nullptr, zb, ta,
+                                  uni_of(ws), csm, s, nullptr, nullptr, nullptr, true);
+        if (e != WM_OK) return e;
+      }
     }
     std::swap(cur, oth);  // cur = z2, oth = z1
     k1 = 2;
@@ -1732,7 +1785,15 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
   }
   // residual, restriction, coarse correction
   if (Lv.sten) {
-    WM_TRY(wm_sten_residual<T>(Lv, h->np, h->p, tiles, ws.sigma.p, rin, cur, res, ta, uni_of(ws), cre, s));
+    if constexpr (STREAM) {
+      StreamArgs a = stream_args(h, ws, bt, Lv, ctab, cre, s);
+      a.z = cur;
+      a.r = rin;
+      a.out = res;
+      WM_TRY(wm_stream(h->p, ST_RESID, a));
+    } else {
+      WM_TRY(wm_sten_residual(Lv, h->np, h->p, tiles, ws.sigma.p, rin, cur, res, ta, uni_of(ws), cre, s));
+    }
   } else {
     WM_LAUNCH(cre, s, k_residual<T><<<ggrid, kBlk, 0, s>>>(Lv.N, Lv.W, ch, tiles, pk, ws.sigma.p, rin, cur, res,
                                                            ta));
@@ -1864,17 +1925,27 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
   const double drop2 = bt.replace_drop * bt.replace_drop;
   int it = 0, n_rep_total = 0;
   bool df_res = bt.df_residual;
+  constexpr bool STREAM = std::is_same<T, float>::value;
+  const int ch_st = STREAM && L0.sten ? wm_stream_items(L0, h->np, h->p, stream_tiles(ws, tiles)) : ch_op;
   for (it = 1; it <= bt.max_iter; ++it) {
     if (L0.sten) {
-      WM_TRY(wm_sten_apply_pq<T>(L0, h->np, h->p, tiles, ws.sigma.p, p, q, ws.tile_active.p, uni_of(ws),
-                                 ws.part[0].p, s));
+      if constexpr (STREAM) {
+        StreamArgs a = stream_args(h, ws, bt, L0, ws.cheb32.p, WM_PC_APPLY64, s);
+        a.z = p;
+        a.out = q;
+        a.part = ws.part[0].p;
+        WM_TRY(wm_stream(h->p, ST_APPLY, a));
+      } else {
+        WM_TRY(wm_sten_apply_pq(L0, h->np, h->p, tiles, ws.sigma.p, p, q, ws.tile_active.p, uni_of(ws),
+                                ws.part[0].p, s));
+      }
     } else {
       WM_LAUNCH(WM_PC_APPLY64, s, k_apply_pq<T><<<ggrid, kBlk, 0, s>>>(N, L0.W, ch, tiles, rows_of<T>(L0),
                                                                        ws.sigma.p, p, q, ws.tile_active.p,
                                                                        ws.part[0].p));
     }
     units(WM_PC_APPLY64, bt, 2.0 * Tb * N, 4.0 * L0.nnz + 4.0 * N);
-    WM_LAUNCH(WM_PC_SCALAR, s, k_scal_alpha<<<tiles, kSumBlk, 0, s>>>(ch_op, ws.part[0].p, ws.rho.p, ws.active.p,
+    WM_LAUNCH(WM_PC_SCALAR, s, k_scal_alpha<<<tiles, kSumBlk, 0, s>>>(ch_st, ws.part[0].p, ws.rho.p, ws.active.p,
                                                                ws.alpha.p, ws.flags.p));
     WM_LAUNCH(WM_PC_CGVEC, s, k_update_xr<T><<<grid, kBlk, 0, s>>>(N, ch, tiles, ws.alpha.p, p, q, ws.x.p, r,
                                                                    ws.tile_active.p, ws.part[0].p));
@@ -1951,9 +2022,9 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
       WM_TRY(bpx<T>(h, ws, bt, r, &z, s));
     else
       WM_TRY(vcycle<T>(h, ws, bt, 0, r, &z, s, &vd));
-    const int ch_dots = vd.fused ? ch_op : ch;
+    const int ch_dots = vd.fused ? ch_st : ch;
     if (vd.fused) units(WM_PC_SMOOTH0, bt, Tb * N, 4.0 * N);  // q read and the two products
-    if (!vd.fused || ws.n_uni_tiles < tiles) {
+    if (!vd.fused || (!STREAM && ws.n_uni_tiles < tiles)) {
       WM_LAUNCH(WM_PC_CGVEC, s, k_dots_rz_zq<T><<<dim3(ch_dots, tiles), kBlk, 0, s>>>(
                                     N, ch_dots, tiles, r, z, q, ws.tile_active.p, ws.part[1].p, ws.part[2].p,
                                     vd.fused ? ws.tile_uni.p : (const int*)nullptr));

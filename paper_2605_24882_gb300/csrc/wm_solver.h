@@ -79,6 +79,8 @@ struct WorkSpace {
   int n_uni_tiles = 0;        // host count of such tiles in the current batch
   DevBuf<int2> uni_groups;    // runs of at most 8 consecutive such tiles of one shift: (first tile, count)
   int n_uni_groups = 0;
+  DevBuf<int2> st_groups;     // the tiles grouped for the streaming kernels (StreamTiles)
+  int st_n[2] = {0, 0};
   int uni_waves = 4;          // grid target of the one-shift kernels (the hierarchy's schedule)
   DevBuf<double> rho, alpha, beta, bb, rr, rr_ref;
   DevBuf<double> part[3];

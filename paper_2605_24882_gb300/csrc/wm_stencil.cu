@@ -1,14 +1,16 @@
-// Shared-memory stencil kernels for the operator-type steps of the solver.
+// Shared-memory stencil kernels: the operator-type steps of the float64 solves and
+// the true residuals of both precisions (the float solves' steps are the
+// streaming kernels of wm_stream.h).
 //
-// A block owns a BU x BV tile of one patch's local DOF grid for TPB system
-// tiles.  It stages the (BU + 2p) x (BV + 2p) window of the input vector
+// A block owns a BU x BV tile of one patch's local DOF grid for one system
+// tile.  It stages the (BU + 2p) x (BV + 2p) window of the input vector
 // (through the extended grid map: halo cells come from the neighbouring
 // patch, or wrap on the torus) into shared memory, once per block, and every
 // warp then sweeps one column of BV outputs with a (2p+1)-row register window,
 // so each staged value is read from shared memory 2p+1 times instead of each
 // neighbour being fetched from L1/L2 (2p+1)^2 times.  Lane = system, so every
-// staged row is one coalesced 128/256-byte transaction and the row's stencil
-// coefficients (S, M) are warp-uniform loads shared by TPB x 32 systems.
+// staged row is one coalesced 256-byte transaction and the row's stencil
+// coefficients (S, M) are warp-uniform loads shared by the 32 systems.
 // Only the owner patch of a shared DOF computes its row.
 #include <algorithm>
 
@@ -30,165 +32,107 @@ struct BvOf {
   static_assert(value % 2 == 0 && value >= 2, "row pairs of the double-float residual");
 };
 
-template <typename T>
-struct V2;
-template <>
-struct V2<float> {
-  using type = float2;
-};
-template <>
-struct V2<double> {
-  using type = double2;
-};
-
 struct StenGeo {
   int nlu, nlv, ELU, ELV, nbu, nbv, N;
   const int32_t* ext;
   const int32_t* own;
 };
 
-// per-thread dot accumulator (products in T, flushed into double every 16)
-template <typename T>
+// per-thread dot accumulator (blocks of 16 products)
 struct DAcc {
   double d = 0.0;
-  T f = 0;
+  double f = 0;
   int n = 0;
-  __device__ __forceinline__ void add(T v) {
+  __device__ __forceinline__ void add(double v) {
     f += v;
     if (++n == 16) {
-      d += (double)f;
+      d += f;
       f = 0;
       n = 0;
     }
   }
-  __device__ __forceinline__ double get() const { return d + (double)f; }
+  __device__ __forceinline__ double get() const { return d + f; }
 };
 
-// per-block partial sums of the TPB tiles (tiles not in `act` are left untouched:
-// another kernel owns them)
-template <int TPB>
-__device__ __forceinline__ void block_reduce(double (&acc)[TPB], double* part, int t0, int tiles, const bool* act) {
-  __shared__ double red[TPB][BU][32];
-#pragma unroll
-  for (int k = 0; k < TPB; ++k) red[k][threadIdx.y][threadIdx.x] = acc[k];
+// the block's partial sum of tile t
+__device__ __forceinline__ void block_reduce(double acc, double* part, int t) {
+  __shared__ double red[BU][32];
+  red[threadIdx.y][threadIdx.x] = acc;
   __syncthreads();
   if (threadIdx.y == 0) {
+    double s = 0.0;
 #pragma unroll
-    for (int k = 0; k < TPB; ++k) {
-      if (t0 + k >= tiles || !act[k]) continue;
-      double s = 0.0;
-#pragma unroll
-      for (int w = 0; w < BU; ++w) s += red[k][w][threadIdx.x];
-      part[((size_t)(t0 + k) * gridDim.x + blockIdx.x) * 32 + threadIdx.x] = s;
-    }
+    for (int w = 0; w < BU; ++w) s += red[w][threadIdx.x];
+    part[((size_t)t * gridDim.x + blockIdx.x) * 32 + threadIdx.x] = s;
   }
 }
 
 // ---------------------------------------------------------------- epilogues
 // Chebyshev step in three-term form (tiles with per-lane shifts):
 // z_next = z + c1 (z - z_prev) + c2 D^{-1} (r - A z), with c1 = 0 at step 0
-// and z_prev = 0 where has_prev is false; out may alias z_prev
-template <typename T, int TPB>
+// and z_prev = 0 where there is none; out may alias z_prev
 struct ChebEpi {
   static constexpr int NIN = 2;  // r and z_prev of the output rows are staged
-  const T* in[2];                // in[1] = nullptr: z_prev = 0
+  const double* in[2];           // in[1] = nullptr: z_prev = 0
   int N, kstep;
-  const T *dS, *dM;
-  T* out;
+  const double *dS, *dM;
+  double* out;
   const double* sigma;
-  const typename V2<T>::type* ctab;  // (c1, c2) per [shift][step] of this level
+  const double2* ctab;  // (c1, c2) per [shift][step] of this level
   const int* sid;
-  T sg[TPB], c1[TPB], c2[TPB];
-  __device__ __forceinline__ void init(int t0, const bool* act) {
-#pragma unroll
-    for (int k = 0; k < TPB; ++k) {
-      int g = (t0 + k) * 32 + threadIdx.x;
-      sg[k] = c1[k] = c2[k] = 0;
-      if (!act[k]) continue;
-      typename V2<T>::type c = ctab[sid[g] * WM_MAX_CHEB + kstep];
-      c1[k] = kstep == 0 ? (T)0 : c.x;
-      c2[k] = c.y;
-      sg[k] = (T)sigma[g];
-    }
+  double sg, c1, c2;
+  __device__ __forceinline__ void init(int t) {
+    const int g = t * 32 + threadIdx.x;
+    const double2 c = ctab[sid[g] * WM_MAX_CHEB + kstep];
+    c1 = kstep == 0 ? 0.0 : c.x;
+    c2 = c.y;
+    sg = sigma[g];
   }
-  // staged[a][k]: input a of tile k at this output row and lane
-  __device__ __forceinline__ void row(int t0, const bool* act, int i, const T* aS, const T* aM, const T* zc,
-                                      const T (*staged)[TPB]) {
-    T ds = dS[i], dm = dM[i];
-#pragma unroll
-    for (int k = 0; k < TPB; ++k)
-      if (act[k]) {
-        size_t o = ((size_t)(t0 + k) * N + i) * 32 + threadIdx.x;
-        T res = staged[0][k] - (aS[k] + sg[k] * aM[k]);
-        T zp = in[1] ? staged[1][k] : (T)0;
-        out[o] = zc[k] + c1[k] * (zc[k] - zp) + c2[k] * res / (ds + sg[k] * dm);
-      }
+  // staged[a]: input a at this output row and lane
+  __device__ __forceinline__ void row(int t, int i, double aS, double aM, double zc, const double* staged) {
+    const double res = staged[0] - (aS + sg * aM);
+    const double zp = in[1] ? staged[1] : 0.0;
+    out[((size_t)t * N + i) * 32 + threadIdx.x] = zc + c1 * (zc - zp) + c2 * res / (dS[i] + sg * dM[i]);
   }
-  __device__ __forceinline__ void finish(int, int, const bool*) {}
+  __device__ __forceinline__ void finish(int) {}
 };
 
 // residual: res = r - A z
-template <typename T, int TPB>
 struct ResidEpi {
   static constexpr int NIN = 1;  // r staged
-  const T* in[1];
+  const double* in[1];
   int N;
-  const T* r;
-  T* res;
+  double* res;
   const double* sigma;
-  T sg[TPB];
-  __device__ __forceinline__ void init(int t0, const bool* act) {
-#pragma unroll
-    for (int k = 0; k < TPB; ++k) sg[k] = act[k] ? (T)sigma[(t0 + k) * 32 + threadIdx.x] : (T)0;
+  double sg;
+  __device__ __forceinline__ void init(int t) { sg = sigma[t * 32 + threadIdx.x]; }
+  __device__ __forceinline__ void row(int t, int i, double aS, double aM, double, const double* staged) {
+    res[((size_t)t * N + i) * 32 + threadIdx.x] = staged[0] - (aS + sg * aM);
   }
-  __device__ __forceinline__ void row(int t0, const bool* act, int i, const T* aS, const T* aM, const T*,
-                                      const T (*staged)[TPB]) {
-#pragma unroll
-    for (int k = 0; k < TPB; ++k)
-      if (act[k]) {
-        size_t o = ((size_t)(t0 + k) * N + i) * 32 + threadIdx.x;
-        res[o] = staged[0][k] - (aS[k] + sg[k] * aM[k]);
-      }
-  }
-  __device__ __forceinline__ void finish(int, int, const bool*) {}
+  __device__ __forceinline__ void finish(int) {}
 };
 
 // outer apply: q = A p, partial (p, q)
-template <typename T, int TPB>
 struct ApplyEpi {
   static constexpr int NIN = 0;
-  const T* in[1];
+  const double* in[1];
   int N;
-  T* q;
+  double* q;
   const double* sigma;
   double* part;
-  T sg[TPB];
-  DAcc<T> acc[TPB];
-  __device__ __forceinline__ void init(int t0, const bool* act) {
-#pragma unroll
-    for (int k = 0; k < TPB; ++k) sg[k] = act[k] ? (T)sigma[(t0 + k) * 32 + threadIdx.x] : (T)0;
+  double sg;
+  DAcc acc;
+  __device__ __forceinline__ void init(int t) { sg = sigma[t * 32 + threadIdx.x]; }
+  __device__ __forceinline__ void row(int t, int i, double aS, double aM, double zc, const double*) {
+    const double qv = aS + sg * aM;
+    q[((size_t)t * N + i) * 32 + threadIdx.x] = qv;
+    acc.add(zc * qv);
   }
-  __device__ __forceinline__ void row(int t0, const bool* act, int i, const T* aS, const T* aM, const T* zc,
-                                      const T (*)[TPB]) {
-#pragma unroll
-    for (int k = 0; k < TPB; ++k)
-      if (act[k]) {
-        size_t o = ((size_t)(t0 + k) * N + i) * 32 + threadIdx.x;
-        T qv = aS[k] + sg[k] * aM[k];
-        q[o] = qv;
-        acc[k].add(zc[k] * qv);
-      }
-  }
-  __device__ __forceinline__ void finish(int t0, int tiles, const bool* act) {
-    double a[TPB];
-#pragma unroll
-    for (int k = 0; k < TPB; ++k) a[k] = acc[k].get();
-    block_reduce<TPB>(a, part, t0, tiles, act);
-  }
+  __device__ __forceinline__ void finish(int t) { block_reduce(acc.get(), part, t); }
 };
 
 // float64 true residual of flagged systems: r = b - A x, partial ||r||^2
-template <typename Tr, int TPB>
+template <typename Tr>
 struct TrueResEpi {
   static constexpr int NIN = 0;
   const double* in[1];
@@ -198,35 +142,25 @@ struct TrueResEpi {
   Tr* r;
   const double* sigma;
   double* part;
-  double sg[TPB];
-  int src[TPB];
-  bool mine[TPB];
-  double acc[TPB];
-  __device__ __forceinline__ void init(int t0, const bool* act) {
-#pragma unroll
-    for (int k = 0; k < TPB; ++k) {
-      int g = (t0 + k) * 32 + threadIdx.x;
-      sg[k] = act[k] ? sigma[g] : 0.0;
-      src[k] = act[k] ? src_of[g] : -1;
-      mine[k] = act[k] && rep[g];
-      acc[k] = 0.0;
-    }
+  double sg;
+  int src;
+  bool mine;
+  double acc;
+  __device__ __forceinline__ void init(int t) {
+    const int g = t * 32 + threadIdx.x;
+    sg = sigma[g];
+    src = src_of[g];
+    mine = rep[g] != 0;
+    acc = 0.0;
   }
-  __device__ __forceinline__ void row(int t0, const bool*, int i, const double* aS, const double* aM, const double*,
-                                      const double (*)[TPB]) {
-#pragma unroll
-    for (int k = 0; k < TPB; ++k)
-      if (mine[k]) {
-        int s = src[k];
-        double b = s >= 0 ? rhs[((size_t)(s / 32) * N + i) * 32 + (s % 32)] : 0.0;
-        double rt = b - (aS[k] + sg[k] * aM[k]);
-        r[((size_t)(t0 + k) * N + i) * 32 + threadIdx.x] = (Tr)rt;
-        acc[k] += rt * rt;
-      }
+  __device__ __forceinline__ void row(int t, int i, double aS, double aM, double, const double*) {
+    if (!mine) return;
+    const double b = src >= 0 ? rhs[((size_t)(src / 32) * N + i) * 32 + (src % 32)] : 0.0;
+    const double rt = b - (aS + sg * aM);
+    r[((size_t)t * N + i) * 32 + threadIdx.x] = (Tr)rt;
+    acc += rt * rt;
   }
-  __device__ __forceinline__ void finish(int t0, int tiles, const bool* act) {
-    block_reduce<TPB>(acc, part, t0, tiles, act);
-  }
+  __device__ __forceinline__ void finish(int t) { block_reduce(acc, part, t); }
 };
 
 // ---------------------------------------------------------------- the kernel
@@ -239,44 +173,30 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
 
-// coefficient row stride in V2 elements, padded to 16-byte multiples
-template <typename T, int P>
-struct CoefStride {
-  static constexpr int S2 = (2 * P + 1) * (2 * P + 1);
-  static constexpr int value = sizeof(typename V2<T>::type) == 8 ? (S2 + 1) / 2 * 2 : S2;
-};
-
-template <typename T, int P, int TPB, int NIN>
+template <int P, int NIN>
 struct SmemLayout {
   static constexpr int BV = BvOf<P>::value;
-  static constexpr int CU = BU + 2 * P, CV = BV + 2 * P, NC = CU * CV;
-  static constexpr int CS = CoefStride<T, P>::value;
-  static constexpr size_t win = (size_t)TPB * NC * 32 * sizeof(T);
-  static constexpr size_t coef = (size_t)BU * BV * CS * sizeof(typename V2<T>::type);
-  static constexpr size_t rows = (size_t)NIN * TPB * BU * BV * 32 * sizeof(T);
+  static constexpr int CU = BU + 2 * P, CV = BV + 2 * P, NC = CU * CV, S2 = (2 * P + 1) * (2 * P + 1);
+  static constexpr size_t win = (size_t)NC * 32 * sizeof(double);
+  static constexpr size_t coef = (size_t)BU * BV * S2 * sizeof(double2);
+  static constexpr size_t rows = (size_t)NIN * BU * BV * 32 * sizeof(double);
   static constexpr size_t ids = (size_t)(NC + BU * BV) * sizeof(int);
   static constexpr size_t total = win + coef + rows + ids;
 };
 
-template <typename T, int P, int TPB, typename Epi>
-__global__ void __launch_bounds__(BU * 32, sizeof(T) == 4 ? 2 : 1) k_sten(StenGeo G, const typename V2<T>::type* __restrict__ csm,
-                                                  const T* __restrict__ src, int tiles,
-                                                  const int* __restrict__ tile_active, const Epi epi_arg,
-                                                  const int* __restrict__ skip_uni) {
-  constexpr int BV = BvOf<P>::value;
-  static_assert(TPB == 1 || TPB == 2, "tile selection below assumes at most two tiles per block");
-  using C2 = typename V2<T>::type;
-  using LY = SmemLayout<T, P, TPB, Epi::NIN>;
-  constexpr int NIN = Epi::NIN;
-  constexpr int SW = 2 * P + 1;
-  constexpr int CU = LY::CU, NC = LY::NC, CS = LY::CS;
-  constexpr int ROWCH = 32 * sizeof(T) / 16;  // 16-byte chunks per staged row
-  constexpr int COEFCH = CS * sizeof(C2) / 16;  // 16-byte chunks per coefficient row
+template <int P, typename Epi>
+__global__ void __launch_bounds__(BU * 32, 1) k_sten(StenGeo G, const double2* __restrict__ csm,
+                                                     const double* __restrict__ src, int tiles,
+                                                     const int* __restrict__ tile_active, const Epi epi_arg,
+                                                     const int* __restrict__ skip_uni) {
+  using LY = SmemLayout<P, Epi::NIN>;
+  constexpr int BV = LY::BV, NIN = Epi::NIN, SW = 2 * P + 1, CU = LY::CU, NC = LY::NC, S2 = LY::S2;
+  constexpr int ROWCH = 32 * sizeof(double) / 16;  // 16-byte chunks per staged row
   Epi epi = epi_arg;  // per-thread copy (its per-tile fields live in registers)
   extern __shared__ __align__(16) unsigned char smraw[];
-  T* sm = reinterpret_cast<T*>(smraw);
-  C2* scf = reinterpret_cast<C2*>(smraw + LY::win);
-  T* srw = reinterpret_cast<T*>(smraw + LY::win + LY::coef);      // [NIN][TPB][BU*BV][32] epilogue inputs
+  double* sm = reinterpret_cast<double*>(smraw);
+  double2* scf = reinterpret_cast<double2*>(smraw + LY::win);
+  double* srw = reinterpret_cast<double*>(smraw + LY::win + LY::coef);       // [NIN][BU*BV][32] epilogue inputs
   int* sid = reinterpret_cast<int*>(smraw + LY::win + LY::coef + LY::rows);  // [NC] cells, then [BU*BV] rows
   int* srow = sid + NC;
   const int lane = threadIdx.x, w = threadIdx.y;
@@ -286,17 +206,10 @@ __global__ void __launch_bounds__(BU * 32, sizeof(T) == 4 ? 2 : 1) k_sten(StenGe
   b /= G.nbu;
   const int bv = b % G.nbv;
   const int m = b / G.nbv;
-  const int t0 = blockIdx.y * TPB;
-  bool act[TPB];
-  bool any = false;
-#pragma unroll
-  for (int k = 0; k < TPB; ++k) {
-    // skip_uni: tiles with a single shift are done by k_sten_uni
-    act[k] = t0 + k < tiles && tile_active[t0 + k] && !(skip_uni && skip_uni[t0 + k]);
-    any |= act[k];
-  }
-  if (!any) return;
-  epi.init(t0, act);
+  const int t = blockIdx.y;
+  // skip_uni: tiles with a single shift are done by k_sten_uni
+  if (t >= tiles || !tile_active[t] || (skip_uni && skip_uni[t])) return;
+  epi.init(t);
   // phase 0: global DOF of every window cell and every output row of the block
   const int32_t* E = G.ext + (size_t)m * G.ELV * G.ELU;
   const int32_t* OWN = G.own + (size_t)m * G.nlv * G.nlu;
@@ -313,32 +226,23 @@ __global__ void __launch_bounds__(BU * 32, sizeof(T) == 4 ? 2 : 1) k_sten(StenGe
     sid[c] = v;
   }
   __syncthreads();
-  // phase 1: asynchronous copies of the window rows and the coefficient rows
-  for (int c = tid; c < TPB * NC * ROWCH; c += BU * 32) {
-    int part = c % ROWCH, cell = (c / ROWCH) % NC, k = c / (ROWCH * NC);
-    int gi = sid[cell];
-    bool ok = gi >= 0 && (TPB == 1 ? act[0] : (k == 0 ? act[0] : act[TPB - 1]));
-    const T* gp = ok ? src + ((size_t)(t0 + k) * G.N + gi) * 32 + part * (16 / sizeof(T)) : src;
-    cp_async16(sm + ((size_t)k * NC + cell) * 32 + part * (16 / sizeof(T)), gp, ok ? 16 : 0);
+  // phase 1: asynchronous copies of the window rows, the coefficient rows and the outputs' inputs
+  for (int c = tid; c < NC * ROWCH; c += BU * 32) {
+    const int part = c % ROWCH, gi = sid[c / ROWCH];
+    cp_async16(sm + (size_t)c * 2, gi >= 0 ? src + ((size_t)t * G.N + gi) * 32 + part * 2 : src, gi >= 0 ? 16 : 0);
   }
-  for (int c = tid; c < BU * BV * COEFCH; c += BU * 32) {
-    int part = c % COEFCH, o = c / COEFCH;
-    int gi = srow[o];
-    const unsigned char* gp = reinterpret_cast<const unsigned char*>(csm) +
-                              (gi >= 0 ? ((size_t)gi * CS * sizeof(C2) + part * 16) : 0);
-    cp_async16(reinterpret_cast<unsigned char*>(scf) + ((size_t)o * CS * sizeof(C2) + part * 16), gp,
-               gi >= 0 ? 16 : 0);
+  for (int c = tid; c < BU * BV * S2; c += BU * 32) {
+    const int gi = srow[c / S2];
+    cp_async16(scf + c, gi >= 0 ? csm + (size_t)gi * S2 + c % S2 : csm, gi >= 0 ? 16 : 0);
   }
 #pragma unroll
   for (int a = 0; a < NIN; ++a) {  // compile-time input index keeps epi in registers
-    const T* base = epi.in[a];
+    const double* base = epi.in[a];
     if (!base) continue;
-    for (int c = tid; c < TPB * BU * BV * ROWCH; c += BU * 32) {
-      int part = c % ROWCH, o = (c / ROWCH) % (BU * BV), k = c / (ROWCH * BU * BV);
-      int gi = srow[o];
-      bool ok = gi >= 0 && (TPB == 1 ? act[0] : (k == 0 ? act[0] : act[TPB - 1]));
-      const T* gp = ok ? base + ((size_t)(t0 + k) * G.N + gi) * 32 + part * (16 / sizeof(T)) : src;
-      cp_async16(srw + (((size_t)a * TPB + k) * BU * BV + o) * 32 + part * (16 / sizeof(T)), gp, ok ? 16 : 0);
+    for (int c = tid; c < BU * BV * ROWCH; c += BU * 32) {
+      const int part = c % ROWCH, o = c / ROWCH, gi = srow[o];
+      cp_async16(srw + ((size_t)a * BU * BV + o) * 32 + part * 2,
+                 gi >= 0 ? base + ((size_t)t * G.N + gi) * 32 + part * 2 : src, gi >= 0 ? 16 : 0);
     }
   }
   cp_async_wait_all();
@@ -346,50 +250,37 @@ __global__ void __launch_bounds__(BU * 32, sizeof(T) == 4 ? 2 : 1) k_sten(StenGe
   // phase 2: each warp sweeps the column iu with a ring of SW staged rows
   const int iu = bu * BU + w;
   if (iu < G.nlu) {
-    T win[TPB][SW][SW];
+    double win[SW][SW];
 #pragma unroll
     for (int r = 0; r < SW - 1; ++r)
 #pragma unroll
-      for (int du = 0; du < SW; ++du)
-#pragma unroll
-        for (int k = 0; k < TPB; ++k) win[k][r][du] = sm[((size_t)k * NC + r * CU + w + du) * 32 + lane];
+      for (int du = 0; du < SW; ++du) win[r][du] = sm[((size_t)r * CU + w + du) * 32 + lane];
 #pragma unroll
     for (int j = 0; j < BV; ++j) {
       const int rn = j + SW - 1;  // staged row entering the window
 #pragma unroll
-      for (int du = 0; du < SW; ++du)
-#pragma unroll
-        for (int k = 0; k < TPB; ++k) win[k][rn % SW][du] = sm[((size_t)k * NC + rn * CU + w + du) * 32 + lane];
+      for (int du = 0; du < SW; ++du) win[rn % SW][du] = sm[((size_t)rn * CU + w + du) * 32 + lane];
       const int i = srow[j * BU + w];
       if (i >= 0) {
-        const C2* cf = scf + (size_t)(j * BU + w) * CS;
-        T aS[TPB], aM[TPB], zc[TPB];
-#pragma unroll
-        for (int k = 0; k < TPB; ++k) aS[k] = aM[k] = 0;
+        const double2* cf = scf + (size_t)(j * BU + w) * S2;
+        double aS = 0, aM = 0;
 #pragma unroll
         for (int dv = 0; dv < SW; ++dv)
 #pragma unroll
           for (int du = 0; du < SW; ++du) {
-            C2 c = cf[dv * SW + du];
-#pragma unroll
-            for (int k = 0; k < TPB; ++k) {
-              T z = win[k][(j + dv) % SW][du];
-              aS[k] += c.x * z;
-              aM[k] += c.y * z;
-            }
+            const double2 c = cf[dv * SW + du];
+            const double z = win[(j + dv) % SW][du];
+            aS += c.x * z;
+            aM += c.y * z;
           }
+        double stg[NIN > 0 ? NIN : 1];
 #pragma unroll
-        for (int k = 0; k < TPB; ++k) zc[k] = win[k][(j + P) % SW][P];
-        T stg[NIN > 0 ? NIN : 1][TPB];
-#pragma unroll
-        for (int a = 0; a < NIN; ++a)
-#pragma unroll
-          for (int k = 0; k < TPB; ++k) stg[a][k] = srw[(((size_t)a * TPB + k) * BU * BV + j * BU + w) * 32 + lane];
-        epi.row(t0, act, i, aS, aM, zc, stg);
+        for (int a = 0; a < NIN; ++a) stg[a] = srw[((size_t)a * BU * BV + j * BU + w) * 32 + lane];
+        epi.row(t, i, aS, aM, win[(j + P) % SW][P], stg);
       }
     }
   }
-  epi.finish(t0, tiles, act);
+  epi.finish(t);
 }
 
 // ------------------------------------------- operator steps, one shift per tile
@@ -412,41 +303,9 @@ __global__ void __launch_bounds__(BU * 32, sizeof(T) == 4 ? 2 : 1) k_sten(StenGe
 // once for the group: the DOF ids of the window and of the output rows and the
 // combined rows
 // A = S + sigma M (with the Chebyshev weights w = c2 / (dS + sigma dM)), so an
-// output costs one FMA per stencil entry and no division.  The group's tiles
-// then stream through shared-memory stage buffers (cp.async copies of the
-// window and the output rows).  Float p = 2 takes two (the next tile copied
-// while the current one is computed) at the three blocks per SM they allow
-// (measured 153.7 against 154.5 ms per bench step with one buffer at four
-// blocks); p = 3 takes one (two would allow only two blocks per SM, which
-// measured slower).
+// output costs one float64 FMA per stencil entry (the unit that bounds this
+// kernel) and no division.
 enum { UNI_CHEB = 0, UNI_RESID = 1, UNI_APPLY = 2, UNI_CHEBDOT = 3, UNI_CHEB1 = 4 };
-// schedule constants of the one-shift kernel: stage buffers in float, output
-// rows per step of a warp (0: two where the register budget allows), partial
-// sums per output
-#ifndef WM_UNI_NST_F32
-#define WM_UNI_NST_F32 1
-#endif
-#ifndef WM_UNI_NST_F32_P2
-#define WM_UNI_NST_F32_P2 2
-#endif
-#ifndef WM_UNI_RPS
-#define WM_UNI_RPS 1
-#endif
-#ifndef WM_UNI_NACC
-#define WM_UNI_NACC 1
-#endif
-#ifndef WM_UNI_MAXB_F32
-#define WM_UNI_MAXB_F32 4
-#endif
-#ifndef WM_UNI_MAXB_F32_P3
-#define WM_UNI_MAXB_F32_P3 4
-#endif
-// tiles per warp pass of the float p = 2 kernels: 0 = two for the residual and
-// the outer apply (measured faster there, 5.5 vs 6.3 and 5.6 vs 5.8 ms per bench
-// step) and one for the Chebyshev modes (two: 66 vs 62 ms); 1 or 2 = all modes
-#ifndef WM_UNI_TPW
-#define WM_UNI_TPW 0
-#endif
 template <int MODE>
 struct UniCheb {
   static constexpr bool value = MODE == UNI_CHEB || MODE == UNI_CHEBDOT;
@@ -455,113 +314,66 @@ template <int MODE>
 struct UniRows {  // staged 32-system rows per output row
   static constexpr int value = MODE == UNI_CHEBDOT ? 3 : (MODE == UNI_CHEB ? 2 : (MODE == UNI_RESID ? 1 : 0));
 };
-template <typename T, int P, int MODE>
+template <int P, int MODE>
 struct UniLayout {
   static constexpr int BV = BvOf<P>::value;
   static constexpr int CU = BU + 2 * P, CV = BV + 2 * P, NC = CU * CV, S2 = (2 * P + 1) * (2 * P + 1);
-  static constexpr int VEC = 16 / sizeof(T);                  // values per 16-byte load
-  static constexpr int S2P = (S2 + VEC - 1) / VEC * VEC;      // padded combined row length
-  static constexpr int CS = CoefStride<T, P>::value;          // (S, M) row stride of the level tables
+  static constexpr int S2P = (S2 + 1) / 2 * 2;                // padded combined row length
   static constexpr int NR = UniRows<MODE>::value;
   static constexpr int ND = UniCheb<MODE>::value ? 2 : 0;     // staged diagonals dS, dM
-  // tiles per warp pass (one stage buffer each) and stage buffers
-  static constexpr int TPW =
-      (sizeof(T) == 4 && P == 2)
-          ? (WM_UNI_TPW == 0 ? ((MODE == UNI_RESID || MODE == UNI_APPLY) ? 2 : 1) : WM_UNI_TPW)
-          : 1;
-  static constexpr int NST = TPW == 2 ? 2 : (sizeof(T) == 4 ? (P == 2 ? WM_UNI_NST_F32_P2 : WM_UNI_NST_F32) : 1);
-  static constexpr size_t win = (size_t)NC * 32 * sizeof(T);  // window of the input vector
-  static constexpr size_t rows = (size_t)NR * BU * BV * 32 * sizeof(T);  // staged rows of the outputs
-  static constexpr size_t stage = win + rows;
-  // raw (S, M) rows, needed at set-up only: they sit in the last stage buffer
-  static constexpr size_t raw = (size_t)BU * BV * CS * sizeof(typename V2<T>::type);
-  static constexpr size_t last = stage > raw ? stage : raw;
-  static constexpr size_t stages = (NST - 1) * stage + last;
-  static constexpr size_t coef = (size_t)BU * BV * S2P * sizeof(T);  // combined rows
-  static constexpr size_t diag = MODE == UNI_CHEB1 ? (size_t)3 * NC * sizeof(T)  // dS, dM, Dinv of the cells
-                                                   : (size_t)(ND + 1) * BU * BV * sizeof(T);  // dS, dM, w
+  static constexpr size_t win = (size_t)NC * 32 * sizeof(double);  // window of the input vector
+  static constexpr size_t stage = win + (size_t)NR * BU * BV * 32 * sizeof(double);  // and rows of the outputs
+  // raw (S, M) rows, needed at set-up only: they sit in the stage buffer
+  static constexpr size_t raw = (size_t)BU * BV * S2 * sizeof(double2);
+  static constexpr size_t stages = stage > raw ? stage : raw;
+  static constexpr size_t coef = (size_t)BU * BV * S2P * sizeof(double);  // combined rows
+  static constexpr size_t diag = MODE == UNI_CHEB1 ? (size_t)3 * NC * sizeof(double)  // dS, dM, Dinv of the cells
+                                                   : (size_t)(ND + 1) * BU * BV * sizeof(double);  // dS, dM, w
   static constexpr size_t diag16 = (diag + 15) / 16 * 16;
   static constexpr size_t ids = (size_t)(NC + BU * BV) * sizeof(int);
-  // float Chebyshev modes: (row id, weight) of every output as one 8-byte entry
-  static constexpr bool PACK_IW = UniCheb<MODE>::value && sizeof(T) == 4;
-  static constexpr size_t iw = PACK_IW ? (size_t)BU * BV * sizeof(int2) : 0;
-  static constexpr size_t total = stages + coef + diag16 + ids + iw;
+  static constexpr size_t total = stages + coef + diag16 + ids;
   // 16-byte copies of one staged tile: window chunks and row chunks, and per thread
-  static constexpr int ROWCH = 32 * sizeof(T) / 16;
+  static constexpr int ROWCH = 32 * sizeof(double) / 16;
   static constexpr int WCH = NC * ROWCH, RCH = BU * BV * ROWCH;
   static constexpr int WPT = (WCH + BU * 32 - 1) / (BU * 32), RPT = (RCH + BU * 32 - 1) / (BU * 32);
   static_assert(stage % 16 == 0 && raw % 16 == 0 && coef % 16 == 0, "16-byte aligned regions");
-  static_assert(!PACK_IW || (stages + coef + diag16 + ids) % 8 == 0, "8-byte aligned (row id, weight) entries");
-};
-template <typename T>
-struct Vec16;
-template <>
-struct Vec16<float> {
-  using type = float4;
-  static __device__ __forceinline__ float at(const float4& v, int k) {
-    return k == 0 ? v.x : k == 1 ? v.y : k == 2 ? v.z : v.w;
-  }
-};
-template <>
-struct Vec16<double> {
-  using type = double2;
-  static __device__ __forceinline__ double at(const double2& v, int k) { return k == 0 ? v.x : v.y; }
 };
 // blocks per SM that the shared memory allows (with the 2 KB of the partial-sum
-// reduction and the 1 KB the runtime reserves per block), at most four (float)
-// or two (double: its copy offsets and window need the registers); this is
-// also the register budget
-template <typename T, int P, int MODE>
+// reduction and the 1 KB the runtime reserves per block), at most two (the copy
+// offsets and the window need the registers); this is also the register budget
+template <int P, int MODE>
 struct UniMinBlocks {
-  static constexpr size_t per = UniLayout<T, P, MODE>::total + 3 * 1024;
+  static constexpr size_t per = UniLayout<P, MODE>::total + 3 * 1024;
   static constexpr int fit = (int)((228 * 1024) / per);
-  static constexpr int cap = sizeof(T) == 4 ? (P == 3 ? WM_UNI_MAXB_F32_P3 : (UniLayout<T, P, MODE>::TPW == 2 ? 3 : WM_UNI_MAXB_F32)) : 2;
-  static constexpr int value = fit >= cap ? cap : (fit < 1 ? 1 : fit);
+  static constexpr int value = fit >= 2 ? 2 : 1;
 };
-// 4- or 8-byte asynchronous copy through L1 (diagonal entries)
-template <int BYTES>
-__device__ __forceinline__ void cp_async_ca(void* smem, const void* gmem, int src_bytes) {
+// 8-byte asynchronous copy through L1 (diagonal entries)
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem, int src_bytes) {
   unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(sa), "l"(gmem), "n"(BYTES), "r"(src_bytes)
-               : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(sa), "l"(gmem), "r"(src_bytes) : "memory");
 }
 
-template <typename T, int P, int MODE>
-__global__ void __launch_bounds__(BU * 32, UniMinBlocks<T, P, MODE>::value)
-    k_sten_uni(StenGeo G, const typename V2<T>::type* __restrict__ csm, const T* __restrict__ dS,
-               const T* __restrict__ dM, const double* __restrict__ sigma, const typename V2<T>::type* __restrict__ ctab,
-               const int* __restrict__ sid, int kstep, const T* __restrict__ z, const T* __restrict__ r, const T* prev,
-               T* out, int tiles, const int* __restrict__ tile_active, const int2* __restrict__ groups, int split,
-               double* __restrict__ part, const T* __restrict__ qd, double* __restrict__ part2,
-               T* __restrict__ out1) {
-  constexpr int BV = BvOf<P>::value;
-  using C2 = typename V2<T>::type;
-  using LY = UniLayout<T, P, MODE>;
+template <int P, int MODE>
+__global__ void __launch_bounds__(BU * 32, (UniMinBlocks<P, MODE>::value))
+    k_sten_uni(StenGeo G, const double2* __restrict__ csm, const double* __restrict__ dS,
+               const double* __restrict__ dM, const double* __restrict__ sigma, const double2* __restrict__ ctab,
+               const int* __restrict__ sid, int kstep, const double* __restrict__ z, const double* __restrict__ r,
+               const double* prev, double* out, int tiles, const int* __restrict__ tile_active,
+               const int2* __restrict__ groups, int split, double* __restrict__ part, const double* __restrict__ qd,
+               double* __restrict__ part2, double* __restrict__ out1) {
+  using LY = UniLayout<P, MODE>;
   constexpr bool CHEB = UniCheb<MODE>::value;
-  using VT = typename Vec16<T>::type;
-  constexpr int SW = 2 * P + 1, CU = LY::CU, NC = LY::NC, S2 = LY::S2, S2P = LY::S2P, VEC = LY::VEC, CS = LY::CS;
-  constexpr int NR = LY::NR, NST = LY::NST, ROWCH = LY::ROWCH, TPW = LY::TPW;
-  constexpr int RPS = WM_UNI_RPS > 0 ? WM_UNI_RPS : (UniMinBlocks<T, P, MODE>::value >= 3 ? 1 : 2);
-  constexpr int NACC = WM_UNI_NACC;
-  constexpr int RW = SW + RPS - 1;     // rows of the register ring
-  static_assert(BV % RPS == 0, "rows per step divide the block height");
-  constexpr int EPT = 16 / sizeof(T);  // values per 16-byte chunk
-  constexpr int NT = BU * 32;          // threads per block
-  constexpr size_t STAGE = LY::stage / sizeof(T);  // stage buffer length in T
+  constexpr int BV = LY::BV, SW = 2 * P + 1, CU = LY::CU, NC = LY::NC, S2 = LY::S2, S2P = LY::S2P;
+  constexpr int NR = LY::NR, ROWCH = LY::ROWCH;
+  constexpr int NT = BU * 32;  // threads per block
   extern __shared__ __align__(16) unsigned char smraw[];
-  T* const stg = reinterpret_cast<T*>(smraw);  // [NST] x ([NC][32] window, [NR][64][32] rows)
-  C2* const sraw = reinterpret_cast<C2*>(smraw + (NST - 1) * LY::stage);  // [64][CS], set-up only
-  T* const scf = reinterpret_cast<T*>(smraw + LY::stages);                // [64][S2P]
-  T* const sdg = reinterpret_cast<T*>(smraw + LY::stages + LY::coef);     // [ND][64], then w [64]
-  T* const swt = sdg + LY::ND * BU * BV;
+  double* const stg = reinterpret_cast<double*>(smraw);    // [NC][32] window, [NR][BU*BV][32] rows
+  double2* const sraw = reinterpret_cast<double2*>(smraw);  // [BU*BV][S2], set-up only
+  double* const scf = reinterpret_cast<double*>(smraw + LY::stages);             // [BU*BV][S2P]
+  double* const sdg = reinterpret_cast<double*>(smraw + LY::stages + LY::coef);  // [ND][BU*BV], then w
+  double* const swt = sdg + LY::ND * BU * BV;
   int* const sid_ = reinterpret_cast<int*>(smraw + LY::stages + LY::coef + LY::diag16);
   int* const srow = sid_ + NC;
-  int2* const siw = reinterpret_cast<int2*>(smraw + LY::stages + LY::coef + LY::diag16 + LY::ids);  // PACK_IW
   const int lane = threadIdx.x, w = threadIdx.y;
   const int tid = w * 32 + lane;
   int b = blockIdx.x;
@@ -579,21 +391,21 @@ __global__ void __launch_bounds__(BU * 32, UniMinBlocks<T, P, MODE>::value)
   for (int t = ta; t < tb; ++t)
     if (tile_active[t]) todo |= 1u << (t - ta);
   if (todo == 0) return;
-  T sg, c1 = 0, c2 = 0, c20 = 0;
+  double sg, c1 = 0, c2 = 0, c20 = 0;
   {
     const int g = gr.x * 32;  // every system of the group has this shift
     if constexpr (CHEB) {
-      const C2 c = ctab[sid[g] * WM_MAX_CHEB + kstep];
-      c1 = kstep == 0 ? (T)0 : c.x;
+      const double2 c = ctab[sid[g] * WM_MAX_CHEB + kstep];
+      c1 = kstep == 0 ? 0.0 : c.x;
       c2 = c.y;
     }
     if constexpr (MODE == UNI_CHEB1) {  // steps 0 and 1
-      const C2 c0 = ctab[sid[g] * WM_MAX_CHEB], c = ctab[sid[g] * WM_MAX_CHEB + 1];
+      const double2 c0 = ctab[sid[g] * WM_MAX_CHEB], c = ctab[sid[g] * WM_MAX_CHEB + 1];
       c20 = c0.y;
       c1 = c.x;
       c2 = c.y;
     }
-    sg = (T)sigma[g];
+    sg = sigma[g];
   }
   // set-up 1: global DOF of every window cell and every output row
   const int32_t* E = G.ext + (size_t)m * G.ELV * G.ELU;
@@ -612,30 +424,24 @@ __global__ void __launch_bounds__(BU * 32, UniMinBlocks<T, P, MODE>::value)
   }
   __syncthreads();
   // set-up 2: (S, M) rows and diagonals, copy offsets
-  constexpr int RAWCH = CS * (int)sizeof(C2) / 16;  // 16-byte chunks per (S, M) row
-  for (int c = tid; c < BU * BV * RAWCH; c += NT) {
-    const int part16 = c % RAWCH, o = c / RAWCH;
-    const int gi = srow[o];
-    cp_async16(reinterpret_cast<unsigned char*>(sraw) + o * (CS * sizeof(C2)) + part16 * 16,
-               gi >= 0 ? reinterpret_cast<const unsigned char*>(csm + (size_t)gi * CS) + part16 * 16
-                       : reinterpret_cast<const unsigned char*>(csm),
-               gi >= 0 ? 16 : 0);
+  for (int c = tid; c < BU * BV * S2; c += NT) {
+    const int gi = srow[c / S2];
+    cp_async16(sraw + c, gi >= 0 ? csm + (size_t)gi * S2 + c % S2 : csm, gi >= 0 ? 16 : 0);
   }
   if constexpr (MODE == UNI_CHEB1) {  // diagonals of every window cell
     for (int c = tid; c < 2 * NC; c += NT) {
       const int gi = sid_[c % NC];
-      const T* base = c < NC ? dS : dM;
-      cp_async_ca<sizeof(T)>(sdg + c, gi >= 0 ? base + gi : dS, gi >= 0 ? (int)sizeof(T) : 0);
+      const double* base = c < NC ? dS : dM;
+      cp_async8(sdg + c, gi >= 0 ? base + gi : dS, gi >= 0 ? 8 : 0);
     }
   }
   if constexpr (CHEB) {
     for (int c = tid; c < 2 * BU * BV; c += NT) {
       const int gi = srow[c % (BU * BV)];
-      const T* base = c < BU * BV ? dS : dM;
-      cp_async_ca<sizeof(T)>(sdg + c, gi >= 0 ? base + gi : dS, gi >= 0 ? (int)sizeof(T) : 0);
+      const double* base = c < BU * BV ? dS : dM;
+      cp_async8(sdg + c, gi >= 0 ? base + gi : dS, gi >= 0 ? 8 : 0);
     }
   }
-  cp_async_commit();
   // each thread's source offsets (within a tile) of its window and row
   // chunks: -1 zero-fills a cell outside the surface, -2 marks no chunk
   int woff[LY::WPT];
@@ -645,7 +451,7 @@ __global__ void __launch_bounds__(BU * 32, UniMinBlocks<T, P, MODE>::value)
     int o = -2;
     if (c < LY::WCH) {
       const int gi = sid_[c / ROWCH];
-      o = gi >= 0 ? gi * 32 + (c % ROWCH) * EPT : -1;
+      o = gi >= 0 ? gi * 32 + (c % ROWCH) * 2 : -1;
     }
     woff[k] = o;
   }
@@ -656,58 +462,44 @@ __global__ void __launch_bounds__(BU * 32, UniMinBlocks<T, P, MODE>::value)
     int o = -2;
     if (NR > 0 && c < LY::RCH) {
       const int gi = srow[c / ROWCH];
-      o = gi >= 0 ? gi * 32 + (c % ROWCH) * EPT : -1;
+      o = gi >= 0 ? gi * 32 + (c % ROWCH) * 2 : -1;
     }
     roff[k] = o;
   }
-  // the 16-byte copies of tile t into stage buffer `buf` (chunk c of the
-  // window lands at element c * EPT, chunk c of row input a at NC * 32 +
-  // a * 64 * 32 + c * EPT); absent inputs (z_prev, q) are not copied
-  auto issue = [&](int t, T* buf) {
+  // the 16-byte copies of tile t into the stage buffer; absent inputs (z_prev, q) are not copied
+  auto issue = [&](int t) {
     const size_t to = (size_t)t * G.N * 32;
 #pragma unroll
     for (int k = 0; k < LY::WPT; ++k) {
       const int o = woff[k];
-      if (o != -2) cp_async16(buf + (tid + k * NT) * EPT, o >= 0 ? z + to + o : z, o >= 0 ? 16 : 0);
+      if (o != -2) cp_async16(stg + (tid + k * NT) * 2, o >= 0 ? z + to + o : z, o >= 0 ? 16 : 0);
     }
 #pragma unroll
     for (int a = 0; a < NR; ++a) {
-      const T* base = a == 0 ? r : (a == 1 ? prev : qd);
+      const double* base = a == 0 ? r : (a == 1 ? prev : qd);
       if (base == nullptr) continue;
 #pragma unroll
       for (int k = 0; k < LY::RPT; ++k) {
         const int o = roff[k];
         if (o != -2)
-          cp_async16(buf + NC * 32 + a * BU * BV * 32 + (tid + k * NT) * EPT, o >= 0 ? base + to + o : base,
+          cp_async16(stg + NC * 32 + a * BU * BV * 32 + (tid + k * NT) * 2, o >= 0 ? base + to + o : base,
                      o >= 0 ? 16 : 0);
       }
     }
-    cp_async_commit();
   };
-  // tiles go through the stage buffers TPW at a time (a pair shares every load
-  // of the combined rows); with PREFETCH the next tile is copied while the
-  // current one is computed
-  constexpr bool PREFETCH = NST == 2 && TPW == 1;
-  int cur = __ffs(todo) - 1;
-  todo &= todo - 1;
-  if constexpr (PREFETCH) {  // the first tile goes to buffer 0 (the raw rows sit in buffer 1)
-    issue(ta + cur, stg);
-    cp_async_wait<1>();
-  } else {
-    cp_async_wait<0>();
-  }
+  cp_async_wait_all();
   __syncthreads();
-  T* sdc = sdg + 2 * NC;  // UNI_CHEB1: Dinv of every window cell
+  double* sdc = sdg + 2 * NC;  // UNI_CHEB1: Dinv of every window cell
   if constexpr (MODE == UNI_CHEB1) {
-    for (int c = tid; c < NC; c += NT) sdc[c] = sid_[c] >= 0 ? (T)1 / (sdg[c] + sg * sdg[NC + c]) : (T)0;
+    for (int c = tid; c < NC; c += NT) sdc[c] = sid_[c] >= 0 ? 1.0 / (sdg[c] + sg * sdg[NC + c]) : 0.0;
     __syncthreads();
   }
   // set-up 3: combined rows and the Chebyshev diagonal weights
   for (int c = tid; c < BU * BV * S2P; c += NT) {
     const int o = c / S2P, sl = c - o * S2P;
-    T a = 0;
+    double a = 0;
     if (sl < S2) {
-      const C2 q = sraw[o * CS + sl];
+      const double2 q = sraw[o * S2 + sl];
       a = q.x + sg * q.y;
       if constexpr (MODE == UNI_CHEB1)  // times c2_0 Dinv of the neighbour's cell: A z1 from r
         a *= c20 * sdc[((o / BU) + sl / SW) * CU + (o % BU) + sl % SW];
@@ -715,174 +507,73 @@ __global__ void __launch_bounds__(BU * 32, UniMinBlocks<T, P, MODE>::value)
     scf[c] = a;
   }
   if constexpr (CHEB)
-    for (int c = tid; c < BU * BV; c += NT) {
-      const T wc = srow[c] >= 0 ? c2 / (sdg[c] + sg * sdg[BU * BV + c]) : (T)0;
-      swt[c] = wc;
-      if constexpr (LY::PACK_IW) siw[c] = make_int2(srow[c], __float_as_int((float)wc));
-    }
-  __syncthreads();  // the raw rows are dead from here on (buffer 1 may be refilled)
+    for (int c = tid; c < BU * BV; c += NT) swt[c] = srow[c] >= 0 ? c2 / (sdg[c] + sg * sdg[BU * BV + c]) : 0.0;
+  __syncthreads();  // the raw rows are dead from here on
   const int iu = bu * BU + w;
-  int bsel = 0;
-  for (;;) {
-    // the tiles of this pass: tt[u] in buffer u (with PREFETCH, buffer bsel)
-    int tt[TPW];
-    bool ok[TPW];
-    tt[0] = ta + cur;
-    ok[0] = true;
-    if constexpr (TPW == 2) {
-      ok[1] = todo != 0;
-      const int c1 = ok[1] ? __ffs(todo) - 1 : cur;
-      if (ok[1]) todo &= todo - 1;
-      tt[1] = ta + c1;
-    }
-    const bool more = todo != 0;
-    const int nxt = more ? __ffs(todo) - 1 : 0;
-    if constexpr (PREFETCH) {
-      if (more) {
-        issue(ta + nxt, stg + (bsel ^ 1) * STAGE);
-        cp_async_wait<1>();
-      } else {
-        cp_async_wait<0>();
-      }
-    } else {
-      issue(tt[0], stg);
-      if constexpr (TPW == 2)
-        if (ok[1]) issue(tt[1], stg + STAGE);
-      cp_async_wait<0>();
-    }
+  while (todo) {
+    const int t = ta + __ffs(todo) - 1;
+    todo &= todo - 1;
+    issue(t);
+    cp_async_wait_all();
     __syncthreads();
-    // each warp sweeps the column iu, RPS output rows per step, with a ring of
-    // RW staged rows in registers per tile; every output sums its stencil in
-    // NACC partial sums (stencil rows dv mod NACC), and each combined-row load
-    // serves the TPW tiles of the pass
-    const T* smv[TPW];
-    const T* srwv[TPW];
-#pragma unroll
-    for (int u = 0; u < TPW; ++u) {
-      smv[u] = PREFETCH ? stg + bsel * STAGE : stg + ((TPW == 2 && !ok[u]) ? 0 : u) * STAGE;
-      srwv[u] = smv[u] + NC * 32;
-    }
-    DAcc<T> dot[TPW];   // UNI_APPLY: (z, A z); UNI_CHEBDOT: (r, z_new) over this thread's outputs
-    DAcc<T> dot2[TPW];  // UNI_CHEBDOT: (z_new, q)
+    // each warp sweeps the column iu with a ring of SW rows in registers
+    const double* const srw = stg + NC * 32;
+    DAcc dot;   // UNI_APPLY: (z, A z); UNI_CHEBDOT: (r, z_new) over this thread's outputs
+    DAcc dot2;  // UNI_CHEBDOT: (z_new, q)
     if (iu < G.nlu) {
-      T win[TPW][RW][SW];
+      double win[SW][SW];
 #pragma unroll
-      for (int u = 0; u < TPW; ++u)
+      for (int rr = 0; rr < SW - 1; ++rr)
 #pragma unroll
-        for (int rr = 0; rr < SW - 1; ++rr)
+        for (int du = 0; du < SW; ++du) win[rr][du] = stg[(rr * CU + w + du) * 32 + lane];
 #pragma unroll
-          for (int du = 0; du < SW; ++du) win[u][rr][du] = smv[u][(rr * CU + w + du) * 32 + lane];
+      for (int j = 0; j < BV; ++j) {
+        const int rn = j + SW - 1;  // staged row entering the window
 #pragma unroll
-      for (int j = 0; j < BV; j += RPS) {
+        for (int du = 0; du < SW; ++du) win[rn % SW][du] = stg[(rn * CU + w + du) * 32 + lane];
+        const int o = j * BU + w;
+        const int i = srow[o];
+        if (i < 0) continue;  // past the patch's edge or another patch's row
+        double az = 0;
 #pragma unroll
-        for (int e = 0; e < RPS; ++e) {
-          const int rn = j + SW - 1 + e;  // staged rows entering the window
-#pragma unroll
-          for (int u = 0; u < TPW; ++u)
-#pragma unroll
-            for (int du = 0; du < SW; ++du) win[u][rn % RW][du] = smv[u][(rn * CU + w + du) * 32 + lane];
+        for (int q = 0; q < S2P / 2; ++q) {
+          const double2 a = reinterpret_cast<const double2*>(scf + (j * BU + w) * S2P)[q];
+          az = fma(a.x, win[(j + (2 * q) / SW) % SW][(2 * q) % SW], az);
+          if (2 * q + 1 < S2) az = fma(a.y, win[(j + (2 * q + 1) / SW) % SW][(2 * q + 1) % SW], az);
         }
-        T acc[TPW][RPS][NACC];
-#pragma unroll
-        for (int u = 0; u < TPW; ++u)
-#pragma unroll
-          for (int k = 0; k < RPS; ++k)
-#pragma unroll
-            for (int h = 0; h < NACC; ++h) acc[u][k][h] = 0;
-#pragma unroll
-        for (int q = 0; q < S2P / VEC; ++q) {
-          VT a[RPS];
-#pragma unroll
-          for (int k = 0; k < RPS; ++k) a[k] = reinterpret_cast<const VT*>(scf + ((j + k) * BU + w) * S2P)[q];
-#pragma unroll
-          for (int e = 0; e < VEC; ++e) {
-            const int sl = q * VEC + e;
-            if (sl < S2) {
-              const int dv = sl / SW, du = sl % SW;
-#pragma unroll
-              for (int k = 0; k < RPS; ++k)
-#pragma unroll
-                for (int u = 0; u < TPW; ++u)
-                  acc[u][k][dv % NACC] =
-                      fma(Vec16<T>::at(a[k], e), win[u][(j + k + dv) % RW][du], acc[u][k][dv % NACC]);
-            }
+        const double zc = win[(j + P) % SW][P];
+        double res;
+        if constexpr (CHEB) {
+          const double rv = srw[o * 32 + lane];
+          const double zp = prev ? srw[(BU * BV + o) * 32 + lane] : 0.0;
+          res = zc + c1 * (zc - zp) + swt[o] * (rv - az);
+          if constexpr (MODE == UNI_CHEBDOT) {
+            dot.add(rv * res);
+            if (qd) dot2.add(res * srw[(2 * BU * BV + o) * 32 + lane]);
           }
+        } else if constexpr (MODE == UNI_CHEB1) {
+          const double dc = sdc[(j + P) * CU + w + P];  // Dinv of the output row
+          const double z1 = c20 * dc * zc;              // zc is r here
+          out1[((size_t)t * G.N + i) * 32 + lane] = z1;
+          res = z1 + c1 * z1 + c2 * dc * (zc - az);
+        } else if constexpr (MODE == UNI_RESID) {
+          res = srw[o * 32 + lane] - az;
+        } else {
+          res = az;
+          dot.add(zc * az);
         }
-#pragma unroll
-        for (int k = 0; k < RPS; ++k) {
-          const int jj = j + k;
-          const int o = jj * BU + w;
-          int i;
-          T wo = 0;  // the output's Chebyshev weight (one 8-byte load with its row id in float)
-          if constexpr (LY::PACK_IW) {
-            const int2 iw = siw[o];
-            i = iw.x;
-            wo = __int_as_float(iw.y);
-          } else {
-            i = srow[o];
-            if constexpr (CHEB) wo = swt[o];
-          }
-          if (i < 0) continue;
-#pragma unroll
-          for (int u = 0; u < TPW; ++u) {
-            if (!ok[u]) continue;
-            const T* const srw = srwv[u];
-            const int t = tt[u];
-            T az = acc[u][k][0];
-#pragma unroll
-            for (int h = 1; h < NACC; ++h) az += acc[u][k][h];
-            const T zc = win[u][(jj + P) % RW][P];
-            T res;
-            if constexpr (CHEB) {
-              const T rv = srw[o * 32 + lane];
-              const T zp = prev ? srw[(BU * BV + o) * 32 + lane] : (T)0;
-              res = zc + c1 * (zc - zp) + wo * (rv - az);
-              if constexpr (MODE == UNI_CHEBDOT) {
-                dot[u].add(rv * res);
-                if (qd) dot2[u].add(res * srw[(2 * BU * BV + o) * 32 + lane]);
-              }
-            } else if constexpr (MODE == UNI_CHEB1) {
-              const T dc = sdc[(jj + P) * CU + w + P];  // Dinv of the output row
-              const T z1 = c20 * dc * zc;               // zc is r here
-              out1[((size_t)t * G.N + i) * 32 + lane] = z1;
-              res = z1 + c1 * z1 + c2 * dc * (zc - az);
-            } else if constexpr (MODE == UNI_RESID) {
-              res = srw[o * 32 + lane] - az;
-            } else {
-              res = az;
-              dot[u].add(zc * az);
-            }
-            out[((size_t)t * G.N + i) * 32 + lane] = res;
-          }
-        }
+        out[((size_t)t * G.N + i) * 32 + lane] = res;
       }
     }
     if constexpr (MODE == UNI_APPLY || MODE == UNI_CHEBDOT) {
-      const bool one[1] = {true};
-#pragma unroll
-      for (int u = 0; u < TPW; ++u) {
-        if (!ok[u]) continue;  // uniform over the block
-        if (u > 0) __syncthreads();
-        double a1[1] = {dot[u].get()};
-        block_reduce<1>(a1, part, tt[u], tiles, one);
-        if (MODE == UNI_CHEBDOT && qd) {
-          __syncthreads();
-          a1[0] = dot2[u].get();
-          block_reduce<1>(a1, part2, tt[u], tiles, one);
-        }
+      block_reduce(dot.get(), part, t);
+      if (MODE == UNI_CHEBDOT && qd) {
+        __syncthreads();
+        block_reduce(dot2.get(), part2, t);
       }
     }
-    __syncthreads();  // the stage buffers (and the reduction buffer) may be refilled
-    if (!more) break;
-    todo &= todo - 1;
-    cur = nxt;
-    if constexpr (PREFETCH) bsel ^= 1;
+    __syncthreads();  // the stage buffer (and the reduction buffer) may be refilled
   }
-}
-
-template <typename T, int P, int TPB, int NIN>
-constexpr size_t smem_bytes() {
-  return SmemLayout<T, P, TPB, NIN>::total;
 }
 
 StenGeo geo_of(const wm_level& L) {
@@ -899,32 +590,18 @@ StenGeo geo_of(const wm_level& L) {
   return G;
 }
 
-template <typename T>
-const typename V2<T>::type* csm_of(const wm_level& L);
-template <>
-const float2* csm_of<float>(const wm_level& L) { return L.d_csm32.p; }
-template <>
-const double2* csm_of<double>(const wm_level& L) { return L.d_csm64.p; }
-
-// tiles per block: two float tiles for p <= 2 (register window 2 x 25), one otherwise
-template <typename T, int P>
-struct Tpb {
-  static constexpr int value = (sizeof(T) == 4 && P <= 2) ? 2 : 1;
-};
-
-template <typename T, int P, typename Epi>
-int launch(const wm_level& L, int np, int tiles, const T* src, const int* tile_active, Epi epi, int cat,
+template <int P, typename Epi>
+int launch(const wm_level& L, int np, int tiles, const double* src, const int* tile_active, const Epi& epi, int cat,
            cudaStream_t s, const int* skip_uni = nullptr) {
-  constexpr int TPB = Tpb<T, P>::value;
-  constexpr size_t sm = smem_bytes<T, P, TPB, Epi::NIN>();
+  constexpr size_t sm = SmemLayout<P, Epi::NIN>::total;
   static bool configured = false;
   if (!configured) {
-    WM_CUDA(cudaFuncSetAttribute(k_sten<T, P, TPB, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    WM_CUDA(cudaFuncSetAttribute(k_sten<P, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     configured = true;
   }
-  dim3 grid(np * L.nbu * L.nbv, (tiles + TPB - 1) / TPB);
-  WM_LAUNCH(cat, s, k_sten<T, P, TPB, Epi><<<grid, dim3(32, BU), sm, s>>>(geo_of(L), csm_of<T>(L), src, tiles,
-                                                                           tile_active, epi, skip_uni));
+  dim3 grid(np * L.nbu * L.nbv, tiles);
+  WM_LAUNCH(cat, s, k_sten<P, Epi><<<grid, dim3(32, BU), sm, s>>>(geo_of(L), L.d_csm64.p, src, tiles, tile_active,
+                                                                  epi, skip_uni));
   WM_CUDA(cudaGetLastError());
   return WM_OK;
 }
@@ -1201,12 +878,9 @@ __global__ void __launch_bounds__(BU * 32, 2)
       }
     }
   }
-  const bool one[1] = {true};
-  double a2[1] = {(double)acc};
-  block_reduce<1>(a2, part, t, tiles, one);
+  block_reduce((double)acc, part, t);
   __syncthreads();
-  a2[0] = tiny && mine ? HUGE_VAL : (double)accb;  // fails the caller's error check
-  block_reduce<1>(a2, part_bound, t, tiles, one);
+  block_reduce(tiny && mine ? HUGE_VAL : (double)accb, part_bound, t);  // +inf fails the caller's error check
 }
 
 // The same residual for groups of one-shift tiles (the list of the one-shift
@@ -1350,28 +1024,23 @@ __global__ void __launch_bounds__(BU * 32, 3)
         if (i1 >= 0) emit(i1, spp.y, cpp.y, b1);
       }
     }
-    const bool one[1] = {true};
-    double a2[1] = {(double)acc};
-    block_reduce<1>(a2, part, t, tiles, one);
+    block_reduce((double)acc, part, t);
     __syncthreads();
-    a2[0] = tiny && mine ? HUGE_VAL : (double)accb;  // fails the caller's error check
-    block_reduce<1>(a2, part_bound, t, tiles, one);
+    block_reduce(tiny && mine ? HUGE_VAL : (double)accb, part_bound, t);  // +inf fails the caller's error check
     __syncthreads();  // the window and the reduction buffer may be refilled
   }
 }
 
-__global__ void k_build_csm(int N, int W, int cs32, int cs64, const int16_t* __restrict__ slot,
-                            const double* __restrict__ S, const double* __restrict__ M, float2* __restrict__ c32,
-                            double2* __restrict__ c64, float4* __restrict__ cdf) {
+__global__ void k_build_csm(int N, int W, int S2, const int16_t* __restrict__ slot, const double* __restrict__ S,
+                            const double* __restrict__ M, double2* __restrict__ c64, float4* __restrict__ cdf) {
   int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (t >= (int64_t)N * W) return;
   int sl = slot[t];
   if (sl < 0) return;
   int i = (int)(t / W);
-  c32[(size_t)i * cs32 + sl] = make_float2((float)S[t], (float)M[t]);
-  c64[(size_t)i * cs64 + sl] = make_double2(S[t], M[t]);
+  c64[(size_t)i * S2 + sl] = make_double2(S[t], M[t]);
   float sh = (float)S[t], mh = (float)M[t];
-  cdf[(size_t)i * cs64 + sl] = make_float4(sh, (float)(S[t] - (double)sh), mh, (float)(M[t] - (double)mh));
+  cdf[(size_t)i * S2 + sl] = make_float4(sh, (float)(S[t] - (double)sh), mh, (float)(M[t] - (double)mh));
 }
 
 }  // namespace
@@ -1391,7 +1060,6 @@ int wm_sten_build(const wm_geom_desc& g, int np, wm_level& L, cudaStream_t s) {
   std::vector<int16_t> slot;
   if (wm_host_stencil(g, np, L, ext, own, slot) != WM_OK) return WM_OK;  // row kernels only
   const int p = g.degree, S2 = (2 * p + 1) * (2 * p + 1);
-  const int cs32 = (S2 + 1) / 2 * 2, cs64 = S2;  // coefficient row strides (16-byte multiples)
   L.ELU = L.nlu + 2 * p;
   L.ELV = L.nlv + 2 * p;
   L.nbu = (L.nlu + BU - 1) / BU;
@@ -1401,19 +1069,17 @@ int wm_sten_build(const wm_geom_desc& g, int np, wm_level& L, cudaStream_t s) {
   WM_TRY(L.d_own.upload(own, s));
   DevBuf<int16_t> d_slot;
   WM_TRY(d_slot.upload(slot, s));
-  WM_TRY(L.d_csm32.alloc((size_t)L.N * cs32));
-  WM_TRY(L.d_csm64.alloc((size_t)L.N * cs64));
-  WM_TRY(L.d_csmdf.alloc((size_t)L.N * cs64));
-  WM_CUDA(cudaMemsetAsync(L.d_csm32.p, 0, sizeof(float2) * (size_t)L.N * cs32, s));
-  WM_CUDA(cudaMemsetAsync(L.d_csm64.p, 0, sizeof(double2) * (size_t)L.N * cs64, s));
-  WM_CUDA(cudaMemsetAsync(L.d_csmdf.p, 0, sizeof(float4) * (size_t)L.N * cs64, s));
+  WM_TRY(L.d_csm64.alloc((size_t)L.N * S2));
+  WM_TRY(L.d_csmdf.alloc((size_t)L.N * S2));
+  WM_CUDA(cudaMemsetAsync(L.d_csm64.p, 0, sizeof(double2) * (size_t)L.N * S2, s));
+  WM_CUDA(cudaMemsetAsync(L.d_csmdf.p, 0, sizeof(float4) * (size_t)L.N * S2, s));
   int64_t n = (int64_t)L.N * L.W;
   WM_LAUNCH(WM_PC_ASSEMBLY, s, k_build_csm<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(
-                                   L.N, L.W, cs32, cs64, d_slot.p, L.d_S64.p, L.d_M64.p, L.d_csm32.p, L.d_csm64.p,
-                                   L.d_csmdf.p));
+                                   L.N, L.W, S2, d_slot.p, L.d_S64.p, L.d_M64.p, L.d_csm64.p, L.d_csmdf.p));
   WM_CUDA(cudaGetLastError());
   WM_CUDA(cudaStreamSynchronize(s));
   d_slot.release();
+  WM_TRY(wm_stream_build(np, p, L, ext, s));
   L.sten = true;
   return WM_OK;
 }
@@ -1443,136 +1109,106 @@ static int device_sms() {
   return n > 0 ? n : 152;
 }
 
-template <typename T, int P, int MODE>
+template <int P, int MODE>
 static int launch_uni(const wm_level& L, int np, int tiles, const UniTiles& ut, int kstep, const double* sigma,
-                      const typename V2<T>::type* ctab, const int* sid, const T* r, const T* z, const T* prev,
-                      T* out, const int* tile_active, double* part, int cat, cudaStream_t s,
-                      const T* qd = nullptr, double* part2 = nullptr, T* out1 = nullptr) {
-  constexpr size_t sm = UniLayout<T, P, MODE>::total;
+                      const double2* ctab, const int* sid, const double* r, const double* z, const double* prev,
+                      double* out, const int* tile_active, double* part, int cat, cudaStream_t s,
+                      const double* qd = nullptr, double* part2 = nullptr, double* out1 = nullptr) {
+  constexpr size_t sm = UniLayout<P, MODE>::total;
   static bool configured = false;
   if (!configured) {
-    WM_CUDA(cudaFuncSetAttribute(k_sten_uni<T, P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    WM_CUDA(cudaFuncSetAttribute(k_sten_uni<P, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     configured = true;
   }
   if (ut.n_groups <= 0) return WM_OK;
   static const int sms = device_sms();
   const int bx = np * L.nbu * L.nbv;
   // blocks that share a group: enough blocks for ut.waves waves
-  const int64_t want = (int64_t)ut.waves * sms * UniMinBlocks<T, P, MODE>::value;
+  const int64_t want = (int64_t)ut.waves * sms * UniMinBlocks<P, MODE>::value;
   int split = 1;
   while (split < kUniGroup && (int64_t)bx * ut.n_groups * split < want) split *= 2;
-  const T* dS = std::is_same<T, double>::value ? (const T*)L.d_dS64.p : (const T*)L.d_dS32.p;
-  const T* dM = std::is_same<T, double>::value ? (const T*)L.d_dM64.p : (const T*)L.d_dM32.p;
   const int gmax = 65535 / split;  // grid.y limit
   for (int g0 = 0; g0 < ut.n_groups; g0 += gmax) {
     const int ng = std::min(gmax, ut.n_groups - g0);
     dim3 grid(bx, ng * split);
-    WM_LAUNCH(cat, s, k_sten_uni<T, P, MODE><<<grid, dim3(32, BU), sm, s>>>(
-                          geo_of(L), csm_of<T>(L), dS, dM, sigma, ctab, sid, kstep, z, r, prev, out, tiles,
-                          tile_active, ut.groups + g0, split, part, qd, part2, out1));
+    WM_LAUNCH(cat, s, k_sten_uni<P, MODE><<<grid, dim3(32, BU), sm, s>>>(
+                          geo_of(L), L.d_csm64.p, L.d_dS64.p, L.d_dM64.p, sigma, ctab, sid, kstep, z, r, prev, out,
+                          tiles, tile_active, ut.groups + g0, split, part, qd, part2, out1));
     WM_CUDA(cudaGetLastError());
   }
   return WM_OK;
 }
 
-template <typename T>
 int wm_sten_cheb_step(const wm_level& L, int np, int p, int tiles, int kstep, const double* sigma,
-                      const typename StenC2<T>::type* ctab, const int* sid, const T* r, const T* z, const T* prev,
-                      T* out, const int* tile_active, const UniTiles& ut, int cat, cudaStream_t s,
-                      const T* q, double* part_rz, double* part_zq, bool generic_only) {
+                      const double2* ctab, const int* sid, const double* r, const double* z, const double* prev,
+                      double* out, const int* tile_active, const UniTiles& ut, int cat, cudaStream_t s,
+                      const double* q, double* part_rz, double* part_zq, bool generic_only) {
   if (generic_only) {
     // the one-shift tiles were done elsewhere: generic kernel for the others only
   } else if (ut.n > 0 && part_rz) {
-    WM_DISPATCH_P(p, { WM_TRY((launch_uni<T, PP, UNI_CHEBDOT>(L, np, tiles, ut, kstep, sigma, ctab, sid, r, z, prev,
-                                                              out, tile_active, part_rz, cat, s, q, part_zq))); });
+    WM_DISPATCH_P(p, { WM_TRY((launch_uni<PP, UNI_CHEBDOT>(L, np, tiles, ut, kstep, sigma, ctab, sid, r, z, prev,
+                                                           out, tile_active, part_rz, cat, s, q, part_zq))); });
   } else if (ut.n > 0) {
-    WM_DISPATCH_P(p, { WM_TRY((launch_uni<T, PP, UNI_CHEB>(L, np, tiles, ut, kstep, sigma, ctab, sid, r, z, prev,
-                                                           out, tile_active, nullptr, cat, s))); });
+    WM_DISPATCH_P(p, { WM_TRY((launch_uni<PP, UNI_CHEB>(L, np, tiles, ut, kstep, sigma, ctab, sid, r, z, prev, out,
+                                                        tile_active, nullptr, cat, s))); });
   }
   if (ut.n >= tiles) return WM_OK;
-  ChebEpi<T, 2> e2;
-  ChebEpi<T, 1> e1;
-  auto fill = [&](auto& e) {
-    e.N = L.N;
-    e.kstep = kstep;
-    e.dS = std::is_same<T, double>::value ? (const T*)L.d_dS64.p : (const T*)L.d_dS32.p;
-    e.dM = std::is_same<T, double>::value ? (const T*)L.d_dM64.p : (const T*)L.d_dM32.p;
-    e.out = out;
-    e.sigma = sigma;
-    e.ctab = ctab;
-    e.sid = sid;
-    e.in[0] = r;
-    e.in[1] = prev;
-  };
-  fill(e2);
-  fill(e1);
+  ChebEpi e;
+  e.N = L.N;
+  e.kstep = kstep;
+  e.dS = L.d_dS64.p;
+  e.dM = L.d_dM64.p;
+  e.out = out;
+  e.sigma = sigma;
+  e.ctab = ctab;
+  e.sid = sid;
+  e.in[0] = r;
+  e.in[1] = prev;
   const int* skip = ut.n > 0 ? ut.flag : nullptr;
-  WM_DISPATCH_P(p, {
-    if constexpr (Tpb<T, PP>::value == 2)
-      return launch<T, PP>(L, np, tiles, z, tile_active, e2, cat, s, skip);
-    else
-      return launch<T, PP>(L, np, tiles, z, tile_active, e1, cat, s, skip);
-  });
+  WM_DISPATCH_P(p, return launch<PP>(L, np, tiles, z, tile_active, e, cat, s, skip));
   return WM_OK;
 }
 
-template <typename T>
-int wm_sten_cheb_first2(const wm_level& L, int np, int p, int tiles, const double* sigma,
-                        const typename StenC2<T>::type* ctab, const int* sid, const T* r, T* z1, T* z2,
-                        const int* tile_active, const UniTiles& ut, int cat, cudaStream_t s) {
-  WM_DISPATCH_P(p, { WM_TRY((launch_uni<T, PP, UNI_CHEB1>(L, np, tiles, ut, 1, sigma, ctab, sid, nullptr, r, nullptr,
-                                                          z2, tile_active, nullptr, cat, s, nullptr, nullptr,
-                                                          z1))); });
+int wm_sten_cheb_first2(const wm_level& L, int np, int p, int tiles, const double* sigma, const double2* ctab,
+                        const int* sid, const double* r, double* z1, double* z2, const int* tile_active,
+                        const UniTiles& ut, int cat, cudaStream_t s) {
+  WM_DISPATCH_P(p, { WM_TRY((launch_uni<PP, UNI_CHEB1>(L, np, tiles, ut, 1, sigma, ctab, sid, nullptr, r, nullptr, z2,
+                                                       tile_active, nullptr, cat, s, nullptr, nullptr, z1))); });
   return WM_OK;
 }
 
-template <typename T>
-int wm_sten_residual(const wm_level& L, int np, int p, int tiles, const double* sigma, const T* r, const T* z,
-                     T* res, const int* tile_active, const UniTiles& ut, int cat, cudaStream_t s) {
+int wm_sten_residual(const wm_level& L, int np, int p, int tiles, const double* sigma, const double* r,
+                     const double* z, double* res, const int* tile_active, const UniTiles& ut, int cat,
+                     cudaStream_t s) {
   if (ut.n > 0) {
-    WM_DISPATCH_P(p, { WM_TRY((launch_uni<T, PP, UNI_RESID>(L, np, tiles, ut, 0, sigma, nullptr, nullptr, r, z,
-                                                            nullptr, res, tile_active, nullptr, cat, s))); });
+    WM_DISPATCH_P(p, { WM_TRY((launch_uni<PP, UNI_RESID>(L, np, tiles, ut, 0, sigma, nullptr, nullptr, r, z, nullptr,
+                                                         res, tile_active, nullptr, cat, s))); });
     if (ut.n >= tiles) return WM_OK;
   }
-  ResidEpi<T, 2> e2;
-  ResidEpi<T, 1> e1;
-  e2.N = e1.N = L.N;
-  e2.r = e1.r = r;
-  e2.res = e1.res = res;
-  e2.sigma = e1.sigma = sigma;
-  e2.in[0] = e1.in[0] = r;
+  ResidEpi e;
+  e.N = L.N;
+  e.res = res;
+  e.sigma = sigma;
+  e.in[0] = r;
   const int* skip = ut.n > 0 ? ut.flag : nullptr;
-  WM_DISPATCH_P(p, {
-    if constexpr (Tpb<T, PP>::value == 2)
-      return launch<T, PP>(L, np, tiles, z, tile_active, e2, cat, s, skip);
-    else
-      return launch<T, PP>(L, np, tiles, z, tile_active, e1, cat, s, skip);
-  });
+  WM_DISPATCH_P(p, return launch<PP>(L, np, tiles, z, tile_active, e, cat, s, skip));
   return WM_OK;
 }
 
-template <typename T>
-int wm_sten_apply_pq(const wm_level& L, int np, int p, int tiles, const double* sigma, const T* pv, T* q,
+int wm_sten_apply_pq(const wm_level& L, int np, int p, int tiles, const double* sigma, const double* pv, double* q,
                      const int* tile_active, const UniTiles& ut, double* part, cudaStream_t s) {
   if (ut.n > 0) {
-    WM_DISPATCH_P(p, { WM_TRY((launch_uni<T, PP, UNI_APPLY>(L, np, tiles, ut, 0, sigma, nullptr, nullptr, nullptr,
-                                                            pv, nullptr, q, tile_active, part, WM_PC_APPLY64,
-                                                            s))); });
+    WM_DISPATCH_P(p, { WM_TRY((launch_uni<PP, UNI_APPLY>(L, np, tiles, ut, 0, sigma, nullptr, nullptr, nullptr, pv,
+                                                         nullptr, q, tile_active, part, WM_PC_APPLY64, s))); });
     if (ut.n >= tiles) return WM_OK;
   }
-  ApplyEpi<T, 2> e2;
-  ApplyEpi<T, 1> e1;
-  e2.N = e1.N = L.N;
-  e2.q = e1.q = q;
-  e2.sigma = e1.sigma = sigma;
-  e2.part = e1.part = part;
+  ApplyEpi e;
+  e.N = L.N;
+  e.q = q;
+  e.sigma = sigma;
+  e.part = part;
   const int* skip = ut.n > 0 ? ut.flag : nullptr;
-  WM_DISPATCH_P(p, {
-    if constexpr (Tpb<T, PP>::value == 2)
-      return launch<T, PP>(L, np, tiles, pv, tile_active, e2, WM_PC_APPLY64, s, skip);
-    else
-      return launch<T, PP>(L, np, tiles, pv, tile_active, e1, WM_PC_APPLY64, s, skip);
-  });
+  WM_DISPATCH_P(p, return launch<PP>(L, np, tiles, pv, tile_active, e, WM_PC_APPLY64, s, skip));
   return WM_OK;
 }
 
@@ -1580,7 +1216,7 @@ template <typename Tr>
 int wm_sten_true_residual(const wm_level& L, int np, int p, int tiles, const double* sigma, const double* x,
                           const double* rhs, const int* src_of, const int* rep, const int* tile_rep, Tr* r,
                           double* part, cudaStream_t s) {
-  TrueResEpi<Tr, 1> e;
+  TrueResEpi<Tr> e;
   e.N = L.N;
   e.rhs = rhs;
   e.src_of = src_of;
@@ -1588,7 +1224,7 @@ int wm_sten_true_residual(const wm_level& L, int np, int p, int tiles, const dou
   e.r = r;
   e.sigma = sigma;
   e.part = part;
-  WM_DISPATCH_P(p, { return launch<double, PP>(L, np, tiles, x, tile_rep, e, WM_PC_TRUERES, s); });
+  WM_DISPATCH_P(p, return launch<PP>(L, np, tiles, x, tile_rep, e, WM_PC_TRUERES, s));
   return WM_OK;
 }
 
@@ -1638,25 +1274,6 @@ int wm_sten_true_residual_df(const wm_level& L, int np, int p, int tiles, const 
   return WM_OK;
 }
 
-template int wm_sten_cheb_step<float>(const wm_level&, int, int, int, int, const double*, const float2*,
-                                      const int*, const float*, const float*, const float*, float*, const int*,
-                                      const UniTiles&, int, cudaStream_t, const float*, double*, double*, bool);
-template int wm_sten_cheb_step<double>(const wm_level&, int, int, int, int, const double*, const double2*,
-                                       const int*, const double*, const double*, const double*, double*, const int*,
-                                       const UniTiles&, int, cudaStream_t, const double*, double*, double*, bool);
-template int wm_sten_cheb_first2<float>(const wm_level&, int, int, int, const double*, const float2*, const int*,
-                                        const float*, float*, float*, const int*, const UniTiles&, int, cudaStream_t);
-template int wm_sten_cheb_first2<double>(const wm_level&, int, int, int, const double*, const double2*, const int*,
-                                         const double*, double*, double*, const int*, const UniTiles&, int,
-                                         cudaStream_t);
-template int wm_sten_residual<float>(const wm_level&, int, int, int, const double*, const float*, const float*, float*,
-                                     const int*, const UniTiles&, int, cudaStream_t);
-template int wm_sten_residual<double>(const wm_level&, int, int, int, const double*, const double*, const double*,
-                                      double*, const int*, const UniTiles&, int, cudaStream_t);
-template int wm_sten_apply_pq<float>(const wm_level&, int, int, int, const double*, const float*, float*, const int*,
-                                     const UniTiles&, double*, cudaStream_t);
-template int wm_sten_apply_pq<double>(const wm_level&, int, int, int, const double*, const double*, double*,
-                                      const int*, const UniTiles&, double*, cudaStream_t);
 template int wm_sten_true_residual<float>(const wm_level&, int, int, int, const double*, const double*, const double*,
                                           const int*, const int*, const int*, float*, double*, cudaStream_t);
 template int wm_sten_true_residual<double>(const wm_level&, int, int, int, const double*, const double*,

@@ -28,26 +28,16 @@ int wm_sten_build(const wm_geom_desc& g, int np, wm_level& L, cudaStream_t s);
 // number of spatial blocks of a stencil launch on the level (partial-sum chunks)
 int wm_sten_chunks(const wm_level& L, int np);
 
-template <typename T>
-struct StenC2;
-template <>
-struct StenC2<float> {
-  using type = float2;
-};
-template <>
-struct StenC2<double> {
-  using type = double2;
-};
-// Three-term Chebyshev step out = z + c1 (z - prev) + c2 D^{-1} (r - A z)
+// Float64 steps.  Three-term Chebyshev step
+// out = z + c1 (z - prev) + c2 D^{-1} (r - A z)
 // (c1 = 0 at kstep 0, prev = nullptr for z_prev = 0; out may alias prev).
 // ctab: (c1, c2) per [shift][step] of the level (WM_MAX_CHEB steps per shift).
 // The one-shift tiles of `ut` go to the combined-coefficient kernel, the
 // others to the generic one.
-template <typename T>
 int wm_sten_cheb_step(const wm_level& L, int np, int p, int tiles, int kstep, const double* sigma,
-                      const typename StenC2<T>::type* ctab, const int* sid, const T* r, const T* z, const T* prev,
-                      T* out, const int* tile_active, const UniTiles& ut, int cat, cudaStream_t s,
-                      const T* q = nullptr, double* part_rz = nullptr, double* part_zq = nullptr,
+                      const double2* ctab, const int* sid, const double* r, const double* z, const double* prev,
+                      double* out, const int* tile_active, const UniTiles& ut, int cat, cudaStream_t s,
+                      const double* q = nullptr, double* part_rz = nullptr, double* part_zq = nullptr,
                       bool generic_only = false);
 // With part_rz set, the one-shift tiles of the step also leave per-block partial
 // sums (r, out) in part_rz and, with q set, (out, q) in part_zq ([tile][chunk][32],
@@ -57,18 +47,16 @@ int wm_sten_cheb_step(const wm_level& L, int np, int p, int tiles, int kstep, co
 // z1 = c2_0 D^{-1} r and z2 = z1 + c1_1 z1 + c2_1 D^{-1} (r - A z1) in one pass
 // over the window of r (the other tiles take the row-form first step and
 // wm_sten_cheb_step with generic_only).
-template <typename T>
-int wm_sten_cheb_first2(const wm_level& L, int np, int p, int tiles, const double* sigma,
-                        const typename StenC2<T>::type* ctab, const int* sid, const T* r, T* z1, T* z2,
-                        const int* tile_active, const UniTiles& ut, int cat, cudaStream_t s);
+int wm_sten_cheb_first2(const wm_level& L, int np, int p, int tiles, const double* sigma, const double2* ctab,
+                        const int* sid, const double* r, double* z1, double* z2, const int* tile_active,
+                        const UniTiles& ut, int cat, cudaStream_t s);
 // residual res = r - A z and outer apply q = A p with per-block partial sums
 // (p, q) in `part` ([tile][chunk][32], chunk = spatial block); the one-shift
 // tiles of `ut` take the combined-coefficient kernel
-template <typename T>
-int wm_sten_residual(const wm_level& L, int np, int p, int tiles, const double* sigma, const T* r, const T* z,
-                     T* res, const int* tile_active, const UniTiles& ut, int cat, cudaStream_t s);
-template <typename T>
-int wm_sten_apply_pq(const wm_level& L, int np, int p, int tiles, const double* sigma, const T* pv, T* q,
+int wm_sten_residual(const wm_level& L, int np, int p, int tiles, const double* sigma, const double* r,
+                     const double* z, double* res, const int* tile_active, const UniTiles& ut, int cat,
+                     cudaStream_t s);
+int wm_sten_apply_pq(const wm_level& L, int np, int p, int tiles, const double* sigma, const double* pv, double* q,
                      const int* tile_active, const UniTiles& ut, double* part, cudaStream_t s);
 template <typename Tr>
 int wm_sten_true_residual(const wm_level& L, int np, int p, int tiles, const double* sigma, const double* x,
@@ -82,3 +70,46 @@ int wm_sten_true_residual(const wm_level& L, int np, int p, int tiles, const dou
 int wm_sten_true_residual_df(const wm_level& L, int np, int p, int tiles, const UniTiles& ut, const double* sigma,
                              const double* x, const double* rhs, const int* src_of, const int* rep,
                              const int* tile_rep, float* r, double* part, double* part_bound, cudaStream_t s);
+
+// ---- streaming kernels of the float solves (wm_stream.h): every tile, any shifts
+constexpr int kStreamTiles = 4;  // tiles of a block
+// The batch's tiles in groups of up to kStreamTiles consecutive ones, (first
+// tile, count): n[1] groups of one shift, then n[0] of any shifts.
+struct StreamTiles {
+  const int2* groups = nullptr;
+  int n[2] = {0, 0};
+  int tiles = 0;
+};
+// the grouping: `uni` flags the tiles of one shift, `shift` is its index
+void wm_stream_groups(const std::vector<int>& uni, const std::vector<int>& shift, std::vector<int2>& groups,
+                      int n[2]);
+// ST_CHEB     three-term Chebyshev step out = z + c1 (z - prev) + c2 D^{-1} (r - A z)
+//             (c1 = 0 at kstep 0; prev = nullptr there; out may alias prev)
+// ST_CHEBDOT  the same, with the partial sums (r, out) in part and (out, q) in part2
+// ST_CHEB1    the first two steps from z = 0 in one pass over z (which is r here):
+//             out1 = z1 = c2_0 D^{-1} r, out = z1 + c1_1 z1 + c2_1 D^{-1} (r - A z1)
+// ST_RESID    out = r - A z
+// ST_APPLY    out = A z, with the partial sums (z, out) in part
+// Partial sums: [tile][item][32], wm_stream_items() items.
+enum { ST_CHEB = 0, ST_RESID = 1, ST_APPLY = 2, ST_CHEBDOT = 3, ST_CHEB1 = 4 };
+struct StreamArgs {
+  const wm_level* L = nullptr;
+  int np = 0;
+  StreamTiles st;
+  int kstep = 0;
+  const double* sigma = nullptr;
+  const float2* ctab = nullptr;  // the level's (c1, c2) per [shift][step]
+  const int* sid = nullptr;
+  const int* tile_active = nullptr;
+  const float *z = nullptr, *r = nullptr, *prev = nullptr, *q = nullptr;
+  float *out = nullptr, *out1 = nullptr;
+  double *part = nullptr, *part2 = nullptr;
+  int cat = 0;
+  cudaStream_t s = nullptr;
+};
+int wm_stream(int p, int mode, const StreamArgs& a);
+int wm_stream_build(int np, int p, wm_level& L, const std::vector<int32_t>& ext, cudaStream_t s);
+// partial sums per tile and system of the kernels that form dot products, and
+// the most that a solve of up to `tiles` tiles leaves over all its tiles
+int wm_stream_items(const wm_level& L, int np, int p, const StreamTiles& st);
+size_t wm_stream_part_max(const wm_level& L, int np, int tiles);
