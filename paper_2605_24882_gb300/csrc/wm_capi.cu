@@ -559,6 +559,13 @@ extern "C" int wm_apply_mass(wm_hier_t h, int level, const double* x, double* y,
   if (n_vec == 0) return WM_OK;
   cudaStream_t s = as_stream(stream);
   const wm_level& L = h->lv[level];
+  const size_t len = (size_t)n_vec * L.N;
+  if (x + len <= y || y + len <= x) {
+    WM_TRY(wm_k_mass_rows(L, n_vec, x, y, s));
+    WM_CUDA(cudaStreamSynchronize(s));
+    return WM_OK;
+  }
+  // overlapping x and y (in place): through tiled copies
   int tiles = (n_vec + WM_LANES - 1) / WM_LANES;
   size_t n = (size_t)tiles * L.N * WM_LANES;
   Tmp t;

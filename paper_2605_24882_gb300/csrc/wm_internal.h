@@ -225,6 +225,8 @@ int wm_k_apply(const wm_level& L, int tiles, const double* sigma, const T* x, T*
                const int* tile_active, cudaStream_t s);
 int wm_k_apply_mass64(const wm_level& L, int tiles, const double* x, double* y,
                       const int* tile_active, cudaStream_t s);
+// y = M x on n vectors in the caller's layout [n][N] (x and y apart)
+int wm_k_mass_rows(const wm_level& L, int n, const double* x, double* y, cudaStream_t s);
 template <typename T>
 int wm_k_prolong_add(const wm_level& fine, int tiles, const T* xc, T* xf, const int* tile_active,
                      cudaStream_t s);
