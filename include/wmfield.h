@@ -358,7 +358,7 @@ int wm_noise_loads_noalloc(wm_hier_t h, uint64_t seed, int n_samples, double* b,
  * iteration) until every shifted residual satisfies |r_k| <= rtol |y_s|, at
  * most max_iter iterations.  f: device [n_samples][N] float64, caller-owned.
  * iterations: host, may be NULL; receives the CG iterations of the slowest
- * pass.  Device scratch is allocated per call (2 n_nodes + 7 float64 vectors
+ * pass.  Device scratch is allocated per call (n_nodes + 6 float64 vectors
  * per sample, samples processed in passes that fit half the free memory) and
  * the call returns after the stream has finished.
  * Errors: WM_ERR_INVALID_ARG (sizes, bounds, host f), WM_ERR_OOM, WM_ERR_CUDA,

@@ -211,6 +211,8 @@ int wm_k_pack_rows(wm_level& L, cudaStream_t s);
 int wm_k_philox(const uint32_t* ctr, uint64_t key, uint32_t* out, int64_t n, cudaStream_t s);
 int wm_k_normals(uint64_t seed, int sample, int stream_id, int64_t q0, int64_t n, double* out,
                  cudaStream_t s);
+// normals 0..N-1 of samples s0 .. s0 + ns - 1 into a tiled buffer [tiles][N][32], zero beyond
+int wm_k_normals_tiled(uint64_t seed, int s0, int ns, int stream_id, int N, double* out, int tiles, cudaStream_t s);
 // loads of rows [row0, row0+ns) of a tiled [tiles][N][32] buffer (row v at tile
 // v/32, lane v%32), row row0 + k holding the loads of sample sample_first + k
 // (its Philox counters); `bl` is scratch of E*nk*ns doubles

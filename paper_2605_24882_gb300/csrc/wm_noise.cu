@@ -78,6 +78,20 @@ __global__ void k_normals(uint64_t seed, int sample, int stream, int64_t q0, int
   out[i] = (q & 1) ? z1 : z0;
 }
 
+// normals 0..N-1 of samples s0 + (tile, lane) into [tiles][N][32], zero from sample
+// s0 + ns on; lane = sample, a thread does the two normals of a pair
+__global__ void k_normals_tiled(uint64_t seed, int s0, int ns, int stream, int N, double* __restrict__ out) {
+  const int t = blockIdx.y, s = t * WM_LANES + threadIdx.x;
+  const int64_t pair = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
+  const int64_t i = 2 * pair;
+  if (i >= N) return;
+  double z0 = 0.0, z1 = 0.0;
+  if (s < ns) normal_pair(seed, s0 + s, stream, pair, &z0, &z1);
+  double* const o = out + ((size_t)t * N + i) * WM_LANES + threadIdx.x;
+  o[0] = z0;
+  if (i + 1 < N) o[WM_LANES] = z1;
+}
+
 // sqrt(w_q a_q) of every Gauss point, [E][nq^2] (the factor k_noise_local
 // forms per sample, with the same operations)
 template <int P>
@@ -176,6 +190,16 @@ int wm_k_philox(const uint32_t* ctr, uint64_t key, uint32_t* out, int64_t n, cud
 int wm_k_normals(uint64_t seed, int sample, int stream_id, int64_t q0, int64_t n, double* out, cudaStream_t s) {
   if (n <= 0) return WM_OK;
   WM_LAUNCH(WM_PC_NOISE, s, k_normals<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(seed, sample, stream_id, q0, n, out));
+  WM_CUDA(cudaGetLastError());
+  return WM_OK;
+}
+
+int wm_k_normals_tiled(uint64_t seed, int s0, int ns, int stream_id, int N, double* out, int tiles,
+                       cudaStream_t s) {
+  if (tiles <= 0 || N <= 0) return WM_OK;
+  const unsigned pairs = (unsigned)((N + 1) / 2);
+  WM_LAUNCH(WM_PC_NOISE, s, k_normals_tiled<<<dim3((pairs + 7) / 8, tiles), dim3(WM_LANES, 8), 0, s>>>(
+                                seed, s0, ns, stream_id, N, out));
   WM_CUDA(cudaGetLastError());
   return WM_OK;
 }

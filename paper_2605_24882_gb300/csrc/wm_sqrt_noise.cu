@@ -12,13 +12,14 @@
 //   a^k_n = a_n zeta^k_{n+1} / zeta^k_n,  b^k_n = b_n (zeta^k_{n+1} / zeta^k_n)^2,
 //   x^k += a^k_n p^k,  p^k = zeta^k_{n+1} r_{n+1} + b^k_n p^k,
 // with a_n, b_n the seed's CG coefficients (a_{-1} = 1, b_{-1} = 0,
-// zeta_{-1} = zeta_0 = 1).  Shift k of a sample stops once
+// zeta_{-1} = zeta_0 = 1).  Only the sum of c_k x^k is wanted, so no x^k is kept: the
+// directions are kept over zeta, d^k = p^k / zeta^k, and
+//   s += sum_k c_k a_n zeta^k_{n+1} d^k,   d^k = r_{n+1} + b_n (zeta^k_{n+1} / zeta^k_n) d^k.  Shift k of a sample stops once
 // |zeta^k| |r| <= rtol |y|.  The shifts are positive, so every shifted system
 // converges no slower than the seed.
 //
-// Layout: samples 32 to a tile, [tiles][N][32] (lane = sample); the shift
-// vectors are node-major blocks [K][tiles][N][32], so the weighted sum over
-// k is an elementwise pass.  Row kernels: one warp per (tile, row), rows in
+// Layout: samples 32 to a tile, [tiles][N][32] (lane = sample); the shifts'
+// directions are node-major blocks [K][tiles][N][32].  Row kernels: one warp per (tile, row), rows in
 // chunks of kRows per block; per-lane partial dot products are reduced over
 // the block's warps and then over the chunks in a fixed order.
 #include <cmath>
@@ -49,16 +50,26 @@ __device__ __forceinline__ void block_partial(double acc, double* __restrict__ p
   }
 }
 
-__device__ __forceinline__ double chunk_sum(const double* __restrict__ part, int nchunk, int nsys, int g) {
+// sum of the chunk partials of sample (tile blockIdx.x, lane) by the block's warps,
+// the same value in all of them (a serial sum per sample, 199 chunks for the
+// 64 x 64 sphere, took 30-40 us a launch)
+__device__ __forceinline__ double tile_sum(const double* __restrict__ part, int nchunk, int tiles) {
+  __shared__ double sh[kWarps][WM_LANES];
   double s = 0.0;
-  for (int c = 0; c < nchunk; ++c) s += part[(size_t)c * nsys + g];
+  for (int c = threadIdx.y; c < nchunk; c += kWarps)
+    s += part[((size_t)c * tiles + blockIdx.x) * WM_LANES + threadIdx.x];
+  sh[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  s = 0.0;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) s += sh[w][threadIdx.x];
   return s;
 }
 
-// r = p = y, p^k = y, x^k = 0 for every shift; partial (r, r)
+// r = p = y, d^k = y for every shift, s = 0; partial (r, r)
 __global__ void __launch_bounds__(256) k_ms_init(int N, int K, const double* __restrict__ ybuf,
                                                  double* __restrict__ r, double* __restrict__ p,
-                                                 double* __restrict__ xs, double* __restrict__ ps,
+                                                 double* __restrict__ acc_s, double* __restrict__ ds,
                                                  double* __restrict__ part) {
   const int t = blockIdx.y, l = threadIdx.x;
   const size_t nblk = (size_t)gridDim.y * N * WM_LANES;
@@ -70,10 +81,8 @@ __global__ void __launch_bounds__(256) k_ms_init(int N, int K, const double* __r
     const double yv = ybuf[o];
     r[o] = yv;
     p[o] = yv;
-    for (int k = 0; k < K; ++k) {
-      xs[(size_t)k * nblk + o] = 0.0;
-      ps[(size_t)k * nblk + o] = yv;
-    }
+    acc_s[o] = 0.0;
+    for (int k = 0; k < K; ++k) ds[(size_t)k * nblk + o] = yv;
     acc += yv * yv;
   }
   block_partial(acc, part, ((size_t)blockIdx.x * gridDim.y + t) * WM_LANES);
@@ -123,14 +132,20 @@ struct SampleState {
 };
 
 // (r, r) of y; a sample with y = 0 is done at once.  Every shift starts at zeta = 1.
-__global__ void k_ms_start(int nsamp, int nchunk, int K, const double* __restrict__ part,
-                           SampleState* __restrict__ st, double* __restrict__ zeta, double* __restrict__ zeta_old,
-                           int* __restrict__ shift_active, int* __restrict__ flags) {
-  int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= nsamp) return;
-  const double v = chunk_sum(part, nchunk, nsamp, g);
-  if (!isfinite(v)) atomicOr(flags, 1);
+__global__ void __launch_bounds__(256) k_ms_start(int nsamp, int nchunk, int K, const double* __restrict__ part,
+                                                  SampleState* __restrict__ st, double* __restrict__ zeta,
+                                                  double* __restrict__ zeta_old, int* __restrict__ shift_active,
+                                                  int* __restrict__ flags) {
+  const int g = blockIdx.x * WM_LANES + threadIdx.x;
+  const double v = tile_sum(part, nchunk, gridDim.x);
   const int act = (v > 0.0 && isfinite(v)) ? 1 : 0;
+  for (int k = threadIdx.y; k < K; k += kWarps) {
+    zeta[(size_t)k * nsamp + g] = 1.0;
+    zeta_old[(size_t)k * nsamp + g] = 1.0;
+    shift_active[(size_t)k * nsamp + g] = act;
+  }
+  if (threadIdx.y != 0) return;
+  if (!isfinite(v)) atomicOr(flags, 1);
   SampleState s;
   s.rr = v;
   s.rr0 = v;
@@ -140,19 +155,15 @@ __global__ void k_ms_start(int nsamp, int nchunk, int K, const double* __restric
   s.b_old = 0.0;
   s.active = act;
   st[g] = s;
-  for (int k = 0; k < K; ++k) {
-    zeta[(size_t)k * nsamp + g] = 1.0;
-    zeta_old[(size_t)k * nsamp + g] = 1.0;
-    shift_active[(size_t)k * nsamp + g] = act;
-  }
 }
 
 // seed step length a_n = (r, r) / (p, M p)
-__global__ void k_ms_alpha(int nsamp, int nchunk, const double* __restrict__ part, SampleState* __restrict__ st,
-                           double* __restrict__ a_out, int* __restrict__ flags) {
-  int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= nsamp) return;
-  const double pq = chunk_sum(part, nchunk, nsamp, g);
+__global__ void __launch_bounds__(256) k_ms_alpha(int nchunk, const double* __restrict__ part,
+                                                  SampleState* __restrict__ st, double* __restrict__ a_out,
+                                                  int* __restrict__ flags) {
+  const int g = blockIdx.x * WM_LANES + threadIdx.x;
+  const double pq = tile_sum(part, nchunk, gridDim.x);
+  if (threadIdx.y != 0) return;
   double a = 0.0;
   if (st[g].active) {
     if (pq > 0.0 && isfinite(pq)) {
@@ -165,31 +176,36 @@ __global__ void k_ms_alpha(int nsamp, int nchunk, const double* __restrict__ par
   a_out[g] = a;
 }
 
-// b_n, and for every shift zeta_{n+1}, a^k_n, b^k_n and its convergence test
-__global__ void k_ms_shifts(int nsamp, int nchunk, int K, const double* __restrict__ part,
-                            const double* __restrict__ w2, double rtol, SampleState* __restrict__ st,
-                            double* __restrict__ zeta, double* __restrict__ zeta_old,
-                            int* __restrict__ shift_active, double* __restrict__ ak, double* __restrict__ bk,
-                            double* __restrict__ zk, double* __restrict__ b_out, int* __restrict__ n_active,
-                            int* __restrict__ flags) {
-  int g = blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= nsamp) return;
+// b_n, and for every shift zeta_{n+1}, the factors g^k = c_k a_n zeta_{n+1} of s and
+// h^k = b_n zeta_{n+1} / zeta_n of d^k, and its convergence test; tile_shift[k][tile] tells
+// whether a sample of the tile has the shift to update.  Warp y takes shifts y, y + 8, ..
+__global__ void __launch_bounds__(256) k_ms_shifts(int nsamp, int nchunk, int K, const double* __restrict__ part,
+                                                   const double* __restrict__ w2, const double* __restrict__ cnode,
+                                                   double rtol, SampleState* __restrict__ st,
+                                                   double* __restrict__ zeta, double* __restrict__ zeta_old,
+                                                   int* __restrict__ shift_active, int* __restrict__ tile_shift,
+                                                   double* __restrict__ gk, double* __restrict__ hk,
+                                                   double* __restrict__ b_out, int* __restrict__ n_active,
+                                                   int* __restrict__ flags) {
+  __shared__ int any[WM_LANES];
+  const int g = blockIdx.x * WM_LANES + threadIdx.x;
+  if (threadIdx.y == 0) any[threadIdx.x] = 0;
   SampleState s = st[g];
-  const double rr_new = chunk_sum(part, nchunk, nsamp, g);
+  const double rr_new = tile_sum(part, nchunk, gridDim.x);  // (its barrier: `any` is set, every warp read st)
   double b = 0.0;
-  int any = 0;
   if (s.active) {
     if (!isfinite(rr_new)) {
-      atomicOr(flags, 1);
+      if (threadIdx.y == 0) atomicOr(flags, 1);
     } else if (s.rr > 0.0) {
       b = rr_new / s.rr;
     }
   }
   const double rnorm = sqrt(rr_new > 0.0 ? rr_new : 0.0), goal = rtol * sqrt(s.rr0);
-  for (int k = 0; k < K; ++k) {
+  for (int k = threadIdx.y; k < K; k += kWarps) {
     const size_t j = (size_t)k * nsamp + g;
-    double a_k = 0.0, b_k = 0.0, z_k = 0.0;
-    if (s.active && shift_active[j]) {
+    const bool on = s.active && shift_active[j];
+    double g_k = 0.0, h_k = 0.0;
+    if (on) {
       const double zc = zeta[j], zo = zeta_old[j];
       const double den = s.a * s.b_old * (zo - zc) + zo * s.a_old * (1.0 + w2[k] * s.a);
       const double zn = zc * zo * s.a_old / den;
@@ -197,62 +213,80 @@ __global__ void k_ms_shifts(int nsamp, int nchunk, int K, const double* __restri
         atomicOr(flags, 1);
         shift_active[j] = 0;
       } else {
-        const double ratio = zn / zc;
-        a_k = s.a * ratio;
-        b_k = b * ratio * ratio;
-        z_k = zn;
+        g_k = cnode[k] * s.a * zn;
+        h_k = b * (zn / zc);
         zeta_old[j] = zc;
         zeta[j] = zn;
         if (fabs(zn) * rnorm <= goal) {
           shift_active[j] = 0;
         } else {
-          any = 1;
+          atomicOr(&any[threadIdx.x], 1);
         }
       }
     }
-    ak[j] = a_k;
-    bk[j] = b_k;
-    zk[j] = z_k;
+    gk[j] = g_k;
+    hk[j] = h_k;
+    const bool tile_on = __any_sync(0xffffffffu, on);
+    if (threadIdx.x == 0) tile_shift[(size_t)k * gridDim.x + blockIdx.x] = tile_on;
   }
+  __syncthreads();
+  if (threadIdx.y != 0) return;
   s.a_old = s.a;
   s.b_old = b;
   s.b = b;
   s.rr = rr_new;
-  s.active = s.active && any;
+  s.active = s.active && any[threadIdx.x];
   st[g] = s;
   b_out[g] = s.active ? b : 0.0;
   if (s.active) atomicAdd(n_active, 1);
 }
 
-// x^k += a^k p^k, p^k = zeta^k r + b^k p^k for every shift; seed p = r + b p
-__global__ void k_ms_update(size_t nblk, int N, int K, int nsamp, const double* __restrict__ ak,
-                            const double* __restrict__ bk, const double* __restrict__ zk,
-                            const double* __restrict__ b, const double* __restrict__ r, double* __restrict__ p,
-                            double* __restrict__ xs, double* __restrict__ ps) {
-  size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (o >= nblk) return;
-  const int g = (int)((o / ((size_t)N * WM_LANES)) * WM_LANES + (o % WM_LANES));
-  const double rv = r[o];
-  for (int k = 0; k < K; ++k) {
-    const size_t j = (size_t)k * nsamp + g, e = (size_t)k * nblk + o;
-    const double pk = ps[e];
-    xs[e] += ak[j] * pk;
-    ps[e] = zk[j] * rv + bk[j] * pk;
+// s += sum_k g^k d^k, d^k = r + h^k d^k for every shift that a sample of the tile still
+// needs (large shifts converge in a few steps); seed p = r + b p.  A thread takes
+// kUpdRows rows of one sample, so that the shift's factors are read once for them.
+// Bytes per (DOF, sample): 40 + 16 K', K' the live shifts; 2 K' float64 FMAs.  The
+// form with every x^k and every shift moved 24 + 32 K and did 3 K: 184 steps at
+// K = 20 and 64 samples of the 64 x 64 sphere took 35 ms of the call's 65.
+constexpr int kUpdRows = 4;
+__global__ void __launch_bounds__(256) k_ms_update(int N, int K, int nsamp, const int* __restrict__ tile_shift,
+                                                   const double* __restrict__ gk, const double* __restrict__ hk,
+                                                   const double* __restrict__ b, const double* __restrict__ r,
+                                                   double* __restrict__ p, double* __restrict__ acc_s,
+                                                   double* __restrict__ ds) {
+  const int t = blockIdx.y, tiles = gridDim.y;
+  const int g = t * WM_LANES + threadIdx.x;
+  const size_t nblk = (size_t)tiles * N * WM_LANES;
+  const int i0 = (blockIdx.x * kWarps + threadIdx.y) * kUpdRows;
+  const int rows = min(kUpdRows, N - i0);
+  if (rows <= 0) return;
+  const size_t o = ((size_t)t * N + i0) * WM_LANES + threadIdx.x;
+  double rv[kUpdRows], s[kUpdRows];
+#pragma unroll
+  for (int u = 0; u < kUpdRows; ++u) {
+    rv[u] = u < rows ? r[o + u * WM_LANES] : 0.0;
+    s[u] = u < rows ? acc_s[o + u * WM_LANES] : 0.0;
   }
-  p[o] = rv + b[g] * p[o];
+  for (int k = 0; k < K; ++k) {
+    if (!tile_shift[(size_t)k * tiles + t]) continue;
+    const double gv = gk[(size_t)k * nsamp + g], hv = hk[(size_t)k * nsamp + g];
+    double* const d = ds + (size_t)k * nblk + o;
+    double dv[kUpdRows];
+#pragma unroll
+    for (int u = 0; u < kUpdRows; ++u) dv[u] = u < rows ? d[u * WM_LANES] : 0.0;
+#pragma unroll
+    for (int u = 0; u < kUpdRows; ++u) {
+      s[u] += gv * dv[u];
+      if (u < rows) d[u * WM_LANES] = rv[u] + hv * dv[u];
+    }
+  }
+  const double bv = b[g];
+#pragma unroll
+  for (int u = 0; u < kUpdRows; ++u)
+    if (u < rows) {
+      acc_s[o + u * WM_LANES] = s[u];
+      p[o + u * WM_LANES] = rv[u] + bv * p[o + u * WM_LANES];
+    }
 }
-
-// acc = sum_k c_k x_k over the node blocks (same tile layout as the samples)
-__global__ void k_ms_combine(size_t nblk, int K, const double* __restrict__ cnode, const double* __restrict__ x,
-                             double* __restrict__ acc) {
-  size_t o = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-  if (o >= nblk) return;
-  double s = 0.0;
-  for (int k = 0; k < K; ++k) s += cnode[k] * x[(size_t)k * nblk + o];
-  acc[o] = s;
-}
-
-inline unsigned blocks_for(size_t n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
 bool on_device(const void* ptr) {
   cudaPointerAttributes a;
@@ -284,35 +318,32 @@ extern "C" int wm_noise_loads_sqrt(wm_hier_t h, uint64_t seed, int n_samples, do
   const wm_level& L = h->lv[0];
   const int N = L.N;
   const int ts = (n_samples + WM_LANES - 1) / WM_LANES;
-  // sample tiles per pass: 2K shift vectors and seven seed/layout vectors per
-  // sample tile within half the free memory
+  // sample tiles per pass: K directions and six seed/layout vectors per sample tile
+  // within half the free memory
   size_t free_b = 0, total_b = 0;
   WM_CUDA(cudaMemGetInfo(&free_b, &total_b));
-  const size_t per_tile = (size_t)(2 * K + 7) * N * WM_LANES * sizeof(double);
+  const size_t per_tile = (size_t)(K + 6) * N * WM_LANES * sizeof(double);
   int tc = (int)std::min<size_t>((size_t)ts, std::max<size_t>(1, (free_b / 2) / per_tile));
   tc = std::min(tc, 65535);
   const int nsamp = tc * WM_LANES;
   const int nchunk = (N + kRows - 1) / kRows;
   const size_t nblk = (size_t)tc * N * WM_LANES;
-  Buf<double> r, p, q, xs, ps, ybuf, yrows, acc, ftile, part, a, b, ak, bk, zk, zeta, zeta_old, d_w2, d_c;
+  Buf<double> r, p, q, ds, ybuf, acc, part, a, b, gk, hk, zeta, zeta_old, d_w2, d_c;
   Buf<SampleState> st;
-  Buf<int> shift_active, counters;
+  Buf<int> shift_active, tile_shift, counters;
   WM_TRY(r.alloc(nblk));
   WM_TRY(p.alloc(nblk));
   WM_TRY(q.alloc(nblk));
-  WM_TRY(xs.alloc(nblk * K));
-  WM_TRY(ps.alloc(nblk * K));
-  WM_TRY(ybuf.alloc(nblk));
-  WM_TRY(yrows.alloc(nblk));
+  WM_TRY(ds.alloc(nblk * K));
+  WM_TRY(ybuf.alloc(nblk));  // y, then f in tiles
   WM_TRY(acc.alloc(nblk));
-  WM_TRY(ftile.alloc(nblk));
   WM_TRY(part.alloc((size_t)nchunk * nsamp));
   WM_TRY(a.alloc(nsamp));
   WM_TRY(b.alloc(nsamp));
   WM_TRY(st.alloc(nsamp));
-  WM_TRY(ak.alloc((size_t)K * nsamp));
-  WM_TRY(bk.alloc((size_t)K * nsamp));
-  WM_TRY(zk.alloc((size_t)K * nsamp));
+  WM_TRY(gk.alloc((size_t)K * nsamp));
+  WM_TRY(hk.alloc((size_t)K * nsamp));
+  WM_TRY(tile_shift.alloc((size_t)K * tc));
   WM_TRY(zeta.alloc((size_t)K * nsamp));
   WM_TRY(zeta_old.alloc((size_t)K * nsamp));
   WM_TRY(shift_active.alloc((size_t)K * nsamp));
@@ -320,32 +351,29 @@ extern "C" int wm_noise_loads_sqrt(wm_hier_t h, uint64_t seed, int n_samples, do
   WM_TRY(d_w2.upload(w2, s));
   WM_TRY(d_c.upload(c, s));
   const dim3 rgrid((unsigned)nchunk, (unsigned)tc), rblock(WM_LANES, kWarps);
-  const unsigned sgrid = blocks_for((size_t)nsamp, 128);
-  const unsigned egrid = blocks_for(nblk, 256);
+  const dim3 ugrid((unsigned)((N + kWarps * kUpdRows - 1) / (kWarps * kUpdRows)), (unsigned)tc);
   int worst_iters = 0;
   bool not_converged = false;
   for (int t0 = 0; t0 < ts; t0 += tc) {
     const int tcur = std::min(tc, ts - t0);  // sample tiles of this pass; unused tiles get y = 0
     const int s0 = t0 * WM_LANES, ns = std::min(n_samples - s0, tcur * WM_LANES);
-    for (int si = 0; si < ns; ++si)
-      WM_TRY(wm_k_normals(seed, s0 + si, kNormalStream, 0, N, yrows.p + (size_t)si * N, s));
-    WM_TRY(wm_k_to_tiled(yrows.p, ns, N, ybuf.p, tc, s));
+    WM_TRY(wm_k_normals_tiled(seed, s0, ns, kNormalStream, N, ybuf.p, tc, s));
     WM_CUDA(cudaMemsetAsync(counters.p, 0, 2 * sizeof(int), s));
-    WM_LAUNCH(WM_PC_NOISE, s, k_ms_init<<<rgrid, rblock, 0, s>>>(N, K, ybuf.p, r.p, p.p, xs.p, ps.p, part.p));
-    WM_LAUNCH(WM_PC_NOISE, s, k_ms_start<<<sgrid, 128, 0, s>>>(nsamp, nchunk, K, part.p, st.p, zeta.p, zeta_old.p,
+    WM_LAUNCH(WM_PC_NOISE, s, k_ms_init<<<rgrid, rblock, 0, s>>>(N, K, ybuf.p, r.p, p.p, acc.p, ds.p, part.p));
+    WM_LAUNCH(WM_PC_NOISE, s, k_ms_start<<<tc, rblock, 0, s>>>(nsamp, nchunk, K, part.p, st.p, zeta.p, zeta_old.p,
                                                                shift_active.p, counters.p + 1));
     int it = 0, host_active = 1;
     while (it < max_iter && host_active > 0) {
       ++it;
       WM_LAUNCH(WM_PC_NOISE, s, k_ms_apply<<<rgrid, rblock, 0, s>>>(N, L.W, L.d_col.p, L.d_M64.p, p.p, q.p, part.p));
-      WM_LAUNCH(WM_PC_NOISE, s, k_ms_alpha<<<sgrid, 128, 0, s>>>(nsamp, nchunk, part.p, st.p, a.p, counters.p + 1));
+      WM_LAUNCH(WM_PC_NOISE, s, k_ms_alpha<<<tc, rblock, 0, s>>>(nchunk, part.p, st.p, a.p, counters.p + 1));
       WM_LAUNCH(WM_PC_NOISE, s, k_ms_resid<<<rgrid, rblock, 0, s>>>(N, a.p, q.p, r.p, part.p));
       WM_CUDA(cudaMemsetAsync(counters.p, 0, sizeof(int), s));
-      WM_LAUNCH(WM_PC_NOISE, s, k_ms_shifts<<<sgrid, 128, 0, s>>>(nsamp, nchunk, K, part.p, d_w2.p, rtol, st.p,
-                                                                  zeta.p, zeta_old.p, shift_active.p, ak.p, bk.p,
-                                                                  zk.p, b.p, counters.p, counters.p + 1));
-      WM_LAUNCH(WM_PC_NOISE, s, k_ms_update<<<egrid, 256, 0, s>>>(nblk, N, K, nsamp, ak.p, bk.p, zk.p, b.p, r.p, p.p,
-                                                                  xs.p, ps.p));
+      WM_LAUNCH(WM_PC_NOISE, s, k_ms_shifts<<<tc, rblock, 0, s>>>(nsamp, nchunk, K, part.p, d_w2.p, d_c.p, rtol, st.p,
+                                                                  zeta.p, zeta_old.p, shift_active.p, tile_shift.p,
+                                                                  gk.p, hk.p, b.p, counters.p, counters.p + 1));
+      WM_LAUNCH(WM_PC_NOISE, s, k_ms_update<<<ugrid, rblock, 0, s>>>(N, K, nsamp, tile_shift.p, gk.p, hk.p, b.p, r.p,
+                                                                     p.p, acc.p, ds.p));
       WM_CUDA(cudaGetLastError());
       if (it % 4 == 0 || it == max_iter) {
         int hc[2] = {0, 0};
@@ -360,10 +388,9 @@ extern "C" int wm_noise_loads_sqrt(wm_hier_t h, uint64_t seed, int n_samples, do
     }
     worst_iters = std::max(worst_iters, it);
     if (host_active > 0) not_converged = true;
-    WM_LAUNCH(WM_PC_NOISE, s, k_ms_combine<<<egrid, 256, 0, s>>>(nblk, K, d_c.p, xs.p, acc.p));
     WM_CUDA(cudaGetLastError());
-    WM_TRY(wm_k_apply_mass64(L, tc, acc.p, ftile.p, nullptr, s));
-    WM_TRY(wm_k_from_tiled(ftile.p, tc, N, f + (size_t)s0 * N, ns, s));
+    WM_TRY(wm_k_apply_mass64(L, tc, acc.p, ybuf.p, nullptr, s));
+    WM_TRY(wm_k_from_tiled(ybuf.p, tc, N, f + (size_t)s0 * N, ns, s));
   }
   int flag = 0;
   WM_CUDA(cudaMemcpyAsync(&flag, counters.p + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
