@@ -639,6 +639,25 @@ static int set_batch_meta(WorkSpace& ws, const wm_schedule& sc, int tiles, const
     n_uni += uni[t];
   }
   ws.n_uni_tiles = n_uni;
+  // other tiles with few distinct shift indices (the double-float residual combines
+  // the rows for each)
+  std::vector<int> few(tiles, 0);
+  ws.n_few_tiles = ws.few_max = 0;
+  for (int t = 0; t < tiles; ++t) {
+    if (uni[t]) continue;
+    int seen[kDfFew], nd = 0;
+    for (int l = 0; l < WM_LANES && nd <= kDfFew; ++l) {
+      const int v = si[(size_t)t * WM_LANES + l];
+      if (std::find(seen, seen + std::min(nd, kDfFew), v) != seen + std::min(nd, kDfFew)) continue;
+      if (nd < kDfFew) seen[nd] = v;
+      ++nd;
+    }
+    if (nd > kDfFew) continue;
+    few[t] = 1;
+    ws.n_few_tiles += 1;
+    ws.few_max = std::max(ws.few_max, nd);
+  }
+  WM_CUDA(cudaMemcpyAsync(ws.tile_few.p, few.data(), tiles * sizeof(int), cudaMemcpyHostToDevice, s));
   // groups of at most kUniGroup consecutive one-shift tiles with the same shift
   // index (one block of the one-shift kernel per group and spatial block)
   std::vector<int2> grp;

@@ -1320,6 +1320,9 @@ static UniTiles uni_of(const WorkSpace& ws) {
   UniTiles u;
   u.flag = ws.tile_uni.p;
   u.n = ws.n_uni_tiles;
+  u.few = ws.tile_few.p;
+  u.n_few = ws.n_few_tiles;
+  u.few_max = ws.few_max;
   u.groups = ws.uni_groups.p;
   u.n_groups = ws.n_uni_groups;
   u.waves = ws.uni_waves;
@@ -1387,6 +1390,7 @@ int WorkSpace::reserve(const wm_hier* h, int tiles, int nshift, bool dbl) {
   WM_TRY(tile_active.alloc(tiles));
   WM_TRY(tile_rep.alloc(tiles));
   WM_TRY(tile_uni.alloc(tiles));
+  WM_TRY(tile_few.alloc(tiles));
   WM_TRY(rho.alloc(ns));
   WM_TRY(alpha.alloc(ns));
   WM_TRY(beta.alloc(ns));
@@ -1421,7 +1425,8 @@ void WorkSpace::release() {
   }
   lvl.clear();
   sigma.release(); sid.release(); src_of.release(); active.release(); rep.release(); restart.release();
-  tile_active.release(); tile_rep.release(); tile_uni.release(); uni_groups.release();
+  tile_active.release(); tile_rep.release(); tile_uni.release(); tile_few.release();
+  uni_groups.release();
   st_groups.release();
   rho.release(); alpha.release(); beta.release(); bb.release(); rr.release(); rr_ref.release();
   for (auto& pp : part) pp.release();
@@ -1970,7 +1975,7 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
         bool done = false;
         if constexpr (std::is_same<T, float>::value) {
           if (df_res) {
-            WM_TRY(wm_sten_true_residual_df(L0, h->np, h->p, tiles, uni_of(ws), ws.sigma.p, ws.x.p, rhs_tiled,
+            WM_TRY(wm_sten_true_residual_df(L0, h->np, h->p, tiles, uni_of(ws), ws.sid.p, ws.sigma.p, ws.x.p, rhs_tiled,
                                             ws.src_of.p, ws.rep.p, ws.tile_rep.p, r, ws.part[1].p, ws.part[2].p, s));
             WM_CUDA(cudaMemsetAsync(cnt + 5, 0, sizeof(int), s));
             WM_LAUNCH(WM_PC_SCALAR, s, k_df_check<<<tiles, kSumBlk, 0, s>>>(ch_op, ws.part[2].p, ws.bb.p,

@@ -76,6 +76,8 @@ struct WorkSpace {
   DevBuf<int> src_of;         // per system right-hand-side sample (-1: padding)
   DevBuf<int> active, rep, restart, tile_active, tile_rep;
   DevBuf<int> tile_uni;       // 1 where the 32 shifts of a tile are equal
+  DevBuf<int> tile_few;       // 1 where another tile has at most kDfFew shift indices
+  int n_few_tiles = 0, few_max = 0;
   int n_uni_tiles = 0;        // host count of such tiles in the current batch
   DevBuf<int2> uni_groups;    // runs of at most 8 consecutive such tiles of one shift: (first tile, count)
   int n_uni_groups = 0;

@@ -13,11 +13,14 @@
 // consecutive such tiles with the same shift index, each (first tile, count).
 // A block of the one-shift kernel serves one group (or part of one).
 constexpr int kUniGroup = 8;
+constexpr int kDfFew = 4;
 struct UniTiles {
   const int* flag = nullptr;     // [tiles] 1 where the 32 shifts of the tile are equal
   int n = 0;                     // number of such tiles
   const int2* groups = nullptr;  // [n_groups] (first tile, count), count in 1..kUniGroup
   int n_groups = 0;
+  const int* few = nullptr;      // [tiles] 1 where a tile not of one shift has at most kDfFew shifts
+  int n_few = 0, few_max = 0;    // number of such tiles, most shifts of one
   int waves = 4;                 // grid target: runs are split until the grid has this many waves
 };
 
@@ -66,8 +69,10 @@ int wm_sten_true_residual(const wm_level& L, int np, int p, int tiles, const dou
 // arithmetic on the FP32 pipes; part_bound receives the per-block partial
 // sums of ||B||^2 with B_i = sum_j |a_ij| |x_j| (the rounding error of entry i
 // is below 2^-42 B_i), or +inf for a system with a value below 2^-102
-// (one-shift tiles of `ut` by groups, the others one tile per block)
-int wm_sten_true_residual_df(const wm_level& L, int np, int p, int tiles, const UniTiles& ut, const double* sigma,
+// (one-shift tiles of `ut` by groups, the others one tile per block: with the rows
+// combined for each shift where there are at most kDfFew)
+int wm_sten_true_residual_df(const wm_level& L, int np, int p, int tiles, const UniTiles& ut, const int* sid,
+                             const double* sigma,
                              const double* x, const double* rhs, const int* src_of, const int* rep,
                              const int* tile_rep, float* r, double* part, double* part_bound, cudaStream_t s);
 

@@ -69,3 +69,19 @@ def test_inactive_tiles_of_a_group_keep_their_results(wm, ns):
     assert st["n_not_converged"] == 0
     err = (d * hier.apply_mass(d)).sum(1) / (ref * hier.apply_mass(ref)).sum(1)
     assert float(err.max()) ** 0.5 < 1e-8
+
+
+@pytest.mark.parametrize("p", [2, 3])
+@pytest.mark.parametrize("ns", [5, 8, 11, 20, 31])
+def test_true_residuals_of_tiles_with_a_few_shifts(wm, p, ns):
+    """Ragged sample counts put up to four (ns >= 11) or more shifts into a tile: the
+    double-float residuals of either kind accept the same solutions as the float64 path
+    (both solved to 1e-9, far above the residuals' 2^-42 error)."""
+    hier = wm.Hierarchy(wm.Geometry("sphere", p, 16), 4)
+    kw = dict(kappa=2.0, beta=0.7, sinc_k=0.5, l_lo=-12, l_hi=12, n_samples=ns, seed=4, rtol=1e-9)
+    u, st = hier.sample_fields(precision="mixed", **kw)
+    ref, _ = hier.sample_fields(precision="fp64", **kw)
+    assert st["n_not_converged"] == 0 and st["n_df_fallbacks"] == 0 and st["max_rel_residual"] <= 1e-9
+    d = u - ref
+    err = (d * hier.apply_mass(d)).sum(1) / (ref * hier.apply_mass(ref)).sum(1)
+    assert float(err.max()) ** 0.5 < 1e-7
