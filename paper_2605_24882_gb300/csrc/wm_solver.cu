@@ -723,7 +723,7 @@ __global__ void __launch_bounds__(256) k_cheb_step(int N, int W, int chunks, int
     c2[k] = cf.y;
   }
   RowRange rr = chunk_rows(N, chunks);
-  for (int i = rr.i0 + threadIdx.y; i < rr.i1; i += kWarps) {
+  for (int i = rr.i0 + threadIdx.y; i < rr.i1; i += blockDim.y) {
     T aS[kTPW], aM[kTPW];
 #pragma unroll
     for (int k = 0; k < kTPW; ++k) aS[k] = aM[k] = 0;
@@ -766,7 +766,7 @@ __global__ void __launch_bounds__(256) k_residual(int N, int W, int chunks, int 
 #pragma unroll
   for (int k = 0; k < kTPW; ++k) sg[k] = ts.act[k] ? (T)sigma[(t0 + k) * WM_LANES + lane] : (T)0;
   RowRange rr = chunk_rows(N, chunks);
-  for (int i = rr.i0 + threadIdx.y; i < rr.i1; i += kWarps) {
+  for (int i = rr.i0 + threadIdx.y; i < rr.i1; i += blockDim.y) {
     T aS[kTPW], aM[kTPW];
 #pragma unroll
     for (int k = 0; k < kTPW; ++k) aS[k] = aM[k] = 0;
@@ -1686,6 +1686,13 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
   const int tiles = bt.tiles;
   const int ch = bt.vcycle_chunks(Lv.N);
   const dim3 ggrid(ch, groups(tiles));
+  // Operator rows in float64: a row of a tile occupies the SM's float64 unit for 50 x 17
+  // cycles (p = 2), so where blocks of 16 rows would not give every SM one, blocks of
+  // two warps take two rows: 152 rows of two tiles 32 -> 17 us a step (event-timed).
+  const bool thin = std::is_same<T, double>::value && (int64_t)((Lv.N + 15) / 16) * groups(tiles) < 152;
+  const dim3 oblk = thin ? dim3(WM_LANES, 2) : kBlk;
+  const int och = thin ? (Lv.N + 1) / 2 : ch;
+  const dim3 ogrid(och, groups(tiles));
   const typename C2T<T>::type* ctab = cheb_tab<T>(ws) + (size_t)l * bt.nshift * WM_MAX_CHEB;
   const auto* pk = rows_of<T>(Lv);
   const T* dS = dS_of<T>(Lv);
@@ -1747,7 +1754,7 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
       }
       if (e != WM_OK) step_rc = e;
     } else {
-      WM_LAUNCH(csm, s, k_cheb_step<T><<<ggrid, kBlk, 0, s>>>(Lv.N, Lv.W, ch, tiles, k, pk, dS, dM, ws.sigma.p,
+      WM_LAUNCH(csm, s, k_cheb_step<T><<<ogrid, oblk, 0, s>>>(Lv.N, Lv.W, och, tiles, k, pk, dS, dM, ws.sigma.p,
                                                               ctab, ws.sid.p, rin, zin, prev, zo, ta));
     }
     units(csm, bt, (has_prev ? 4.0 : 3.0) * Tb * Lv.N, 2.0 * Lv.nnz + 8.0 * Lv.N);
@@ -1800,7 +1807,7 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
       WM_TRY(wm_sten_residual(Lv, h->np, h->p, tiles, ws.sigma.p, rin, cur, res, ta, uni_of(ws), cre, s));
     }
   } else {
-    WM_LAUNCH(cre, s, k_residual<T><<<ggrid, kBlk, 0, s>>>(Lv.N, Lv.W, ch, tiles, pk, ws.sigma.p, rin, cur, res,
+    WM_LAUNCH(cre, s, k_residual<T><<<ogrid, oblk, 0, s>>>(Lv.N, Lv.W, och, tiles, pk, ws.sigma.p, rin, cur, res,
                                                            ta));
   }
   units(cre, bt, 3.0 * Tb * Lv.N, 4.0 * Lv.nnz + 3.0 * Lv.N);

@@ -72,6 +72,7 @@ __device__ __forceinline__ void block_reduce(double acc, double* part, int t) {
 // z_next = z + c1 (z - z_prev) + c2 D^{-1} (r - A z), with c1 = 0 at step 0
 // and z_prev = 0 where there is none; out may alias z_prev
 struct ChebEpi {
+  static constexpr bool PARTIALS = false;
   static constexpr int NIN = 2;  // r and z_prev of the output rows are staged
   const double* in[2];           // in[1] = nullptr: z_prev = 0
   int N, kstep;
@@ -99,6 +100,7 @@ struct ChebEpi {
 
 // residual: res = r - A z
 struct ResidEpi {
+  static constexpr bool PARTIALS = false;
   static constexpr int NIN = 1;  // r staged
   const double* in[1];
   int N;
@@ -114,6 +116,7 @@ struct ResidEpi {
 
 // outer apply: q = A p, partial (p, q)
 struct ApplyEpi {
+  static constexpr bool PARTIALS = true;
   static constexpr int NIN = 0;
   const double* in[1];
   int N;
@@ -134,6 +137,7 @@ struct ApplyEpi {
 // float64 true residual of flagged systems: r = b - A x, partial ||r||^2
 template <typename Tr>
 struct TrueResEpi {
+  static constexpr bool PARTIALS = true;
   static constexpr int NIN = 0;
   const double* in[1];
   int N;
@@ -173,9 +177,9 @@ __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
 }
 
-template <int P, int NIN>
+template <int P, int BVT, int NIN>
 struct SmemLayout {
-  static constexpr int BV = BvOf<P>::value;
+  static constexpr int BV = BVT;
   static constexpr int CU = BU + 2 * P, CV = BV + 2 * P, NC = CU * CV, S2 = (2 * P + 1) * (2 * P + 1);
   static constexpr size_t win = (size_t)NC * 32 * sizeof(double);
   static constexpr size_t coef = (size_t)BU * BV * S2 * sizeof(double2);
@@ -184,12 +188,16 @@ struct SmemLayout {
   static constexpr size_t total = win + coef + rows + ids;
 };
 
-template <int P, typename Epi>
+// BVT: outputs of a warp.  The float64 unit of an SM does one warp FMA in 17 cycles, so a
+// block of 8 x 6 outputs (2,400 of them) takes 20 us however many SMs are idle: launches
+// of fewer blocks than SMs take blocks two rows high.  One sample on the 8 x 8 sphere
+// (51 systems, 48 blocks): a Chebyshev step 34 -> 16 us (event-timed).
+template <int P, int BVT, typename Epi>
 __global__ void __launch_bounds__(BU * 32, 1) k_sten(StenGeo G, const double2* __restrict__ csm,
                                                      const double* __restrict__ src, int tiles,
                                                      const int* __restrict__ tile_active, const Epi epi_arg,
                                                      const int* __restrict__ skip_uni) {
-  using LY = SmemLayout<P, Epi::NIN>;
+  using LY = SmemLayout<P, BVT, Epi::NIN>;
   constexpr int BV = LY::BV, NIN = Epi::NIN, SW = 2 * P + 1, CU = LY::CU, NC = LY::NC, S2 = LY::S2;
   constexpr int ROWCH = 32 * sizeof(double) / 16;  // 16-byte chunks per staged row
   Epi epi = epi_arg;  // per-thread copy (its per-tile fields live in registers)
@@ -590,20 +598,31 @@ StenGeo geo_of(const wm_level& L) {
   return G;
 }
 
+template <int P, int BVT, typename Epi>
+int launch_bv(const wm_level& L, int np, int tiles, const double* src, const int* tile_active, const Epi& epi, int cat,
+              cudaStream_t s, const int* skip_uni) {
+  constexpr size_t sm = SmemLayout<P, BVT, Epi::NIN>::total;
+  static bool configured = false;
+  if (!configured) {
+    WM_CUDA(cudaFuncSetAttribute(k_sten<P, BVT, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    configured = true;
+  }
+  StenGeo G = geo_of(L);
+  G.nbv = (L.nlv + BVT - 1) / BVT;
+  dim3 grid(np * G.nbu * G.nbv, tiles);
+  WM_LAUNCH(cat, s, k_sten<P, BVT, Epi><<<grid, dim3(32, BU), sm, s>>>(G, L.d_csm64.p, src, tiles, tile_active, epi,
+                                                                       skip_uni));
+  WM_CUDA(cudaGetLastError());
+  return WM_OK;
+}
+// (steps that leave per-block partial sums keep the standard height: the caller
+// counts its blocks)
 template <int P, typename Epi>
 int launch(const wm_level& L, int np, int tiles, const double* src, const int* tile_active, const Epi& epi, int cat,
            cudaStream_t s, const int* skip_uni = nullptr) {
-  constexpr size_t sm = SmemLayout<P, Epi::NIN>::total;
-  static bool configured = false;
-  if (!configured) {
-    WM_CUDA(cudaFuncSetAttribute(k_sten<P, Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    configured = true;
-  }
-  dim3 grid(np * L.nbu * L.nbv, tiles);
-  WM_LAUNCH(cat, s, k_sten<P, Epi><<<grid, dim3(32, BU), sm, s>>>(geo_of(L), L.d_csm64.p, src, tiles, tile_active,
-                                                                  epi, skip_uni));
-  WM_CUDA(cudaGetLastError());
-  return WM_OK;
+  if (Epi::PARTIALS || (int64_t)np * L.nbu * L.nbv * tiles >= 152)
+    return launch_bv<P, BvOf<P>::value>(L, np, tiles, src, tile_active, epi, cat, s, skip_uni);
+  return launch_bv<P, 2>(L, np, tiles, src, tile_active, epi, cat, s, skip_uni);
 }
 
 // ------------------------------------------- double-float true residual

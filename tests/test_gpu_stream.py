@@ -85,3 +85,19 @@ def test_true_residuals_of_tiles_with_a_few_shifts(wm, p, ns):
     d = u - ref
     err = (d * hier.apply_mass(d)).sum(1) / (ref * hier.apply_mass(ref)).sum(1)
     assert float(err.max()) ** 0.5 < 1e-7
+
+
+@pytest.mark.parametrize("surf", [("sphere", 2, 8, 8, 4), ("sphere", 3, 16, 16, 5), ("torus", 2, 16, 8, 1)])
+@pytest.mark.parametrize("ns", [1, 40])
+def test_float64_blocks_of_few_rows_keep_the_arithmetic(wm, surf, ns):
+    """One system per launch (few blocks: two rows per block) and the same system among
+    `ns` x 20 of other shifts (full blocks) give the same float64 V-cycle bit for bit."""
+    import torch
+    kind, p, nu, nv, levels = surf
+    hier = wm.Hierarchy(wm.Geometry(kind, p, nu, nv), levels)
+    g = torch.Generator(device="cuda").manual_seed(ns)
+    r = torch.randn((20 * ns, hier.num_dofs(0)), dtype=torch.float64, device="cuda", generator=g)
+    sg = np.geomspace(1.0, 1e4, 20 * ns)
+    z = hier.vcycle(r, sg, precision="fp64", smoother_degree=3)
+    pair = hier.vcycle(r[:2], sg[:2], precision="fp64", smoother_degree=3)
+    assert torch.equal(z[:2], pair)
