@@ -728,6 +728,7 @@ __global__ void __launch_bounds__(256) k_cheb_step(int N, int W, int chunks, int
 #pragma unroll
     for (int k = 0; k < kTPW; ++k) aS[k] = aM[k] = 0;
     const auto* e = pk + (size_t)i * W;
+#pragma unroll 5  // (the loads of several entries in flight)
     for (int w = 0; w < W; ++w) {
       auto en = ld_row(e + w);
 #pragma unroll
@@ -771,6 +772,7 @@ __global__ void __launch_bounds__(256) k_residual(int N, int W, int chunks, int 
 #pragma unroll
     for (int k = 0; k < kTPW; ++k) aS[k] = aM[k] = 0;
     const auto* e = pk + (size_t)i * W;
+#pragma unroll 5  // (the loads of several entries in flight)
     for (int w = 0; w < W; ++w) {
       auto en = ld_row(e + w);
 #pragma unroll
@@ -1178,7 +1180,10 @@ __global__ void k_power_init(int N, double* v) {
   }
 }
 
-// w = D^{-1} A v; partials (w, w), (v, v)
+// w = D^{-1} A v; with LAST the partials (w, w), (v, v).  The iterates are not scaled
+// in between: fifteen products with a matrix whose largest eigenvalue is below 25
+// (p <= 4) stay far inside the float64 range.
+template <bool LAST>
 __global__ void __launch_bounds__(256) k_power_step(int N, int W, int chunks, int tiles,
                                                     const PkRow64* __restrict__ pk, const double* __restrict__ dS,
                                                     const double* __restrict__ dM, const double* __restrict__ sigma,
@@ -1191,6 +1196,7 @@ __global__ void __launch_bounds__(256) k_power_step(int N, int W, int chunks, in
   double acc[2][1] = {{0.0}, {0.0}};
   for (int i = rr.i0 + threadIdx.y; i < rr.i1; i += kWarps) {
     double aS = 0.0, aM = 0.0;
+#pragma unroll 5
     for (int k = 0; k < W; ++k) {
       PkRow64 en = ld_row(pk + (size_t)i * W + k);
       double x = vt[(size_t)en.col * WM_LANES + threadIdx.x];
@@ -1199,21 +1205,16 @@ __global__ void __launch_bounds__(256) k_power_step(int N, int W, int chunks, in
     }
     double wv = (aS + sg * aM) / (dS[i] + sg * dM[i]);
     w[vidx(t, N, i)] = wv;
-    double vv = vt[(size_t)i * WM_LANES + threadIdx.x];
-    acc[0][0] += wv * wv;
-    acc[1][0] += vv * vv;
+    if constexpr (LAST) {
+      double vv = vt[(size_t)i * WM_LANES + threadIdx.x];
+      acc[0][0] += wv * wv;
+      acc[1][0] += vv * vv;
+    }
   }
-  double* parts[2] = {part_ww, part_vv};
-  block_reduce_store<2, 1>(acc, parts, chunks, t, tiles);
-}
-
-__global__ void k_power_scale(int N, int chunks, const double* part_ww, double* w) {
-  int t = blockIdx.y;
-  int g = t * WM_LANES + threadIdx.x;
-  double nw = sqrt(sum_parts(part_ww, chunks, g));
-  double inv = nw > 0 ? 1.0 / nw : 0.0;
-  RowRange rr = chunk_rows(N, chunks);
-  for (int i = rr.i0 + threadIdx.y; i < rr.i1; i += kWarps) w[vidx(t, N, i)] *= inv;
+  if constexpr (LAST) {
+    double* parts[2] = {part_ww, part_vv};
+    block_reduce_store<2, 1>(acc, parts, chunks, t, tiles);
+  }
 }
 
 __global__ void k_power_final(int nshift, int chunks, const double* part_ww, const double* part_vv, double* lmax) {
@@ -1468,15 +1469,24 @@ static int estimate_lmax(const wm_hier* h, WorkSpace& ws, const std::vector<doub
   bt.tiles = tiles;
   for (int l = 0; l < L - 1; ++l) {
     const wm_level& Lv = h->lv[l];
-    int ch = bt.chunks_for(Lv.N);
+    // row chunks: the last step's partials within 64, the others eight rows where that
+    // keeps the grid within a few thousand blocks (each SM's float64 unit is the bound)
+    const int ch = bt.chunks_for(Lv.N);
+    const int most = std::max(1, 8 * 152 / tiles);
+    const int chf = std::max(ch, std::min(most, (Lv.N + kWarps - 1) / kWarps));
     WM_LAUNCH(WM_PC_SETUP, s, k_power_init<<<dim3(64, tiles), kBlk, 0, s>>>(Lv.N, ws.pw_v.p));
     double* v = ws.pw_v.p;
     double* w = ws.pw_w.p;
     for (int it = 0; it < 15; ++it) {
-      WM_LAUNCH(WM_PC_SETUP, s, k_power_step<<<dim3(ch, tiles), kBlk, 0, s>>>(
-                                    Lv.N, Lv.W, ch, tiles, Lv.d_pk64.p, Lv.d_dS64.p, Lv.d_dM64.p, ws.pw_sigma.p, v, w,
-                                    ws.part[0].p, ws.part[1].p));
-      if (it < 14) WM_LAUNCH(WM_PC_SETUP, s, k_power_scale<<<dim3(ch, tiles), kBlk, 0, s>>>(Lv.N, ch, ws.part[0].p, w));
+      auto args = [&](auto* kernel, int c) {
+        WM_LAUNCH(WM_PC_SETUP, s, kernel<<<dim3(c, tiles), kBlk, 0, s>>>(
+                                      Lv.N, Lv.W, c, tiles, Lv.d_pk64.p, Lv.d_dS64.p, Lv.d_dM64.p, ws.pw_sigma.p, v,
+                                      w, ws.part[0].p, ws.part[1].p));
+      };
+      if (it < 14)
+        args(k_power_step<false>, chf);
+      else
+        args(k_power_step<true>, ch);
       std::swap(v, w);
     }
     WM_LAUNCH(WM_PC_SETUP, s, k_power_final<<<nblk(nsh, 128), 128, 0, s>>>(nsh, ch, ws.part[0].p, ws.part[1].p,
