@@ -8,6 +8,7 @@
 // Dror, Shaw, SC'11): ten rounds of two 32x32->64 multiplications by
 // 0xD2511F53 and 0xCD9E8D57 with the key bumped by (0x9E3779B9, 0xBB67AE85).
 #include "wm_internal.h"
+#include "wm_normal_tables.h"
 
 namespace {
 
@@ -34,9 +35,58 @@ __device__ __forceinline__ U4 philox10(U4 c, uint32_t k0, uint32_t k1) {
   return c;
 }
 
-__device__ __forceinline__ double uniform53(uint32_t hi, uint32_t lo) {
-  uint64_t a = (uint64_t)(hi >> 5), b = (uint64_t)(lo >> 6);
-  return (double)(a * 67108864ull + b + 1ull) * 1.1102230246251565e-16;  // 2^-53
+// the 53-bit uniform (n 2^-53) of two words, n in [1, 2^53]
+__device__ __forceinline__ uint64_t uniform53(uint32_t hi, uint32_t lo) {
+  return ((uint64_t)(hi >> 5) << 26) + (uint64_t)(lo >> 6) + 1ull;
+}
+
+// log(n 2^-53) for n in [1, 2^53]: table-driven reduction (P. T. P. Tang, "Table-driven
+// implementation of the logarithm function in IEEE floating-point arithmetic", 1990) to
+// log 2^e + log c + log1p(r) with |r| <= 2^-7 and the Taylor series of log1p, the
+// leading sums kept exact.  Sixteen float64 operations, error below an ulp.
+__device__ __forceinline__ double log_u53(uint64_t n) {
+  const int sh = __clzll((long long)n) - 11;  // -1 for 2^53
+  const uint64_t mant = (sh >= 0 ? n << sh : n >> 1) & 0xFFFFFFFFFFFFFull;
+  const int j = (int)(mant >> 45);
+  const int half = j >= 53;  // m/2 in [0.707, 1): log u near 0 has no cancellation
+  const double m = __longlong_as_double((long long)(((uint64_t)(1023 - half) << 52) | mant));
+  // e = half - 1 - sh as a double by its bits (-53 .. 0)
+  const double e = __hiloint2double(0x43300000, 1024 + half - 1 - sh) - 4503599627371520.0;  // 2^52 + 1024
+  const LogEntry t = kLogTab[j];
+  const double r = fma(m, t.ic, -1.0);
+  const double h = fma(e, kLn2Hi, t.hi);  // exact
+  const double s = h + r;
+  const double lo = ((h - s) + r) + fma(e, kLn2Lo, t.lo);
+  const double r2 = r * r;
+  double q = -1.0 / 8.0;
+  q = fma(q, r, 1.0 / 7.0);
+  q = fma(q, r, -1.0 / 6.0);
+  q = fma(q, r, 1.0 / 5.0);
+  q = fma(q, r, -1.0 / 4.0);
+  q = fma(q, r, 1.0 / 3.0);
+  q = fma(q, r, -1.0 / 2.0);
+  return s + fma(r2, q, lo);
+}
+
+// cos and sin of 2 pi n 2^-53, n in [1, 2^53]: the nearest 64th of a turn from the table
+// and the Taylor series of the rest (at most pi / 64)
+__device__ __forceinline__ void sincos_u53(uint64_t n, double* sn, double* cs) {
+  const int j = (int)((n + (1ull << 46)) >> 47);
+  // the rest d = n - j 2^47 (|d| <= 2^46) as a double by its bits
+  const long long d = (long long)(n - ((uint64_t)j << 47));
+  const double x = (__longlong_as_double(0x4330000000000000ll + (d + (1ll << 47))) - 4644337115725824.0) * kTurn53;
+  const double2 t = kTurn[j & 63];
+  const double x2 = x * x;
+  double a = fma(x2, 1.0 / 362880.0, -1.0 / 5040.0);
+  a = fma(a, x2, 1.0 / 120.0);
+  a = fma(a, x2, -1.0 / 6.0);
+  const double sx = fma(a, x2 * x, x);
+  double b = fma(x2, 1.0 / 40320.0, -1.0 / 720.0);
+  b = fma(b, x2, 1.0 / 24.0);
+  b = fma(b, x2, -1.0 / 2.0);
+  const double cm = b * x2;  // cos x - 1
+  *cs = t.x + fma(t.x, cm, -(t.y * sx));
+  *sn = t.y + fma(t.y, cm, t.x * sx);
 }
 
 // The Box–Muller pair of normals with pair index `pair` of (seed, sample, stream).
@@ -48,11 +98,9 @@ __device__ __forceinline__ void normal_pair(uint64_t seed, int sample, int strea
   c.z = (uint32_t)stream;
   c.w = (uint32_t)(pair >> 32);
   U4 o = philox10(c, (uint32_t)(seed & 0xFFFFFFFFull), (uint32_t)(seed >> 32));
-  double u1 = uniform53(o.x, o.y);
-  double u2 = uniform53(o.z, o.w);
-  double rad = sqrt(-2.0 * log(u1));
+  double rad = sqrt(-2.0 * log_u53(uniform53(o.x, o.y)));
   double s, co;
-  sincos(2.0 * M_PI * u2, &s, &co);
+  sincos_u53(uniform53(o.z, o.w), &s, &co);
   *z0 = rad * co;
   *z1 = rad * s;
 }
@@ -106,60 +154,76 @@ __global__ void k_noise_weights(int E, int nu, int nv, const double* __restrict_
   w[q] = sqrt(gw[gu] * gw[gv] * elw * metric[4 * q]);
 }
 
-// One thread per (element e, sample s0+sl): the (p+1)^2 local load
-// contributions sum_q sqrt(w_q a_q) xi_q phi_k(x_q) of the element, xi the
+// One thread per (EPT elements, sample s0+sl): the (p+1)^2 local load
+// contributions sum_q sqrt(w_q a_q) xi_q phi_k(x_q) of each element, xi the
 // Philox normals of sample s0 + sl.  bl layout [E][nk][ns].  WT: the factors
 // sqrt(w_q a_q) from the table of k_noise_weights instead of per sample.
-template <int P, bool WT = false>
+// Bound by the float64 unit (595 G operations a second): about 62 a normal pair with the
+// logarithm, sine and cosine above (90 with the general ones of 2 pi u and the
+// conversions) and 13 for the contraction.  EPT = 2 where (p+1)^2 is odd and there are
+// threads enough: two elements share their middle pair, nine pairs instead of ten.
+// 256 samples of the 64 x 64 sphere, with the gather: 4.87 -> 3.23 ms.
+template <int P, bool WT, int EPT>
 __global__ void k_noise_local(int E, int nu, int nv, int ns, int s0, uint64_t seed,
                               const double* __restrict__ metric, const double* __restrict__ gw,
                               const double* __restrict__ bu, const double* __restrict__ bv, double* __restrict__ bl,
-                              const double* __restrict__ wtab = nullptr) {
-  constexpr int NQ = P + 1, NK = (P + 1) * (P + 1), NQ2 = NQ * NQ;
+                              const double* __restrict__ wtab) {
+  constexpr int NQ = P + 1, NK = (P + 1) * (P + 1), NQ2 = NQ * NQ, NP = EPT * NQ2;
   int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (tid >= (int64_t)E * ns) return;
-  int64_t e = tid / ns;
-  int sl = (int)(tid - e * ns);
-  int eu = (int)(e % nu);
-  int ev = (int)((e / nu) % nv);
-  double xi[NQ2 + 1];
-  int64_t q0 = e * NQ2;
-  int64_t pr0 = q0 >> 1, pr1 = (q0 + NQ2 - 1) >> 1;
-  for (int64_t pr = pr0; pr <= pr1; ++pr) {
-    double z0, z1;
-    normal_pair(seed, s0 + sl, 0, pr, &z0, &z1);
-    int j0 = (int)(2 * pr - q0);
-    if (j0 >= 0) xi[j0] = z0;
-    if (j0 + 1 < NQ2) xi[j0 + 1] = z1;
-  }
-  double wq[NQ2];
-  if constexpr (WT) {
+  const int64_t e0 = tid / ns * EPT;
+  if (e0 >= E) return;
+  int sl = (int)(tid % ns);
+  double xi[NP + 1];
+  const int64_t q0 = e0 * NQ2;
+  // points of the thread, in pairs of the sample's sequence; an odd first point is the
+  // second of its pair
+  if constexpr (NP % 2 == 0) {  // q0 is even
 #pragma unroll
-    for (int j = 0; j < NQ2; ++j) wq[j] = wtab[q0 + j] * xi[j];
+    for (int h = 0; h < NP / 2; ++h) normal_pair(seed, s0 + sl, 0, (q0 >> 1) + h, &xi[2 * h], &xi[2 * h + 1]);
   } else {
-    double elw = 1.0 / ((double)nu * nv);
-#pragma unroll
-    for (int j = 0; j < NQ2; ++j) {
-      int gv = j / NQ, gu = j % NQ;
-      wq[j] = sqrt(gw[gu] * gw[gv] * elw * metric[4 * (q0 + j)]) * xi[j];
+    int64_t pr0 = q0 >> 1, pr1 = (q0 + NP - 1) >> 1;
+    for (int64_t pr = pr0; pr <= pr1; ++pr) {
+      double z0, z1;
+      normal_pair(seed, s0 + sl, 0, pr, &z0, &z1);
+      int j0 = (int)(2 * pr - q0);
+      if (j0 >= 0) xi[j0] = z0;
+      if (j0 + 1 < NP) xi[j0 + 1] = z1;
     }
   }
-  const double* BU = bu + (size_t)eu * (P + 1) * NQ;
-  const double* BV = bv + (size_t)ev * (P + 1) * NQ;
 #pragma unroll
-  for (int kv = 0; kv <= P; ++kv)
+  for (int h = 0; h < EPT; ++h) {
+    const int64_t e = e0 + h;
+    if (e >= E) break;
+    const int eu = (int)(e % nu), ev = (int)((e / nu) % nv);
+    double wq[NQ2];
+    if constexpr (WT) {
 #pragma unroll
-    for (int ku = 0; ku <= P; ++ku) {
-      double acc = 0.0;
+      for (int j = 0; j < NQ2; ++j) wq[j] = wtab[e * NQ2 + j] * xi[h * NQ2 + j];
+    } else {
+      double elw = 1.0 / ((double)nu * nv);
 #pragma unroll
-      for (int gv = 0; gv < NQ; ++gv) {
-        double t = 0.0;
-#pragma unroll
-        for (int gu = 0; gu < NQ; ++gu) t += BU[ku * NQ + gu] * wq[gv * NQ + gu];
-        acc += BV[kv * NQ + gv] * t;
+      for (int j = 0; j < NQ2; ++j) {
+        int gv = j / NQ, gu = j % NQ;
+        wq[j] = sqrt(gw[gu] * gw[gv] * elw * metric[4 * (e * NQ2 + j)]) * xi[h * NQ2 + j];
       }
-      bl[((size_t)e * NK + kv * (P + 1) + ku) * ns + sl] = acc;
     }
+    const double* BU = bu + (size_t)eu * (P + 1) * NQ;
+    const double* BV = bv + (size_t)ev * (P + 1) * NQ;
+#pragma unroll
+    for (int kv = 0; kv <= P; ++kv)
+#pragma unroll
+      for (int ku = 0; ku <= P; ++ku) {
+        double acc = 0.0;
+#pragma unroll
+        for (int gv = 0; gv < NQ; ++gv) {
+          double t = 0.0;
+#pragma unroll
+          for (int gu = 0; gu < NQ; ++gu) t += BU[ku * NQ + gu] * wq[gv * NQ + gu];
+          acc += BV[kv * NQ + gv] * t;
+        }
+        bl[((size_t)e * NK + kv * (P + 1) + ku) * ns + sl] = acc;
+      }
+  }
 }
 
 // One thread per (DOF i, row s0+sl): b[tile][i][lane] = sum over the element
@@ -207,15 +271,20 @@ int wm_k_normals_tiled(uint64_t seed, int s0, int ns, int stream_id, int N, doub
 int wm_k_noise_tiled(const wm_hier* h, uint64_t seed, int sample_first, int row0, int ns, double* b_tiled,
                      double* bl, cudaStream_t s) {
   const wm_level& L = h->lv[0];
-  int64_t n1 = (int64_t)L.E * ns;
-  unsigned g1 = (unsigned)((n1 + 127) / 128);
-#define WM_NL(PP)                                                                                              \
-  if (L.d_noise_w.p)                                                                                           \
-    k_noise_local<PP, true><<<g1, 128, 0, s>>>(L.E, L.nu, L.nv, ns, sample_first, seed, L.d_metric.p, h->d_gw.p, \
-                                               L.d_bu.p, L.d_bv.p, bl, L.d_noise_w.p);                          \
-  else                                                                                                         \
-    k_noise_local<PP><<<g1, 128, 0, s>>>(L.E, L.nu, L.nv, ns, sample_first, seed, L.d_metric.p, h->d_gw.p,      \
-                                         L.d_bu.p, L.d_bv.p, bl)
+  const int64_t n1 = (int64_t)L.E * ns;
+  // two elements per thread from 1,024 threads per SM on
+  const bool two = n1 >= 2ll * 152 * 1024;
+#define WM_NLE(PP, WT_, EPT_)                                                                                     \
+  k_noise_local<PP, WT_, EPT_><<<(unsigned)(((L.E + EPT_ - 1) / EPT_ * (int64_t)ns + 127) / 128), 128, 0, s>>>(     \
+      L.E, L.nu, L.nv, ns, sample_first, seed, L.d_metric.p, h->d_gw.p, L.d_bu.p, L.d_bv.p, bl, L.d_noise_w.p)
+#define WM_NL(PP)                                            \
+  if (L.d_noise_w.p) {                                       \
+    if (PP % 2 == 0 && two)                                  \
+      WM_NLE(PP, true, (PP % 2 == 0 ? 2 : 1));               \
+    else                                                     \
+      WM_NLE(PP, true, 1);                                   \
+  } else                                                     \
+    WM_NLE(PP, false, 1)
   wm_prof_begin(WM_PC_NOISE, s);
   switch (h->p) {
     case 1: WM_NL(1); break;
@@ -225,6 +294,7 @@ int wm_k_noise_tiled(const wm_hier* h, uint64_t seed, int sample_first, int row0
     default: return WM_ERR_UNSUPPORTED;
   }
 #undef WM_NL
+#undef WM_NLE
   wm_prof_end(WM_PC_NOISE, s);
   WM_CUDA(cudaGetLastError());
   int64_t n2 = (int64_t)L.N * ns;
@@ -331,10 +401,10 @@ extern "C" int wm_noise_loads_noalloc(wm_hier_t h, uint64_t seed, int n_samples,
   int64_t n1 = (int64_t)L.E * n_samples;
   unsigned g1 = (unsigned)((n1 + 127) / 128);
   switch (h->p) {
-    case 1: WM_LAUNCH(WM_PC_NOISE, s, k_noise_local<1><<<g1, 128, 0, s>>>(L.E, L.nu, L.nv, n_samples, 0, seed, L.d_metric.p, h->d_gw.p, L.d_bu.p, L.d_bv.p, bl)); break;
-    case 2: WM_LAUNCH(WM_PC_NOISE, s, k_noise_local<2><<<g1, 128, 0, s>>>(L.E, L.nu, L.nv, n_samples, 0, seed, L.d_metric.p, h->d_gw.p, L.d_bu.p, L.d_bv.p, bl)); break;
-    case 3: WM_LAUNCH(WM_PC_NOISE, s, k_noise_local<3><<<g1, 128, 0, s>>>(L.E, L.nu, L.nv, n_samples, 0, seed, L.d_metric.p, h->d_gw.p, L.d_bu.p, L.d_bv.p, bl)); break;
-    case 4: WM_LAUNCH(WM_PC_NOISE, s, k_noise_local<4><<<g1, 128, 0, s>>>(L.E, L.nu, L.nv, n_samples, 0, seed, L.d_metric.p, h->d_gw.p, L.d_bu.p, L.d_bv.p, bl)); break;
+    case 1: WM_LAUNCH(WM_PC_NOISE, s, (k_noise_local<1, false, 1><<<g1, 128, 0, s>>>(L.E, L.nu, L.nv, n_samples, 0, seed, L.d_metric.p, h->d_gw.p, L.d_bu.p, L.d_bv.p, bl, nullptr))); break;
+    case 2: WM_LAUNCH(WM_PC_NOISE, s, (k_noise_local<2, false, 1><<<g1, 128, 0, s>>>(L.E, L.nu, L.nv, n_samples, 0, seed, L.d_metric.p, h->d_gw.p, L.d_bu.p, L.d_bv.p, bl, nullptr))); break;
+    case 3: WM_LAUNCH(WM_PC_NOISE, s, (k_noise_local<3, false, 1><<<g1, 128, 0, s>>>(L.E, L.nu, L.nv, n_samples, 0, seed, L.d_metric.p, h->d_gw.p, L.d_bu.p, L.d_bv.p, bl, nullptr))); break;
+    case 4: WM_LAUNCH(WM_PC_NOISE, s, (k_noise_local<4, false, 1><<<g1, 128, 0, s>>>(L.E, L.nu, L.nv, n_samples, 0, seed, L.d_metric.p, h->d_gw.p, L.d_bu.p, L.d_bv.p, bl, nullptr))); break;
     default: return WM_ERR_UNSUPPORTED;
   }
   WM_CUDA(cudaGetLastError());
