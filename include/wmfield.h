@@ -226,8 +226,10 @@ int wm_assemble_hierarchy(wm_geom_t geom, int n_levels, void* stream, wm_hier_t*
  * with NULL restores them.  Errors: WM_ERR_INVALID_ARG for values out of range.
  */
 typedef struct {
-  int uni_run;      /* consecutive one-shift tiles one block of the stencil kernels
-                       serves (window ids and combined rows built once), 1..8 (8)   */
+  int uni_run;      /* consecutive one-shift tiles one block of the float64 stencil
+                       and the true-residual kernels serves (window ids and combined
+                       rows built once), 1..8 (8); the float streaming kernels take
+                       four at a time                                               */
   int uni_waves;    /* grid target of those kernels, in waves of resident blocks:
                        runs are split over more blocks until the grid reaches it,
                        1..64 (4)                                                    */

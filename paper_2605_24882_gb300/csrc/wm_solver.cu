@@ -17,7 +17,8 @@
 //
 // Layout: systems are packed 32 per tile, vectors are [tiles][N][32]; lane =
 // system.  Levels with a stencil form run their operator steps in the
-// shared-memory kernels of wm_stencil.cu; the row kernels here give each warp
+// streaming kernels of wm_stream.h (float) and the shared-memory kernels of
+// wm_stencil.cu (float64, true residuals); the row kernels here give each warp
 // one row of kTPW tiles, a row's packed entries (column, S, M) loaded once per
 // warp and reused for 4 x 32 systems.  Per-system dot products are per-lane
 // sums over rows followed by a fixed-order reduction over warps and chunks
@@ -172,6 +173,7 @@ __global__ void __launch_bounds__(256) k_apply_pq(int N, int W, int chunks, int 
                                                   const double* __restrict__ sigma, const T* __restrict__ p,
                                                   T* __restrict__ q, const int* __restrict__ tile_active,
                                                   double* part_pq) {
+  wm_wait_previous();
   const int t0 = blockIdx.y * kTPW;
   const int lane = threadIdx.x;
   bool act[kTPW];
@@ -299,6 +301,7 @@ template <typename T>
 __global__ void k_update_xr(int N, int chunks, int tiles, const double* __restrict__ alpha, const T* __restrict__ p,
                             const T* __restrict__ q, double* __restrict__ x, T* __restrict__ r,
                             const int* __restrict__ tile_active, double* part_rr) {
+  wm_wait_previous();
   int t = blockIdx.y;
   if (!tile_active[t]) return;
   double a = alpha[t * WM_LANES + threadIdx.x];
@@ -347,6 +350,7 @@ template <typename T>
 __global__ void k_dots_rz_zq(int N, int chunks, int tiles, const T* __restrict__ r, const T* __restrict__ z,
                              const T* __restrict__ q, const int* __restrict__ tile_active, double* part_rz,
                              double* part_zq, const int* __restrict__ skip) {
+  wm_wait_previous();
   int t = blockIdx.y;
   if (!tile_active[t] || (skip && skip[t])) return;  // skip: tiles whose partials another kernel formed
   RowRange rr = chunk_rows(N, chunks);
@@ -367,6 +371,7 @@ __global__ void k_dots_rz_zq(int N, int chunks, int tiles, const T* __restrict__
 template <typename T>
 __global__ void k_update_p(int N, int chunks, const double* __restrict__ beta, const T* __restrict__ z,
                            T* __restrict__ p, const int* __restrict__ tile_active) {
+  wm_wait_previous();
   int t = blockIdx.y;
   if (!tile_active[t]) return;
   T b = (T)beta[t * WM_LANES + threadIdx.x];
@@ -452,6 +457,7 @@ __global__ void __launch_bounds__(WM_LANES * kSumWarps)
 
 __global__ void __launch_bounds__(WM_LANES * kSumWarps)
     k_scal_alpha(int chunks, const double* part_pq, const double* rho, int* active, double* alpha, int* flags) {
+  wm_wait_previous();
   __shared__ SumSm sm;
   const int g = blockIdx.x * WM_LANES + threadIdx.x;
   const bool act = active[g] != 0;
@@ -475,6 +481,7 @@ __global__ void __launch_bounds__(WM_LANES * kSumWarps)
     k_scal_conv(int chunks, const double* part_rr, const double* bb, const double* rr_ref, double rtol2,
                 double drop2, double* rr, int* active, int* rep, int* tile_active, int* tile_rep, int* counters,
                 int* flags) {
+  wm_wait_previous();
   __shared__ SumSm sm;
   const int g = blockIdx.x * WM_LANES + threadIdx.x;
   const bool act = active[g] != 0;
@@ -507,6 +514,7 @@ __global__ void __launch_bounds__(WM_LANES * kSumWarps)
 __global__ void __launch_bounds__(WM_LANES * kSumWarps)
     k_scal_replace(int chunks, const double* part_rr, const double* bb, double rtol2, const int* rep, double* rr,
                    double* rr_ref, int* active, int* restart, int* tile_active, int* counters, int* flags) {
+  wm_wait_previous();
   __shared__ SumSm sm;
   const int g = blockIdx.x * WM_LANES + threadIdx.x;
   const bool mine = rep[g] && active[g];
@@ -534,6 +542,7 @@ __global__ void __launch_bounds__(WM_LANES * kSumWarps)
 // residuals are recomputed in float64)
 __global__ void __launch_bounds__(WM_LANES * kSumWarps)
     k_df_check(int chunks, const double* part_b, const double* bb, double lim2, const int* rep, int* counter) {
+  wm_wait_previous();
   __shared__ SumSm sm;
   const int g = blockIdx.x * WM_LANES + threadIdx.x;
   const bool mine = rep[g] != 0;
@@ -545,6 +554,7 @@ __global__ void __launch_bounds__(WM_LANES * kSumWarps)
 __global__ void __launch_bounds__(WM_LANES * kSumWarps)
     k_scal_beta(int chunks, const double* part_rz, const double* part_zq, const double* alpha, const int* active,
                 int* restart, double* rho, double* beta) {
+  wm_wait_previous();
   __shared__ SumSm sm;
   const int g = blockIdx.x * WM_LANES + threadIdx.x;
   const bool upd = active[g] && !restart[g];
@@ -643,6 +653,7 @@ __global__ void k_cheb_first(int N, int chunks, int tiles, const T* __restrict__
                              const T* __restrict__ dM, const double* __restrict__ sigma,
                              const typename C2T<T>::type* __restrict__ ctab, const int* __restrict__ sid,
                              T* __restrict__ z, const int* __restrict__ tile_active, const int* __restrict__ skip) {
+  wm_wait_previous();
   const int t0 = blockIdx.y * kTPW;
   TileSet ts = tile_set(t0, tiles, tile_active);
   if (skip) {  // tiles done by another kernel
@@ -707,6 +718,7 @@ __global__ void __launch_bounds__(256) k_cheb_step(int N, int W, int chunks, int
                                                    const int* __restrict__ sid, const T* __restrict__ r,
                                                    const T* __restrict__ zin, const T* prev, T* out,
                                                    const int* __restrict__ tile_active) {
+  wm_wait_previous();
   const int t0 = blockIdx.y * kTPW;
   const int lane = threadIdx.x;
   TileSet ts = tile_set(t0, tiles, tile_active);
@@ -759,6 +771,7 @@ __global__ void __launch_bounds__(256) k_residual(int N, int W, int chunks, int 
                                                   const double* __restrict__ sigma, const T* __restrict__ r,
                                                   const T* __restrict__ z, T* __restrict__ res,
                                                   const int* __restrict__ tile_active) {
+  wm_wait_previous();
   const int t0 = blockIdx.y * kTPW;
   const int lane = threadIdx.x;
   TileSet ts = tile_set(t0, tiles, tile_active);
@@ -799,6 +812,7 @@ __global__ void __launch_bounds__(256) k_transfer(int Nout, int Nin, int chunks,
                                                   const typename TrT<T>::type* __restrict__ ent,
                                                   const T* __restrict__ in, T* __restrict__ out,
                                                   const int* __restrict__ tile_active) {
+  wm_wait_previous();
   const int t0 = blockIdx.y * kTPW;
   const int lane = threadIdx.x;
   TileSet ts = tile_set(t0, tiles, tile_active);
@@ -856,6 +870,7 @@ __global__ void __launch_bounds__(256) k_transfer(int Nout, int Nin, int chunks,
 template <typename T>
 __global__ void k_coarse_solve(int N, const double* __restrict__ Ainv, const int* __restrict__ sid,
                                const T* __restrict__ r, T* __restrict__ z, const int* __restrict__ tile_active) {
+  wm_wait_previous();
   int t = blockIdx.y;
   if (!tile_active[t]) return;
   int g = t * WM_LANES + threadIdx.x;
@@ -926,6 +941,7 @@ template <bool STAGED, int LN>
 __global__ void __launch_bounds__(WM_LANES * kTailWarps, 1)
     k_vcycle_tail(const TailDesc D, const double* __restrict__ sigma, const int* __restrict__ sid,
                   const float* __restrict__ rin, float* __restrict__ zout, const int* __restrict__ tile_active) {
+  wm_wait_previous();
   extern __shared__ __align__(16) float sh[];
   constexpr int SPL = WM_LANES / LN;      // rows of a warp at once
   constexpr int RST = kTailWarps * SPL;   // rows of the block at once
@@ -1654,8 +1670,8 @@ static int vcycle_tail(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, 
   auto launch = [&](auto* kernel) -> int {
     WM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     WM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, pct));
-    WM_LAUNCH(WM_PC_VTAIL, s, kernel<<<bt.tiles * (split ? 4 : 1), blk, smem, s>>>(D, ws.sigma.p, ws.sid.p, rin, zo,
-                                                                                     ws.tile_active.p));
+    WM_TRY(wm_launch_next(WM_PC_VTAIL, kernel, bt.tiles * (split ? 4 : 1), blk, smem, s, D, ws.sigma.p, ws.sid.p,
+        rin, zo, ws.tile_active.p));
     return WM_OK;
   };
   if (split)
@@ -1714,8 +1730,8 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
   const int cre = l == 0 ? WM_PC_RESID0 : WM_PC_RESIDC;
   if (l == L - 1) {
     int gx = std::max(1, std::min(64, (Lv.N + kWarps - 1) / kWarps));
-    WM_LAUNCH(WM_PC_COARSE, s, k_coarse_solve<T><<<dim3(gx, tiles), kBlk, 0, s>>>(Lv.N, ws.ainv.p, ws.sid.p, rin, za,
-                                                                                   ta));
+    WM_TRY(wm_launch_next(WM_PC_COARSE, k_coarse_solve<T>, dim3(gx, tiles), kBlk, 0, s, Lv.N, ws.ainv.p, ws.sid.p,
+        rin, za, ta));
     units(WM_PC_COARSE, bt, 2.0 * Tb * Lv.N, 2.0 * Lv.N * Lv.N);
     WM_CUDA(cudaGetLastError());
     *zout = za;
@@ -1764,8 +1780,9 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
       }
       if (e != WM_OK) step_rc = e;
     } else {
-      WM_LAUNCH(csm, s, k_cheb_step<T><<<ogrid, oblk, 0, s>>>(Lv.N, Lv.W, och, tiles, k, pk, dS, dM, ws.sigma.p,
-                                                              ctab, ws.sid.p, rin, zin, prev, zo, ta));
+      const int e = wm_launch_next(csm, k_cheb_step<T>, ogrid, oblk, 0, s, Lv.N, Lv.W, och, tiles, k, pk, dS, dM,
+                                   ws.sigma.p, ctab, ws.sid.p, rin, zin, prev, zo, ta);
+      if (e != WM_OK) step_rc = e;
     }
     units(csm, bt, (has_prev ? 4.0 : 3.0) * Tb * Lv.N, 2.0 * Lv.nnz + 8.0 * Lv.N);
   };
@@ -1787,8 +1804,8 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
                                  csm, s));
       units(csm, bt, 3.0 * Tb * Lv.N, 2.0 * Lv.nnz + 8.0 * Lv.N);
       if (ws.n_uni_tiles < tiles) {
-        WM_LAUNCH(csm, s, k_cheb_first<T><<<ggrid, kBlk, 0, s>>>(Lv.N, ch, tiles, rin, dS, dM, ws.sigma.p, ctab,
-                                                                 ws.sid.p, za, ta, ws.tile_uni.p));
+        WM_TRY(wm_launch_next(csm, k_cheb_first<T>, ggrid, kBlk, 0, s, Lv.N, ch, tiles, rin, dS, dM, ws.sigma.p,
+            ctab, ws.sid.p, za, ta, ws.tile_uni.p));
         int e = wm_sten_cheb_step(Lv, h->np, h->p, tiles, 1, ws.sigma.p, ctab, ws.sid.p, rin, za, nullptr, zb, ta,
                                   uni_of(ws), csm, s, nullptr, nullptr, nullptr, true);
         if (e != WM_OK) return e;
@@ -1797,8 +1814,8 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
     std::swap(cur, oth);  // cur = z2, oth = z1
     k1 = 2;
   } else {
-    WM_LAUNCH(csm, s, k_cheb_first<T><<<ggrid, kBlk, 0, s>>>(Lv.N, ch, tiles, rin, dS, dM, ws.sigma.p, ctab,
-                                                             ws.sid.p, za, ta, (const int*)nullptr));
+    WM_TRY(wm_launch_next(csm, k_cheb_first<T>, ggrid, kBlk, 0, s, Lv.N, ch, tiles, rin, dS, dM, ws.sigma.p, ctab,
+        ws.sid.p, za, ta, (const int*)nullptr));
     units(csm, bt, 2.0 * Tb * Lv.N, 3.0 * Lv.N);
   }
   for (int k = k1; k < nu; ++k) {
@@ -1817,21 +1834,21 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
       WM_TRY(wm_sten_residual(Lv, h->np, h->p, tiles, ws.sigma.p, rin, cur, res, ta, uni_of(ws), cre, s));
     }
   } else {
-    WM_LAUNCH(cre, s, k_residual<T><<<ogrid, oblk, 0, s>>>(Lv.N, Lv.W, och, tiles, pk, ws.sigma.p, rin, cur, res,
-                                                           ta));
+    WM_TRY(wm_launch_next(cre, k_residual<T>, ogrid, oblk, 0, s, Lv.N, Lv.W, och, tiles, pk, ws.sigma.p, rin, cur,
+        res, ta));
   }
   units(cre, bt, 3.0 * Tb * Lv.N, 4.0 * Lv.nnz + 3.0 * Lv.N);
   WM_TRY(step_rc);
   const wm_level& Cv = h->lv[l + 1];
   T* rc = vb<T>(ws.lvl[l + 1].r);
   const int chc = bt.vcycle_chunks(Cv.N);
-  WM_LAUNCH(WM_PC_RESTRICT, s, k_transfer<T, false><<<dim3(chc, groups(tiles)), kBlk, 0, s>>>(
-                                   Cv.N, Lv.N, chc, tiles, Lv.d_Rptr.p, R_of<T>(Lv), res, rc, ta));
+  WM_TRY(wm_launch_next(WM_PC_RESTRICT, (k_transfer<T, false>), dim3(chc, groups(tiles)), kBlk, 0, s, Cv.N, Lv.N,
+      chc, tiles, Lv.d_Rptr.p, R_of<T>(Lv), res, rc, ta));
   units(WM_PC_RESTRICT, bt, Tb * (Lv.N + Cv.N), 2.0 * Lv.nnzP);
   T* zc = nullptr;
   WM_TRY(vcycle<T>(h, ws, bt, l + 1, rc, &zc, s));
-  WM_LAUNCH(WM_PC_PROLONG, s, k_transfer<T, true><<<ggrid, kBlk, 0, s>>>(Lv.N, Cv.N, ch, tiles, Lv.d_Pptr.p,
-                                                                         P_of<T>(Lv), zc, cur, ta));
+  WM_TRY(wm_launch_next(WM_PC_PROLONG, (k_transfer<T, true>), ggrid, kBlk, 0, s, Lv.N, Cv.N, ch, tiles, Lv.d_Pptr.p,
+      P_of<T>(Lv), zc, cur, ta));
   units(WM_PC_PROLONG, bt, Tb * (2.0 * Lv.N + Cv.N), 2.0 * Lv.nnzP);
   // post-smoothing from the corrected z (no z_prev at step 0)
   for (int k = 0; k < nu; ++k) {
@@ -1859,17 +1876,16 @@ static int bpx(const wm_hier* h, WorkSpace& ws, const Batch& bt, const T* rin, T
     const wm_level& Cv = h->lv[l + 1];
     const T* rl = l == 0 ? rin : vb<T>(ws.lvl[l].r);
     const int chc = bt.vcycle_chunks(Cv.N);
-    WM_LAUNCH(WM_PC_RESTRICT, s, k_transfer<T, false><<<dim3(chc, groups(tiles)), kBlk, 0, s>>>(
-                                     Cv.N, Lv.N, chc, tiles, Lv.d_Rptr.p, R_of<T>(Lv), rl, vb<T>(ws.lvl[l + 1].r),
-                                     ta));
+    WM_TRY(wm_launch_next(WM_PC_RESTRICT, (k_transfer<T, false>), dim3(chc, groups(tiles)), kBlk, 0, s, Cv.N, Lv.N,
+        chc, tiles, Lv.d_Rptr.p, R_of<T>(Lv), rl, vb<T>(ws.lvl[l + 1].r), ta));
     units(WM_PC_RESTRICT, bt, Tb * (Lv.N + Cv.N), 2.0 * Lv.nnzP);
   }
   {
     const wm_level& Cv = h->lv[L - 1];
     const T* rc = L == 1 ? rin : vb<T>(ws.lvl[L - 1].r);
     int gx = std::max(1, std::min(64, (Cv.N + kWarps - 1) / kWarps));
-    WM_LAUNCH(WM_PC_COARSE, s, k_coarse_solve<T><<<dim3(gx, tiles), kBlk, 0, s>>>(Cv.N, ws.ainv.p, ws.sid.p, rc,
-                                                                                   vb<T>(ws.lvl[L - 1].za), ta));
+    WM_TRY(wm_launch_next(WM_PC_COARSE, k_coarse_solve<T>, dim3(gx, tiles), kBlk, 0, s, Cv.N, ws.ainv.p, ws.sid.p,
+        rc, vb<T>(ws.lvl[L - 1].za), ta));
     units(WM_PC_COARSE, bt, 2.0 * Tb * Cv.N, 2.0 * Cv.N * Cv.N);
   }
   for (int l = L - 2; l >= 0; --l) {
@@ -1883,9 +1899,8 @@ static int bpx(const wm_hier* h, WorkSpace& ws, const Batch& bt, const T* rin, T
     WM_LAUNCH(cat, s, k_diag_scale<T><<<ggrid, kBlk, 0, s>>>(Lv.N, ch, tiles, rl, dS_of<T>(Lv), dM_of<T>(Lv),
                                                              ws.sigma.p, zl, ta));
     units(cat, bt, 2.0 * Tb * Lv.N, 3.0 * Lv.N);
-    WM_LAUNCH(WM_PC_PROLONG, s, k_transfer<T, true><<<ggrid, kBlk, 0, s>>>(Lv.N, Cv.N, ch, tiles, Lv.d_Pptr.p,
-                                                                           P_of<T>(Lv), vb<T>(ws.lvl[l + 1].za), zl,
-                                                                           ta));
+    WM_TRY(wm_launch_next(WM_PC_PROLONG, (k_transfer<T, true>), ggrid, kBlk, 0, s, Lv.N, Cv.N, ch, tiles,
+        Lv.d_Pptr.p, P_of<T>(Lv), vb<T>(ws.lvl[l + 1].za), zl, ta));
     units(WM_PC_PROLONG, bt, Tb * (2.0 * Lv.N + Cv.N), 2.0 * Lv.nnzP);
   }
   WM_CUDA(cudaGetLastError());
@@ -1931,9 +1946,8 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
     WM_TRY(bpx<T>(h, ws, bt, r, &z, s));
   else
     WM_TRY(vcycle<T>(h, ws, bt, 0, r, &z, s));
-  WM_LAUNCH(WM_PC_CGVEC, s, k_dots_rz_zq<T><<<grid, kBlk, 0, s>>>(N, ch, tiles, r, z, (const T*)nullptr,
-                                                                  ws.tile_active.p, ws.part[1].p, ws.part[2].p,
-                                                                  (const int*)nullptr));
+  WM_TRY(wm_launch_next(WM_PC_CGVEC, k_dots_rz_zq<T>, grid, kBlk, 0, s, N, ch, tiles, r, z, (const T*)nullptr,
+      ws.tile_active.p, ws.part[1].p, ws.part[2].p, (const int*)nullptr));
   WM_LAUNCH(WM_PC_SCALAR, s, k_scal_init<<<tiles, kSumBlk, 0, s>>>(ch, ws.part[0].p, ws.part[1].p, ws.src_of.p,
                                                             ws.bb.p, ws.rho.p, ws.rr.p, ws.rr_ref.p, ws.active.p,
                                                             ws.restart.p, ws.flags.p));
@@ -1942,7 +1956,7 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
   WM_CUDA(cudaGetLastError());
   // p = z
   WM_CUDA(cudaMemsetAsync(ws.beta.p, 0, nsys_pad * sizeof(double), s));
-  WM_LAUNCH(WM_PC_CGVEC, s, k_update_p<T><<<grid, kBlk, 0, s>>>(N, ch, ws.beta.p, z, p, ws.tile_active.p));
+  WM_TRY(wm_launch_next(WM_PC_CGVEC, k_update_p<T>, grid, kBlk, 0, s, N, ch, ws.beta.p, z, p, ws.tile_active.p));
   const double rtol2 = bt.rtol * bt.rtol;
   const double drop2 = bt.replace_drop * bt.replace_drop;
   int it = 0, n_rep_total = 0;
@@ -1962,22 +1976,20 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
                                 ws.part[0].p, s));
       }
     } else {
-      WM_LAUNCH(WM_PC_APPLY64, s, k_apply_pq<T><<<ggrid, kBlk, 0, s>>>(N, L0.W, ch, tiles, rows_of<T>(L0),
-                                                                       ws.sigma.p, p, q, ws.tile_active.p,
-                                                                       ws.part[0].p));
+      WM_TRY(wm_launch_next(WM_PC_APPLY64, k_apply_pq<T>, ggrid, kBlk, 0, s, N, L0.W, ch, tiles, rows_of<T>(L0),
+          ws.sigma.p, p, q, ws.tile_active.p, ws.part[0].p));
     }
     units(WM_PC_APPLY64, bt, 2.0 * Tb * N, 4.0 * L0.nnz + 4.0 * N);
-    WM_LAUNCH(WM_PC_SCALAR, s, k_scal_alpha<<<tiles, kSumBlk, 0, s>>>(ch_st, ws.part[0].p, ws.rho.p, ws.active.p,
-                                                               ws.alpha.p, ws.flags.p));
-    WM_LAUNCH(WM_PC_CGVEC, s, k_update_xr<T><<<grid, kBlk, 0, s>>>(N, ch, tiles, ws.alpha.p, p, q, ws.x.p, r,
-                                                                   ws.tile_active.p, ws.part[0].p));
+    WM_TRY(wm_launch_next(WM_PC_SCALAR, k_scal_alpha, tiles, kSumBlk, 0, s, ch_st, ws.part[0].p, ws.rho.p,
+        ws.active.p, ws.alpha.p, ws.flags.p));
+    WM_TRY(wm_launch_next(WM_PC_CGVEC, k_update_xr<T>, grid, kBlk, 0, s, N, ch, tiles, ws.alpha.p, p, q, ws.x.p, r,
+        ws.tile_active.p, ws.part[0].p));
     units(WM_PC_CGVEC, bt, (16.0 + 4.0 * Tb) * N, 6.0 * N);
     WM_CUDA(cudaMemsetAsync(cnt, 0, 8 * sizeof(int), s));
     WM_CUDA(cudaMemsetAsync(ws.tile_active.p, 0, tiles * sizeof(int), s));
     WM_CUDA(cudaMemsetAsync(ws.tile_rep.p, 0, tiles * sizeof(int), s));
-    WM_LAUNCH(WM_PC_SCALAR, s, k_scal_conv<<<tiles, kSumBlk, 0, s>>>(ch, ws.part[0].p, ws.bb.p, ws.rr_ref.p, rtol2,
-                                                              drop2, ws.rr.p, ws.active.p, ws.rep.p, ws.tile_active.p,
-                                                              ws.tile_rep.p, cnt, ws.flags.p));
+    WM_TRY(wm_launch_next(WM_PC_SCALAR, k_scal_conv, tiles, kSumBlk, 0, s, ch, ws.part[0].p, ws.bb.p, ws.rr_ref.p,
+        rtol2, drop2, ws.rr.p, ws.active.p, ws.rep.p, ws.tile_active.p, ws.tile_rep.p, cnt, ws.flags.p));
     WM_CUDA(cudaGetLastError());
     WM_CUDA(cudaMemcpyAsync(ws.host_small, cnt, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
     WM_CUDA(cudaStreamSynchronize(s));
@@ -1995,8 +2007,8 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
             WM_TRY(wm_sten_true_residual_df(L0, h->np, h->p, tiles, uni_of(ws), ws.sid.p, ws.sigma.p, ws.x.p, rhs_tiled,
                                             ws.src_of.p, ws.rep.p, ws.tile_rep.p, r, ws.part[1].p, ws.part[2].p, s));
             WM_CUDA(cudaMemsetAsync(cnt + 5, 0, sizeof(int), s));
-            WM_LAUNCH(WM_PC_SCALAR, s, k_df_check<<<tiles, kSumBlk, 0, s>>>(ch_op, ws.part[2].p, ws.bb.p,
-                                                                     0.01 * rtol2, ws.rep.p, cnt + 5));
+            WM_TRY(wm_launch_next(WM_PC_SCALAR, k_df_check, tiles, kSumBlk, 0, s, ch_op, ws.part[2].p, ws.bb.p, 0.01
+                * rtol2, ws.rep.p, cnt + 5));
             WM_CUDA(cudaGetLastError());
             WM_CUDA(cudaMemcpyAsync(ws.host_small + 8, cnt + 5, sizeof(int), cudaMemcpyDeviceToHost, s));
             WM_CUDA(cudaStreamSynchronize(s));
@@ -2024,9 +2036,8 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
       }
       WM_CUDA(cudaMemsetAsync(cnt, 0, 8 * sizeof(int), s));
       WM_CUDA(cudaMemsetAsync(ws.tile_active.p, 0, tiles * sizeof(int), s));
-      WM_LAUNCH(WM_PC_SCALAR, s, k_scal_replace<<<tiles, kSumBlk, 0, s>>>(ch_op, ws.part[1].p, ws.bb.p, rtol2,
-                                                                   ws.rep.p, ws.rr.p, ws.rr_ref.p, ws.active.p,
-                                                                   ws.restart.p, ws.tile_active.p, cnt, ws.flags.p));
+      WM_TRY(wm_launch_next(WM_PC_SCALAR, k_scal_replace, tiles, kSumBlk, 0, s, ch_op, ws.part[1].p, ws.bb.p, rtol2,
+          ws.rep.p, ws.rr.p, ws.rr_ref.p, ws.active.p, ws.restart.p, ws.tile_active.p, cnt, ws.flags.p));
       WM_CUDA(cudaGetLastError());
       WM_CUDA(cudaMemcpyAsync(ws.host_small, cnt, 4 * sizeof(int), cudaMemcpyDeviceToHost, s));
       WM_CUDA(cudaStreamSynchronize(s));
@@ -2047,15 +2058,13 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
     const int ch_dots = vd.fused ? ch_st : ch;
     if (vd.fused) units(WM_PC_SMOOTH0, bt, Tb * N, 4.0 * N);  // q read and the two products
     if (!vd.fused || (!STREAM && ws.n_uni_tiles < tiles)) {
-      WM_LAUNCH(WM_PC_CGVEC, s, k_dots_rz_zq<T><<<dim3(ch_dots, tiles), kBlk, 0, s>>>(
-                                    N, ch_dots, tiles, r, z, q, ws.tile_active.p, ws.part[1].p, ws.part[2].p,
-                                    vd.fused ? ws.tile_uni.p : (const int*)nullptr));
+      WM_TRY(wm_launch_next(WM_PC_CGVEC, k_dots_rz_zq<T>, dim3(ch_dots, tiles), kBlk, 0, s, N, ch_dots, tiles, r, z,
+          q, ws.tile_active.p, ws.part[1].p, ws.part[2].p, vd.fused ? ws.tile_uni.p : (const int*)nullptr));
       if (!vd.fused) units(WM_PC_CGVEC, bt, 3.0 * Tb * N, 4.0 * N);
     }
-    WM_LAUNCH(WM_PC_SCALAR, s, k_scal_beta<<<tiles, kSumBlk, 0, s>>>(ch_dots, ws.part[1].p, ws.part[2].p,
-                                                              ws.alpha.p, ws.active.p, ws.restart.p, ws.rho.p,
-                                                              ws.beta.p));
-    WM_LAUNCH(WM_PC_CGVEC, s, k_update_p<T><<<grid, kBlk, 0, s>>>(N, ch, ws.beta.p, z, p, ws.tile_active.p));
+    WM_TRY(wm_launch_next(WM_PC_SCALAR, k_scal_beta, tiles, kSumBlk, 0, s, ch_dots, ws.part[1].p, ws.part[2].p,
+        ws.alpha.p, ws.active.p, ws.restart.p, ws.rho.p, ws.beta.p));
+    WM_TRY(wm_launch_next(WM_PC_CGVEC, k_update_p<T>, grid, kBlk, 0, s, N, ch, ws.beta.p, z, p, ws.tile_active.p));
     units(WM_PC_CGVEC, bt, 3.0 * Tb * N, 2.0 * N);
     WM_CUDA(cudaGetLastError());
   }

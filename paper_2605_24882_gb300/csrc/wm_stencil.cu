@@ -197,6 +197,7 @@ __global__ void __launch_bounds__(BU * 32, 1) k_sten(StenGeo G, const double2* _
                                                      const double* __restrict__ src, int tiles,
                                                      const int* __restrict__ tile_active, const Epi epi_arg,
                                                      const int* __restrict__ skip_uni) {
+  wm_wait_previous();
   using LY = SmemLayout<P, BVT, Epi::NIN>;
   constexpr int BV = LY::BV, NIN = Epi::NIN, SW = 2 * P + 1, CU = LY::CU, NC = LY::NC, S2 = LY::S2;
   constexpr int ROWCH = 32 * sizeof(double) / 16;  // 16-byte chunks per staged row
@@ -369,6 +370,7 @@ __global__ void __launch_bounds__(BU * 32, (UniMinBlocks<P, MODE>::value))
                const double* prev, double* out, int tiles, const int* __restrict__ tile_active,
                const int2* __restrict__ groups, int split, double* __restrict__ part, const double* __restrict__ qd,
                double* __restrict__ part2, double* __restrict__ out1) {
+  wm_wait_previous();
   using LY = UniLayout<P, MODE>;
   constexpr bool CHEB = UniCheb<MODE>::value;
   constexpr int BV = LY::BV, SW = 2 * P + 1, CU = LY::CU, NC = LY::NC, S2 = LY::S2, S2P = LY::S2P;
@@ -610,8 +612,8 @@ int launch_bv(const wm_level& L, int np, int tiles, const double* src, const int
   StenGeo G = geo_of(L);
   G.nbv = (L.nlv + BVT - 1) / BVT;
   dim3 grid(np * G.nbu * G.nbv, tiles);
-  WM_LAUNCH(cat, s, k_sten<P, BVT, Epi><<<grid, dim3(32, BU), sm, s>>>(G, L.d_csm64.p, src, tiles, tile_active, epi,
-                                                                       skip_uni));
+  WM_TRY(wm_launch_next(cat, (k_sten<P, BVT, Epi>), grid, dim3(32, BU), sm, s, G, L.d_csm64.p, src, tiles,
+      tile_active, epi, skip_uni));
   WM_CUDA(cudaGetLastError());
   return WM_OK;
 }
@@ -734,6 +736,7 @@ __global__ void __launch_bounds__(BU * 32, 2)
                       const double* __restrict__ rhs, const int* __restrict__ src_of, const int* __restrict__ rep,
                       float* __restrict__ r, double* __restrict__ part, double* __restrict__ part_bound,
                       const int* __restrict__ skip_uni, const int* __restrict__ few) {
+  wm_wait_previous();
   constexpr int BV = BvOf<P>::value;
   using LY = DfLayout<P>;
   constexpr int SW = 2 * P + 1, CU = LY::CU, NC = LY::NC, S2 = LY::S2;
@@ -918,6 +921,7 @@ __global__ void __launch_bounds__(BU * 32, 2)
                           const double* __restrict__ rhs, const int* __restrict__ src_of,
                           const int* __restrict__ rep, float* __restrict__ r, double* __restrict__ part,
                           double* __restrict__ part_bound) {
+  wm_wait_previous();
   using LY = DfFewLayout<P>;
   constexpr int BV = LY::BV, SW = 2 * P + 1, CU = LY::CU, NC = LY::NC, S2 = LY::S2, NPS = LY::NPS;
   constexpr int NT = BU * 32;
@@ -1061,6 +1065,7 @@ __global__ void __launch_bounds__(BU * 32, 3)
                           const double* __restrict__ sigma, const double* __restrict__ rhs,
                           const int* __restrict__ src_of, const int* __restrict__ rep, float* __restrict__ r,
                           double* __restrict__ part, double* __restrict__ part_bound) {
+  wm_wait_previous();
   constexpr int BV = BvOf<P>::value;
   using LY = DfUniLayout<P>;
   constexpr int SW = 2 * P + 1, CU = LY::CU, NC = LY::NC, S2 = LY::S2;
@@ -1286,9 +1291,9 @@ static int launch_uni(const wm_level& L, int np, int tiles, const UniTiles& ut, 
   for (int g0 = 0; g0 < ut.n_groups; g0 += gmax) {
     const int ng = std::min(gmax, ut.n_groups - g0);
     dim3 grid(bx, ng * split);
-    WM_LAUNCH(cat, s, k_sten_uni<P, MODE><<<grid, dim3(32, BU), sm, s>>>(
-                          geo_of(L), L.d_csm64.p, L.d_dS64.p, L.d_dM64.p, sigma, ctab, sid, kstep, z, r, prev, out,
-                          tiles, tile_active, ut.groups + g0, split, part, qd, part2, out1));
+    WM_TRY(wm_launch_next(cat, (k_sten_uni<P, MODE>), grid, dim3(32, BU), sm, s, geo_of(L), L.d_csm64.p, L.d_dS64.p,
+        L.d_dM64.p, sigma, ctab, sid, kstep, z, r, prev, out, tiles, tile_active, ut.groups + g0, split, part, qd,
+        part2, out1));
     WM_CUDA(cudaGetLastError());
   }
   return WM_OK;
@@ -1407,23 +1412,22 @@ static int launch_df(const wm_level& L, int np, int tiles, const UniTiles& ut, c
     const int gmax = 65535 / split;
     for (int g0 = 0; g0 < ut.n_groups; g0 += gmax) {
       const int ng = std::min(gmax, ut.n_groups - g0);
-      WM_LAUNCH(WM_PC_TRUERES, s, k_sten_trueres_df_uni<P><<<dim3(bx, ng * split), dim3(32, BU), smu, s>>>(
-                                      geo_of(L), L.d_csmdf.p, x, tiles, tile_rep, ut.groups + g0, split, sigma, rhs,
-                                      src_of, rep, r, part, part_bound));
+      WM_TRY(wm_launch_next(WM_PC_TRUERES, k_sten_trueres_df_uni<P>, dim3(bx, ng * split), dim3(32, BU), smu, s,
+          geo_of(L), L.d_csmdf.p, x, tiles, tile_rep, ut.groups + g0, split, sigma, rhs, src_of, rep, r, part,
+          part_bound));
       WM_CUDA(cudaGetLastError());
     }
   }
   const dim3 grid(bx, tiles);
   if (ut.n_few > 0) {
-    WM_LAUNCH(WM_PC_TRUERES, s, k_sten_trueres_df_few<P><<<grid, dim3(32, BU), DfFewLayout<P>::total(ut.few_max), s>>>(
-                                    geo_of(L), L.d_csmdf.p, x, tiles, tile_rep, ut.few, ut.few_max, sid, sigma, rhs,
-                                    src_of, rep, r, part, part_bound));
+    WM_TRY(wm_launch_next(WM_PC_TRUERES, k_sten_trueres_df_few<P>, grid, dim3(32, BU),
+        DfFewLayout<P>::total(ut.few_max), s, geo_of(L), L.d_csmdf.p, x, tiles, tile_rep, ut.few, ut.few_max, sid,
+        sigma, rhs, src_of, rep, r, part, part_bound));
     WM_CUDA(cudaGetLastError());
   }
   if (ut.n + ut.n_few < tiles) {
-    WM_LAUNCH(WM_PC_TRUERES, s, k_sten_trueres_df<P><<<grid, dim3(32, BU), sm, s>>>(
-                                    geo_of(L), L.d_csmdf.p, x, tiles, tile_rep, sigma, rhs, src_of, rep, r, part,
-                                    part_bound, ut.flag, ut.few));
+    WM_TRY(wm_launch_next(WM_PC_TRUERES, k_sten_trueres_df<P>, grid, dim3(32, BU), sm, s, geo_of(L), L.d_csmdf.p, x,
+        tiles, tile_rep, sigma, rhs, src_of, rep, r, part, part_bound, ut.flag, ut.few));
     WM_CUDA(cudaGetLastError());
   }
   return WM_OK;

@@ -140,6 +140,7 @@ __global__ void __launch_bounds__(kBU * 32, TPB == 1 ? kBlocks1 : kBlocks)
              const float* prev, const float* __restrict__ q, float* out, float* __restrict__ out1,
              const int2* __restrict__ groups, int g0, const int* __restrict__ tile_active, double* __restrict__ part,
              double* __restrict__ part2) {
+  wm_wait_previous();
   using LY = StreamLayout<P, MODE, NSH, TPB>;
   using CR = ColRow<P>;
   constexpr int SW = CR::SW, S2 = CR::S2, CW = LY::CW, NIN = LY::NIN, STAGE = LY::STAGE, CELL = LY::CELL;
@@ -510,10 +511,9 @@ int launch_stream_n(const StreamArgs& a, const StreamGeo& G, const int2* groups,
     configured = true;
   }
   for (int g0 = 0; g0 < n; g0 += 65535) {  // grid.y limit
-    WM_LAUNCH(a.cat, a.s,
-              k_stream<P, MODE, NSH, TPB><<<dim3(G.items, std::min(65535, n - g0)), dim3(32, kBU), sm, a.s>>>(
-                  G, a.sigma, a.ctab, a.sid, a.kstep, a.z, a.r, a.prev, a.q, a.out, a.out1, groups, g0,
-                  a.tile_active, a.part, a.part2));
+    WM_TRY(wm_launch_next(a.cat, (k_stream<P, MODE, NSH, TPB>), dim3(G.items, std::min(65535, n - g0)), dim3(32,
+        kBU), sm, a.s, G, a.sigma, a.ctab, a.sid, a.kstep, a.z, a.r, a.prev, a.q, a.out, a.out1, groups, g0,
+        a.tile_active, a.part, a.part2));
     WM_CUDA(cudaGetLastError());
   }
   return WM_OK;
