@@ -21,8 +21,7 @@ namespace {
 
 constexpr int BU = 8;   // outputs per block along u (one warp each)
 // outputs per warp along v: for p = 2 the patches have 2^l + 2 local DOFs per
-// side, which a height of 6 covers with less waste than 8 (66 and 18 exactly;
-// coarse-level smoothing 33.9 -> 32.0 ms per bench step)
+// side, which a height of 6 covers with less waste than 8 (66 and 18 exactly)
 #ifndef WM_BV_P2
 #define WM_BV_P2 6
 #endif

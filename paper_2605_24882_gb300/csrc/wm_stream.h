@@ -25,7 +25,7 @@
 // reads) and latency at 16 warps per SM, which the 128 registers of the running
 // sums of four tiles allow.  The tile-at-a-time kernel it replaces read every
 // window value 2p+1 times and the coefficients once per tile (26 load wavefronts
-// and 105 instructions per output against 19 and 60).  Chebyshev step, level 0 of
+// and 105 instructions per output against 16 and 60).  Chebyshev step, level 0 of
 // the 64 x 64 sphere (p = 2), 568 tiles in runs of eight of one shift: 1.83 -> 1.47 ms
 // (3.2 -> 4.0 TB/s); 256 x 256 torus (p = 3), 72 tiles in such runs 1.09 -> 0.66 ms.
 // Mixed shifts, rate of the level-0 smoothing: 213 systems on the 256 x 256 sphere
