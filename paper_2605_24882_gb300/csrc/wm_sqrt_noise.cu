@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(256) k_ms_init(int N, int K, const double* __r
 __global__ void __launch_bounds__(256) k_ms_apply(int N, int W, const int32_t* __restrict__ col,
                                                   const double* __restrict__ M, const double* __restrict__ p,
                                                   double* __restrict__ q, double* __restrict__ part) {
+  wm_wait_previous();
   const int t = blockIdx.y, l = threadIdx.x;
   const double* pt = p + (size_t)t * N * WM_LANES;
   double acc = 0.0;
@@ -112,6 +113,7 @@ __global__ void __launch_bounds__(256) k_ms_apply(int N, int W, const int32_t* _
 __global__ void __launch_bounds__(256) k_ms_resid(int N, const double* __restrict__ a,
                                                   const double* __restrict__ q, double* __restrict__ r,
                                                   double* __restrict__ part) {
+  wm_wait_previous();
   const int t = blockIdx.y, l = threadIdx.x;
   const double av = a[(size_t)t * WM_LANES + l];
   double acc = 0.0;
@@ -160,7 +162,9 @@ __global__ void __launch_bounds__(256) k_ms_start(int nsamp, int nchunk, int K, 
 // seed step length a_n = (r, r) / (p, M p)
 __global__ void __launch_bounds__(256) k_ms_alpha(int nchunk, const double* __restrict__ part,
                                                   SampleState* __restrict__ st, double* __restrict__ a_out,
-                                                  int* __restrict__ flags) {
+                                                  int* __restrict__ n_active, int* __restrict__ flags) {
+  wm_wait_previous();
+  if (blockIdx.x == 0 && threadIdx.x == 0 && threadIdx.y == 0) *n_active = 0;  // counted by this step's k_ms_shifts
   const int g = blockIdx.x * WM_LANES + threadIdx.x;
   const double pq = tile_sum(part, nchunk, gridDim.x);
   if (threadIdx.y != 0) return;
@@ -187,6 +191,7 @@ __global__ void __launch_bounds__(256) k_ms_shifts(int nsamp, int nchunk, int K,
                                                    double* __restrict__ gk, double* __restrict__ hk,
                                                    double* __restrict__ b_out, int* __restrict__ n_active,
                                                    int* __restrict__ flags) {
+  wm_wait_previous();
   __shared__ int any[WM_LANES];
   const int g = blockIdx.x * WM_LANES + threadIdx.x;
   if (threadIdx.y == 0) any[threadIdx.x] = 0;
@@ -253,6 +258,7 @@ __global__ void __launch_bounds__(256) k_ms_update(int N, int K, int nsamp, cons
                                                    const double* __restrict__ b, const double* __restrict__ r,
                                                    double* __restrict__ p, double* __restrict__ acc_s,
                                                    double* __restrict__ ds) {
+  wm_wait_previous();
   const int t = blockIdx.y, tiles = gridDim.y;
   const int g = t * WM_LANES + threadIdx.x;
   const size_t nblk = (size_t)tiles * N * WM_LANES;
@@ -365,15 +371,16 @@ extern "C" int wm_noise_loads_sqrt(wm_hier_t h, uint64_t seed, int n_samples, do
     int it = 0, host_active = 1;
     while (it < max_iter && host_active > 0) {
       ++it;
-      WM_LAUNCH(WM_PC_NOISE, s, k_ms_apply<<<rgrid, rblock, 0, s>>>(N, L.W, L.d_col.p, L.d_M64.p, p.p, q.p, part.p));
-      WM_LAUNCH(WM_PC_NOISE, s, k_ms_alpha<<<tc, rblock, 0, s>>>(nchunk, part.p, st.p, a.p, counters.p + 1));
-      WM_LAUNCH(WM_PC_NOISE, s, k_ms_resid<<<rgrid, rblock, 0, s>>>(N, a.p, q.p, r.p, part.p));
-      WM_CUDA(cudaMemsetAsync(counters.p, 0, sizeof(int), s));
-      WM_LAUNCH(WM_PC_NOISE, s, k_ms_shifts<<<tc, rblock, 0, s>>>(nsamp, nchunk, K, part.p, d_w2.p, d_c.p, rtol, st.p,
-                                                                  zeta.p, zeta_old.p, shift_active.p, tile_shift.p,
-                                                                  gk.p, hk.p, b.p, counters.p, counters.p + 1));
-      WM_LAUNCH(WM_PC_NOISE, s, k_ms_update<<<ugrid, rblock, 0, s>>>(N, K, nsamp, tile_shift.p, gk.p, hk.p, b.p, r.p,
-                                                                     p.p, acc.p, ds.p));
+      WM_TRY(wm_launch_next(WM_PC_NOISE, k_ms_apply, rgrid, rblock, 0, s, N, L.W, L.d_col.p, L.d_M64.p, p.p, q.p,
+                            part.p));
+      WM_TRY(wm_launch_next(WM_PC_NOISE, k_ms_alpha, tc, rblock, 0, s, nchunk, part.p, st.p, a.p, counters.p,
+                            counters.p + 1));
+      WM_TRY(wm_launch_next(WM_PC_NOISE, k_ms_resid, rgrid, rblock, 0, s, N, a.p, q.p, r.p, part.p));
+      WM_TRY(wm_launch_next(WM_PC_NOISE, k_ms_shifts, tc, rblock, 0, s, nsamp, nchunk, K, part.p, d_w2.p, d_c.p, rtol,
+                            st.p, zeta.p, zeta_old.p, shift_active.p, tile_shift.p, gk.p, hk.p, b.p, counters.p,
+                            counters.p + 1));
+      WM_TRY(wm_launch_next(WM_PC_NOISE, k_ms_update, ugrid, rblock, 0, s, N, K, nsamp, tile_shift.p, gk.p, hk.p, b.p,
+                            r.p, p.p, acc.p, ds.p));
       WM_CUDA(cudaGetLastError());
       if (it % 4 == 0 || it == max_iter) {
         int hc[2] = {0, 0};
