@@ -612,8 +612,9 @@ extern "C" int wm_restrict(wm_hier_t h, int level, const double* rf, double* rc,
   return transfer(h, level, rf, rc, n_vec, false, stream);
 }
 
-static int set_batch_meta(WorkSpace& ws, const wm_schedule& sc, int tiles, const std::vector<double>& sigma,
-                          const std::vector<int>& sid, const std::vector<int>& src, cudaStream_t s) {
+static int set_batch_meta(wm_hier_t h, WorkSpace& ws, int tiles, const std::vector<double>& sigma,
+                          const std::vector<int>& sid, const std::vector<int>& src, cudaStream_t s,
+                          int64_t per_batch = 0) {
   size_t n = (size_t)tiles * WM_LANES;
   std::vector<double> sg(n, sigma.empty() ? 1.0 : sigma[0]);
   std::vector<int> si(n, 0), sr(n, -1);
@@ -627,6 +628,9 @@ static int set_batch_meta(WorkSpace& ws, const wm_schedule& sc, int tiles, const
       si[g] = si[g - 1];
     }
   }
+  const wm_schedule& sc = h->sched;
+  const double far = *std::max_element(sg.begin(), sg.end());
+  ws.far = std::any_of(h->lv.begin(), h->lv.end(), [&](const wm_level& L) { return wm_stream_far(L, far); });
   // tiles whose 32 shifts are equal (bit for bit) take the combined-coefficient kernels
   std::vector<int> uni(tiles, 1);
   int n_uni = 0;
@@ -639,25 +643,19 @@ static int set_batch_meta(WorkSpace& ws, const wm_schedule& sc, int tiles, const
     n_uni += uni[t];
   }
   ws.n_uni_tiles = n_uni;
-  // other tiles with few distinct shift indices (the double-float residual combines
-  // the rows for each)
-  std::vector<int> few(tiles, 0);
-  ws.n_few_tiles = ws.few_max = 0;
+  // chunks of the other tiles' dot products at a V-cycle's end (k_dots_rz_zq): 1 the vector
+  // kernels' chunks, 2 the stencil blocks' where the tile shares the solve with tiles of
+  // one shift.  A remainder tile that a batch takes along (batch_size) counts as a solve of
+  // its own, which keeps the float sums of both as they are in two batches.
+  const int whole = per_batch > WM_LANES ? std::min<int64_t>(tiles, per_batch / WM_LANES) : tiles;
+  bool fused = false;
+  for (int t = 0; t < whole; ++t) fused |= uni[t] != 0;
+  std::vector<int> dots(tiles);
+  ws.dots_sten = false;
   for (int t = 0; t < tiles; ++t) {
-    if (uni[t]) continue;
-    int seen[kDfFew], nd = 0;
-    for (int l = 0; l < WM_LANES && nd <= kDfFew; ++l) {
-      const int v = si[(size_t)t * WM_LANES + l];
-      if (std::find(seen, seen + std::min(nd, kDfFew), v) != seen + std::min(nd, kDfFew)) continue;
-      if (nd < kDfFew) seen[nd] = v;
-      ++nd;
-    }
-    if (nd > kDfFew) continue;
-    few[t] = 1;
-    ws.n_few_tiles += 1;
-    ws.few_max = std::max(ws.few_max, nd);
+    dots[t] = uni[t] ? 0 : fused && t < whole ? 2 : 1;
+    ws.dots_sten |= dots[t] == 2;
   }
-  WM_CUDA(cudaMemcpyAsync(ws.tile_few.p, few.data(), tiles * sizeof(int), cudaMemcpyHostToDevice, s));
   // groups of at most kUniGroup consecutive one-shift tiles with the same shift
   // index (one block of the one-shift kernel per group and spatial block)
   std::vector<int2> grp;
@@ -676,10 +674,17 @@ static int set_batch_meta(WorkSpace& ws, const wm_schedule& sc, int tiles, const
   }
   std::vector<int> tshift(tiles);
   for (int t = 0; t < tiles; ++t) tshift[t] = si[(size_t)t * WM_LANES];
-  std::vector<int2> sgrp;
-  wm_stream_groups(uni, tshift, sgrp, ws.st_n);
+  std::vector<int4> sgrp;
+  std::vector<int> order;
+  wm_stream_groups(uni, tshift, sgrp, order, &ws.st);
   WM_TRY(ws.st_groups.alloc(sgrp.size()));
-  WM_CUDA(cudaMemcpyAsync(ws.st_groups.p, sgrp.data(), sgrp.size() * sizeof(int2), cudaMemcpyHostToDevice, s));
+  WM_TRY(ws.st_order.alloc(tiles));
+  ws.st.groups = ws.st_groups.p;
+  ws.st.order = ws.st_order.p;
+  for (int k = 0; k < ws.st.n_uni; ++k) dots[order[k]] = k < ws.st.n_pair ? 0 : 3;
+  WM_CUDA(cudaMemcpyAsync(ws.st_groups.p, sgrp.data(), sgrp.size() * sizeof(int4), cudaMemcpyHostToDevice, s));
+  WM_CUDA(cudaMemcpyAsync(ws.tile_dots.p, dots.data(), tiles * sizeof(int), cudaMemcpyHostToDevice, s));
+  WM_CUDA(cudaMemcpyAsync(ws.st_order.p, order.data(), tiles * sizeof(int), cudaMemcpyHostToDevice, s));
   ws.n_uni_groups = (int)grp.size();
   ws.uni_waves = sc.uni_waves;
   if (!grp.empty()) {
@@ -727,7 +732,7 @@ extern "C" int wm_vcycle(wm_hier_t h, int n_vec, const double* sigma, const doub
       src[g] = g;
     }
   }
-  WM_TRY(set_batch_meta(ws, h->sched, tiles, sg, sid, src, s));
+  WM_TRY(set_batch_meta(h, ws, tiles, sg, sid, src, s));
   WM_TRY(wm_prepare_shifts(h, ws, shl, s));
   Batch bt;
   bt.schedule(h->sched);
@@ -881,10 +886,10 @@ int64_t batch_size(wm_hier_t h, WorkSpace& ws, const wm_sample_desc* d, int64_t 
   return std::max<int64_t>(1, per_batch);
 }
 
-// one batched solve of the systems [g0, g1) of a pass (g = j * ns + s); the
-// solutions are left in ws.x
+// one batched solve of the systems [g0, g1) of a pass (g = j * ns + s) that takes
+// per_batch at a time; the solutions are left in ws.x
 int solve_range(wm_hier_t h, WorkSpace& ws, const wm_sample_desc* d, const Pass& ps, int64_t g0, int64_t g1,
-                const double* rhs_t, wm_stats* st, int* worst, cudaStream_t s) {
+                int64_t per_batch, const double* rhs_t, wm_stats* st, int* worst, cudaStream_t s) {
   bool dbl = d->precision == WM_FP64;
   int nj = (int)ps.sigma.size();
   int nb = (int)(g1 - g0);
@@ -898,7 +903,7 @@ int solve_range(wm_hier_t h, WorkSpace& ws, const wm_sample_desc* d, const Pass&
     sid[k] = ps.sid_base + j;
     src[k] = (int)(g % ps.ns);
   }
-  WM_TRY(set_batch_meta(ws, h->sched, tiles, sg, sid, src, s));
+  WM_TRY(set_batch_meta(h, ws, tiles, sg, sid, src, s, per_batch));
   Batch bt;
   bt.schedule(h->sched);
   bt.tiles = tiles;
@@ -940,7 +945,7 @@ int run_pass(wm_hier_t h, WorkSpace& ws, const wm_sample_desc* d, const Pass& ps
   WM_TRY(ws.reserve(h, (int)((per_batch + WM_LANES - 1) / WM_LANES), ps.nshift_total, d->precision == WM_FP64));
   for (int64_t g0 = 0; g0 < nsys; g0 += per_batch) {
     int64_t g1 = std::min(nsys, g0 + per_batch);
-    WM_TRY(solve_range(h, ws, d, ps, g0, g1, rhs_t, st, worst, s));
+    WM_TRY(solve_range(h, ws, d, ps, g0, g1, per_batch, rhs_t, st, worst, s));
     WM_TRY(sink((int)g0, (int)g1, s));
   }
   return WM_OK;
@@ -1334,7 +1339,7 @@ int sample_fields_group(wm_hier_t h, const std::vector<const wm_sample_desc*>& D
       const int tiles = (nb + WM_LANES - 1) / WM_LANES;
       std::vector<double> bsg(sg.begin() + g0, sg.begin() + g1);
       std::vector<int> bsid(sid.begin() + g0, sid.begin() + g1), bsrc(src.begin() + g0, src.begin() + g1);
-      WM_TRY(set_batch_meta(ws, h->sched, tiles, bsg, bsid, bsrc, s));
+      WM_TRY(set_batch_meta(h, ws, tiles, bsg, bsid, bsrc, s, per_batch));
       Batch bt;
       bt.schedule(h->sched);
       bt.tiles = tiles;
@@ -1600,12 +1605,12 @@ extern "C" int wm_sample_fields_backward(wm_hier_t h, const wm_sample_desc* d, c
         if (xp[p]) {
           xb = xp[p] + (size_t)(g0 / WM_LANES) * N * WM_LANES;
         } else {
-          WM_TRY(solve_range(h, ws, d, fp, g0, g1, rp[p], st, &worst, s));
+          WM_TRY(solve_range(h, ws, d, fp, g0, g1, per_batch_f, rp[p], st, &worst, s));
           xb = ws.x.p;
         }
         WM_TRY(wm_k_apply_mass64(L0, tiles, xb, ws.mx.p, nullptr, s));
       }
-      WM_TRY(solve_range(h, ws, d, fp, g0, g1, dout, st, &worst, s));
+      WM_TRY(solve_range(h, ws, d, fp, g0, g1, per_batch_f, dout, st, &worst, s));
       WM_TRY(wm_sinc_accumulate(h, ns, (int)g0, (int)g1, ws.coef.p, ws.x.p, dr, s));
       if (grad_kappa) {
         WM_TRY(wm_system_dots(ws, tiles, N, ws.x.p, ws.mx.p, dots, s));

@@ -150,6 +150,7 @@ struct wm_level {
   DevBuf<int32_t> d_st_ext, d_st_done;
   DevBuf<float2> d_st_dext;
   DevBuf<unsigned char> d_st_cols;
+  float diag_max[2] = {0.f, 0.f};  // of S and M
   // the same coefficients as float pairs (S_hi, S_lo, M_hi, M_lo) for the
   // double-float residual
   DevBuf<float4> d_csmdf;

@@ -345,25 +345,62 @@ __global__ void k_update_xr(int N, int chunks, int tiles, const double* __restri
   block_reduce_store<1, 1>(v, parts, chunks, t, tiles);
 }
 
-// partials (r, z) and (z, q)
+// Partial sums of the dot products at a V-cycle's end: the chunks of a tile by its kind
+// (kind = nullptr: n[1] for all; 0 and 3: tiles of one shift, 1 and 2: others), in rows
+// of `stride` chunks.
+struct DotRows {
+  const int* kind = nullptr;
+  int n[4] = {0, 0, 0, 0};
+  int stride = 0;
+  __device__ __forceinline__ int of(int t) const { return n[kind ? kind[t] : 1]; }
+};
+
+// partials (r, z) and (z, q) of the tiles in `list` (nullptr: all)
 template <typename T>
-__global__ void k_dots_rz_zq(int N, int chunks, int tiles, const T* __restrict__ r, const T* __restrict__ z,
+__global__ void k_dots_rz_zq(int N, int tiles, const T* __restrict__ r, const T* __restrict__ z,
                              const T* __restrict__ q, const int* __restrict__ tile_active, double* part_rz,
-                             double* part_zq, const int* __restrict__ skip) {
+                             double* part_zq, const DotRows D, const int* __restrict__ list) {
   wm_wait_previous();
-  int t = blockIdx.y;
-  if (!tile_active[t] || (skip && skip[t])) return;  // skip: tiles whose partials another kernel formed
+  const int t = list ? list[blockIdx.y] : blockIdx.y;
+  const int chunks = D.of(t);
+  if (!tile_active[t] || (int)blockIdx.x >= chunks) return;
   RowRange rr = chunk_rows(N, chunks);
-  Acc<T> a0, a1;
-  for (int i = rr.i0 + threadIdx.y; i < rr.i1; i += kWarps) {
-    size_t k = vidx(t, N, i);
-    T zv = z[k];
-    a0.add(r[k] * zv);
-    if (q) a1.add(zv * q[k]);
+  // Acc's sums, sixteen rows of a warp at a time: a test for the flush in every row costs
+  // the float64 unit's time even where it fails (117 million rows x systems with it: 864 us)
+  constexpr int UR = 4, GR = 16 / UR;  // rows in flight together
+  double d0 = 0.0, d1 = 0.0;
+  int i = rr.i0 + threadIdx.y;
+  for (; i + 15 * kWarps < rr.i1; i += 16 * kWarps) {
+    T f0 = 0, f1 = 0;
+#pragma unroll
+    for (int h = 0; h < GR; ++h) {
+      T rv[UR], zv[UR], qv[UR];
+#pragma unroll
+      for (int u = 0; u < UR; ++u) {
+        const size_t k = vidx(t, N, i + (h * UR + u) * kWarps);
+        rv[u] = r[k];
+        zv[u] = z[k];
+        qv[u] = q ? q[k] : (T)0;
+      }
+#pragma unroll
+      for (int u = 0; u < UR; ++u) {
+        f0 += rv[u] * zv[u];
+        f1 += zv[u] * qv[u];
+      }
+    }
+    d0 += (double)f0;
+    d1 += (double)f1;
   }
-  double v[2][1] = {{a0.get()}, {a1.get()}};
+  T f0 = 0, f1 = 0;
+  for (; i < rr.i1; i += kWarps) {
+    const size_t k = vidx(t, N, i);
+    const T zv = z[k];
+    f0 += r[k] * zv;
+    if (q) f1 += zv * q[k];
+  }
+  double v[2][1] = {{d0 + (double)f0}, {d1 + (double)f1}};
   double* parts[2] = {part_rz, part_zq};
-  block_reduce_store<2, 1>(v, parts, chunks, t, tiles);
+  block_reduce_store<2, 1>(v, parts, D.stride, t, tiles);
 }
 
 // p = z + beta p; with beta = 0 (the first direction, a restart) p = z without
@@ -416,11 +453,13 @@ struct SumSm {
 };
 // sum of the chunk partials of system (tile blockIdx.x, lane); valid in warp 0.
 // Every thread of the block calls it; `want` false skips the lane's loads (0).
-__device__ __forceinline__ double tile_parts(const double* part, int chunks, bool want, SumSm& sm) {
+// stride: chunks of a tile's row of `part` (0: chunks).
+__device__ __forceinline__ double tile_parts(const double* part, int chunks, bool want, SumSm& sm, int stride = 0) {
   const int t = blockIdx.x, lane = threadIdx.x, y = threadIdx.y;
+  if (stride == 0) stride = chunks;
   double s = 0.0;
   if (want)
-    for (int c = y; c < chunks; c += kSumWarps) s += part[((size_t)t * chunks + c) * WM_LANES + lane];
+    for (int c = y; c < chunks; c += kSumWarps) s += part[((size_t)t * stride + c) * WM_LANES + lane];
   sm.v[y][lane] = s;
   __syncthreads();
   double r = 0.0;
@@ -552,14 +591,15 @@ __global__ void __launch_bounds__(WM_LANES * kSumWarps)
 }
 
 __global__ void __launch_bounds__(WM_LANES * kSumWarps)
-    k_scal_beta(int chunks, const double* part_rz, const double* part_zq, const double* alpha, const int* active,
+    k_scal_beta(const DotRows D, const double* part_rz, const double* part_zq, const double* alpha, const int* active,
                 int* restart, double* rho, double* beta) {
   wm_wait_previous();
   __shared__ SumSm sm;
   const int g = blockIdx.x * WM_LANES + threadIdx.x;
   const bool upd = active[g] && !restart[g];
-  const double rz = tile_parts(part_rz, chunks, true, sm);
-  const double zq = tile_parts(part_zq, chunks, upd, sm);
+  const int chunks = D.of(blockIdx.x);
+  const double rz = tile_parts(part_rz, chunks, true, sm, D.stride);
+  const double zq = tile_parts(part_zq, chunks, upd, sm, D.stride);
   if (threadIdx.y != 0) return;
   double b = 0.0;
   if (upd) {
@@ -1337,30 +1377,19 @@ static UniTiles uni_of(const WorkSpace& ws) {
   UniTiles u;
   u.flag = ws.tile_uni.p;
   u.n = ws.n_uni_tiles;
-  u.few = ws.tile_few.p;
-  u.n_few = ws.n_few_tiles;
-  u.few_max = ws.few_max;
   u.groups = ws.uni_groups.p;
   u.n_groups = ws.n_uni_groups;
   u.waves = ws.uni_waves;
   return u;
 }
 
-// the batch's tiles as the streaming kernels take them
-static StreamTiles stream_tiles(const WorkSpace& ws, int tiles) {
-  StreamTiles t;
-  t.tiles = tiles;
-  t.groups = ws.st_groups.p;
-  for (int k = 0; k < 2; ++k) t.n[k] = ws.st_n[k];
-  return t;
-}
 // what every step of the streaming kernels on a level takes
 static StreamArgs stream_args(const wm_hier* h, const WorkSpace& ws, const Batch& bt, const wm_level& L,
                               const float2* ctab, int cat, cudaStream_t s) {
   StreamArgs a;
   a.L = &L;
   a.np = h->np;
-  a.st = stream_tiles(ws, bt.tiles);
+  a.st = ws.st;
   a.sigma = ws.sigma.p;
   a.ctab = ctab;
   a.sid = ws.sid.p;
@@ -1407,7 +1436,7 @@ int WorkSpace::reserve(const wm_hier* h, int tiles, int nshift, bool dbl) {
   WM_TRY(tile_active.alloc(tiles));
   WM_TRY(tile_rep.alloc(tiles));
   WM_TRY(tile_uni.alloc(tiles));
-  WM_TRY(tile_few.alloc(tiles));
+  WM_TRY(tile_dots.alloc(tiles));
   WM_TRY(rho.alloc(ns));
   WM_TRY(alpha.alloc(ns));
   WM_TRY(beta.alloc(ns));
@@ -1442,9 +1471,8 @@ void WorkSpace::release() {
   }
   lvl.clear();
   sigma.release(); sid.release(); src_of.release(); active.release(); rep.release(); restart.release();
-  tile_active.release(); tile_rep.release(); tile_uni.release(); tile_few.release();
-  uni_groups.release();
-  st_groups.release();
+  tile_active.release(); tile_rep.release(); tile_uni.release(); tile_dots.release();
+  uni_groups.release(); st_groups.release(); st_order.release();
   rho.release(); alpha.release(); beta.release(); bb.release(); rr.release(); rr_ref.release();
   for (auto& pp : part) pp.release();
   flags.release(); counters.release(); lmax.release(); ainv.release(); shifts.release(); statd.release();
@@ -1695,13 +1723,15 @@ struct VDots {
   const T* q = nullptr;
   double* prz = nullptr;
   double* pzq = nullptr;
+  int stride = 0;  // partial sums of a tile's row
   bool fused = false;
 };
 
 // one V-cycle from level l on residual rin, returns the buffer holding z.
 // With dots given (level 0 of the outer solve), the last post-smoothing step of
-// the one-shift tiles also forms the partials (r, z) and (z, q) of the outer CG
-// in dots->prz / dots->pzq; dots->fused reports whether it did.
+// one-shift tiles also forms the partials (r, z) and (z, q) of the outer CG in
+// dots->prz / dots->pzq (float: of the tiles that wm_stream_items counts);
+// dots->fused reports whether it did.
 template <typename T>
 static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const T* rin, T** zout, cudaStream_t s,
                   VDots<T>* dots = nullptr) {
@@ -1748,6 +1778,7 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
     }
   }
   constexpr bool STREAM = std::is_same<T, float>::value;  // the float steps of stencil levels
+  const bool sten = Lv.sten && !(STREAM && ws.far);
   T* res = vb<T>(B.res);
   const int nu = bt.degree_of(l);
   int step_rc = WM_OK;
@@ -1755,7 +1786,8 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
   // (has_prev false: z_prev = 0, or unused at k = 0)
   auto cheb_step = [&](int k, const T* zin, T* zo, bool has_prev, VDots<T>* dd) {
     const T* prev = has_prev ? zo : nullptr;
-    if (Lv.sten) {
+    if (sten) {
+      const bool fuse = dd && ws.n_uni_tiles > 0;
       int e = WM_OK;
       if constexpr (STREAM) {
         StreamArgs a = stream_args(h, ws, bt, Lv, ctab, csm, s);
@@ -1764,20 +1796,19 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
         a.r = rin;
         a.prev = prev;
         a.out = zo;
-        if (dd) {
+        if (fuse) {
           a.q = dd->q;
           a.part = dd->prz;
           a.part2 = dd->pzq;
-          dd->fused = true;
+          a.pstride = dd->stride;
         }
-        e = wm_stream(h->p, dd ? ST_CHEBDOT : ST_CHEB, a);
+        e = wm_stream(h->p, fuse ? ST_CHEBDOT : ST_CHEB, a);
       } else {
-        const bool fuse = dd && ws.n_uni_tiles > 0;
         e = wm_sten_cheb_step(Lv, h->np, h->p, tiles, k, ws.sigma.p, ctab, ws.sid.p, rin, zin, prev, zo, ta,
                               uni_of(ws), csm, s, fuse ? dd->q : nullptr, fuse ? dd->prz : nullptr,
                               fuse ? dd->pzq : nullptr);
-        if (fuse) dd->fused = true;
       }
+      if (fuse) dd->fused = true;
       if (e != WM_OK) step_rc = e;
     } else {
       const int e = wm_launch_next(csm, k_cheb_step<T>, ogrid, oblk, 0, s, Lv.N, Lv.W, och, tiles, k, pk, dS, dM,
@@ -1791,10 +1822,10 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
   T* cur = za;
   T* oth = zb;
   int k1 = 1;
-  if (Lv.sten && (STREAM || ws.n_uni_tiles > 0) && nu >= 2) {
+  if (sten && (STREAM || ws.n_uni_tiles > 0) && nu >= 2) {
     if constexpr (STREAM) {
       StreamArgs a = stream_args(h, ws, bt, Lv, ctab, csm, s);
-      a.z = rin;
+      a.z = a.r = rin;
       a.out1 = za;
       a.out = zb;
       WM_TRY(wm_stream(h->p, ST_CHEB1, a));
@@ -1823,7 +1854,7 @@ static int vcycle(const wm_hier* h, WorkSpace& ws, const Batch& bt, int l, const
     std::swap(cur, oth);
   }
   // residual, restriction, coarse correction
-  if (Lv.sten) {
+  if (sten) {
     if constexpr (STREAM) {
       StreamArgs a = stream_args(h, ws, bt, Lv, ctab, cre, s);
       a.z = cur;
@@ -1946,8 +1977,10 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
     WM_TRY(bpx<T>(h, ws, bt, r, &z, s));
   else
     WM_TRY(vcycle<T>(h, ws, bt, 0, r, &z, s));
-  WM_TRY(wm_launch_next(WM_PC_CGVEC, k_dots_rz_zq<T>, grid, kBlk, 0, s, N, ch, tiles, r, z, (const T*)nullptr,
-      ws.tile_active.p, ws.part[1].p, ws.part[2].p, (const int*)nullptr));
+  DotRows all;
+  all.n[1] = all.stride = ch;
+  WM_TRY(wm_launch_next(WM_PC_CGVEC, k_dots_rz_zq<T>, grid, kBlk, 0, s, N, tiles, r, z, (const T*)nullptr,
+      ws.tile_active.p, ws.part[1].p, ws.part[2].p, all, (const int*)nullptr));
   WM_LAUNCH(WM_PC_SCALAR, s, k_scal_init<<<tiles, kSumBlk, 0, s>>>(ch, ws.part[0].p, ws.part[1].p, ws.src_of.p,
                                                             ws.bb.p, ws.rho.p, ws.rr.p, ws.rr_ref.p, ws.active.p,
                                                             ws.restart.p, ws.flags.p));
@@ -1962,9 +1995,17 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
   int it = 0, n_rep_total = 0;
   bool df_res = bt.df_residual;
   constexpr bool STREAM = std::is_same<T, float>::value;
-  const int ch_st = STREAM && L0.sten ? wm_stream_items(L0, h->np, h->p, stream_tiles(ws, tiles)) : ch_op;
+  const bool sten = L0.sten && !(STREAM && ws.far);  // the outer apply's kernel
+  int n_fused = ws.st.n_uni;  // of the first tiles of ws.st.order whose dot products the V-cycle's last step forms
+  const int ch_st = !sten ? ch : STREAM ? wm_stream_items(L0, h->np, h->p, ws.st, &n_fused) : ch_op;
+  DotRows rows;  // where the V-cycle's last step forms those of some tiles
+  rows.kind = ws.tile_dots.p;
+  rows.n[0] = n_fused > 0 ? ch_st : ch_op;
+  rows.n[1] = STREAM ? ch : ch_op;  // (float64 sums hardly depend on it)
+  rows.n[2] = rows.n[3] = ch_op;
+  rows.stride = std::max(ch_st, std::max(rows.n[1], ch_op));
   for (it = 1; it <= bt.max_iter; ++it) {
-    if (L0.sten) {
+    if (sten) {
       if constexpr (STREAM) {
         StreamArgs a = stream_args(h, ws, bt, L0, ws.cheb32.p, WM_PC_APPLY64, s);
         a.z = p;
@@ -2004,7 +2045,7 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
         bool done = false;
         if constexpr (std::is_same<T, float>::value) {
           if (df_res) {
-            WM_TRY(wm_sten_true_residual_df(L0, h->np, h->p, tiles, uni_of(ws), ws.sid.p, ws.sigma.p, ws.x.p, rhs_tiled,
+            WM_TRY(wm_sten_true_residual_df(L0, h->np, h->p, tiles, uni_of(ws), ws.sigma.p, ws.x.p, rhs_tiled,
                                             ws.src_of.p, ws.rep.p, ws.tile_rep.p, r, ws.part[1].p, ws.part[2].p, s));
             WM_CUDA(cudaMemsetAsync(cnt + 5, 0, sizeof(int), s));
             WM_TRY(wm_launch_next(WM_PC_SCALAR, k_df_check, tiles, kSumBlk, 0, s, ch_op, ws.part[2].p, ws.bb.p, 0.01
@@ -2045,25 +2086,31 @@ static int fcg(const wm_hier* h, WorkSpace& ws, const Batch& bt, const double* r
       bt.active_tiles = ws.host_small[2];
     }
     if (n_active == 0) break;
-    // the V-cycle's last step forms (r, z) and (z, q) for the one-shift tiles
-    // (chunks = its spatial blocks); the dots kernel covers the other tiles
+    // the V-cycle's last step forms (r, z) and (z, q) for the first n_fused of the
+    // one-shift tiles (float64: for all of them), the dots kernels for the others
     VDots<T> vd;
     vd.q = q;
     vd.prz = ws.part[1].p;
     vd.pzq = ws.part[2].p;
+    vd.stride = rows.stride;
     if (bt.precond == WM_PRECOND_BPX)
       WM_TRY(bpx<T>(h, ws, bt, r, &z, s));
     else
       WM_TRY(vcycle<T>(h, ws, bt, 0, r, &z, s, &vd));
-    const int ch_dots = vd.fused ? ch_st : ch;
+    const DotRows& dr = vd.fused ? rows : all;
     if (vd.fused) units(WM_PC_SMOOTH0, bt, Tb * N, 4.0 * N);  // q read and the two products
-    if (!vd.fused || (!STREAM && ws.n_uni_tiles < tiles)) {
-      WM_TRY(wm_launch_next(WM_PC_CGVEC, k_dots_rz_zq<T>, dim3(ch_dots, tiles), kBlk, 0, s, N, ch_dots, tiles, r, z,
-          q, ws.tile_active.p, ws.part[1].p, ws.part[2].p, vd.fused ? ws.tile_uni.p : (const int*)nullptr));
+    if constexpr (STREAM)
+      if (vd.fused && n_fused < ws.st.n_uni)
+        WM_TRY(wm_sten_dots(L0, h->np, h->p, ws.st.order + n_fused, ws.st.n_uni - n_fused, r, z, q, ws.tile_active.p,
+                            ws.part[1].p, ws.part[2].p, rows.stride, s));
+    if (!vd.fused || ws.st.n_uni < tiles) {
+      const int skip = vd.fused ? ws.st.n_uni : 0, most = vd.fused && (ws.dots_sten || !STREAM) ? ch_op : ch;
+      WM_TRY(wm_launch_next(WM_PC_CGVEC, k_dots_rz_zq<T>, dim3(most, tiles - skip), kBlk, 0, s, N, tiles, r, z, q,
+          ws.tile_active.p, ws.part[1].p, ws.part[2].p, dr, vd.fused ? ws.st.order + skip : nullptr));
       if (!vd.fused) units(WM_PC_CGVEC, bt, 3.0 * Tb * N, 4.0 * N);
     }
-    WM_TRY(wm_launch_next(WM_PC_SCALAR, k_scal_beta, tiles, kSumBlk, 0, s, ch_dots, ws.part[1].p, ws.part[2].p,
-        ws.alpha.p, ws.active.p, ws.restart.p, ws.rho.p, ws.beta.p));
+    WM_TRY(wm_launch_next(WM_PC_SCALAR, k_scal_beta, tiles, kSumBlk, 0, s, dr, ws.part[1].p, ws.part[2].p, ws.alpha.p,
+        ws.active.p, ws.restart.p, ws.rho.p, ws.beta.p));
     WM_TRY(wm_launch_next(WM_PC_CGVEC, k_update_p<T>, grid, kBlk, 0, s, N, ch, ws.beta.p, z, p, ws.tile_active.p));
     units(WM_PC_CGVEC, bt, 3.0 * Tb * N, 2.0 * N);
     WM_CUDA(cudaGetLastError());
@@ -2151,9 +2198,11 @@ int wm_system_dots(WorkSpace& ws, int tiles, int N, const double* a, const doubl
     return WM_ERR_INVALID_ARG;
   }
   WM_TRY(set_all_tiles_active(ws, tiles, s));
+  DotRows all;
+  all.n[1] = all.stride = ch;
   WM_LAUNCH(WM_PC_SINC, s, k_dots_rz_zq<double><<<dim3(ch, tiles), kBlk, 0, s>>>(
-                               N, ch, tiles, a, b, (const double*)nullptr, ws.tile_active.p, ws.part[1].p,
-                               ws.part[2].p, (const int*)nullptr));
+                               N, tiles, a, b, (const double*)nullptr, ws.tile_active.p, ws.part[1].p, ws.part[2].p,
+                               all, nullptr));
   WM_LAUNCH(WM_PC_SINC, s, k_sum_parts<<<nblk(nsys_pad, 128), 128, 0, s>>>(nsys_pad, ch, ws.part[1].p, ws.dots.p));
   WM_CUDA(cudaGetLastError());
   out.resize(nsys_pad);

@@ -7,6 +7,7 @@
 #endif
 
 #include "wm_internal.h"
+#include "wm_stencil.h"
 
 // float or double buffer (only the one of the solve's precision is allocated)
 struct VBuf {
@@ -76,13 +77,15 @@ struct WorkSpace {
   DevBuf<int> src_of;         // per system right-hand-side sample (-1: padding)
   DevBuf<int> active, rep, restart, tile_active, tile_rep;
   DevBuf<int> tile_uni;       // 1 where the 32 shifts of a tile are equal
-  DevBuf<int> tile_few;       // 1 where another tile has at most kDfFew shift indices
-  int n_few_tiles = 0, few_max = 0;
+  DevBuf<int> tile_dots;      // chunks of a tile's dot products (DotRows)
+  bool dots_sten = false;     // tile_dots has a 2
   int n_uni_tiles = 0;        // host count of such tiles in the current batch
   DevBuf<int2> uni_groups;    // runs of at most 8 consecutive such tiles of one shift: (first tile, count)
   int n_uni_groups = 0;
-  DevBuf<int2> st_groups;     // the tiles grouped for the streaming kernels (StreamTiles)
-  int st_n[2] = {0, 0};
+  DevBuf<int4> st_groups;     // the tiles grouped for the streaming kernels (StreamTiles)
+  DevBuf<int> st_order;
+  StreamTiles st;
+  bool far = false;           // a shift of the batch is beyond the streaming kernels (wm_stream_far)
   int uni_waves = 4;          // grid target of the one-shift kernels (the hierarchy's schedule)
   DevBuf<double> rho, alpha, beta, bb, rr, rr_ref;
   DevBuf<double> part[3];

@@ -626,6 +626,55 @@ int launch(const wm_level& L, int np, int tiles, const double* src, const int* t
   return launch_bv<P, 2>(L, np, tiles, src, tile_active, epi, cat, s, skip_uni);
 }
 
+// dot products of float vectors by the row blocks of the kernels above: products of a
+// column's rows in float, then double
+template <int P>
+__global__ void __launch_bounds__(BU * 32)
+    k_sten_dots(StenGeo G, const int* __restrict__ list, const float* __restrict__ r, const float* __restrict__ z,
+                const float* __restrict__ q, const int* __restrict__ tile_active, double* __restrict__ part_rz,
+                double* __restrict__ part_zq, int stride) {
+  wm_wait_previous();
+  constexpr int BV = BvOf<P>::value;
+  const int t = list[blockIdx.y], lane = threadIdx.x, w = threadIdx.y;
+  if (!tile_active[t]) return;
+  int b = blockIdx.x;
+  const int bu = b % G.nbu;
+  b /= G.nbu;
+  const int bv = b % G.nbv, m = b / G.nbv;
+  const int iu = bu * BU + w;
+  float rz = 0.f, zq = 0.f;
+  if (iu < G.nlu) {
+    const int32_t* own = G.own + ((size_t)m * G.nlv + bv * BV) * G.nlu + iu;
+    int id[BV];
+    float rv[BV], zv[BV], qv[BV];
+#pragma unroll
+    for (int j = 0; j < BV; ++j) id[j] = bv * BV + j < G.nlv ? own[(size_t)j * G.nlu] : -1;
+#pragma unroll
+    for (int j = 0; j < BV; ++j) {
+      const size_t o = ((size_t)t * G.N + max(id[j], 0)) * 32 + lane;
+      rv[j] = id[j] >= 0 ? r[o] : 0.f;
+      zv[j] = id[j] >= 0 ? z[o] : 0.f;
+      qv[j] = id[j] >= 0 ? q[o] : 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < BV; ++j)
+      if (id[j] >= 0) {
+        rz = fmaf(rv[j], zv[j], rz);
+        zq = fmaf(zv[j], qv[j], zq);
+      }
+  }
+  __shared__ double red[2][BU][32];
+  red[0][w][lane] = rz;
+  red[1][w][lane] = zq;
+  __syncthreads();
+  if (w < 2) {
+    double a = 0.0;
+#pragma unroll
+    for (int y = 0; y < BU; ++y) a += red[w][y][lane];
+    (w == 0 ? part_rz : part_zq)[((size_t)t * stride + blockIdx.x) * 32 + lane] = a;
+  }
+}
+
 // ------------------------------------------- double-float true residual
 // r = b - (S x + sigma M x) of the systems flagged for residual replacement,
 // with every operation on the FP32 pipes: the FP64 rate of this part is
@@ -734,7 +783,7 @@ __global__ void __launch_bounds__(BU * 32, 2)
                       const int* __restrict__ tile_rep, const double* __restrict__ sigma,
                       const double* __restrict__ rhs, const int* __restrict__ src_of, const int* __restrict__ rep,
                       float* __restrict__ r, double* __restrict__ part, double* __restrict__ part_bound,
-                      const int* __restrict__ skip_uni, const int* __restrict__ few) {
+                      const int* __restrict__ skip_uni) {
   wm_wait_previous();
   constexpr int BV = BvOf<P>::value;
   using LY = DfLayout<P>;
@@ -753,7 +802,7 @@ __global__ void __launch_bounds__(BU * 32, 2)
   const int bv = b % G.nbv;
   const int m = b / G.nbv;
   const int t = blockIdx.y;
-  if (t >= tiles || !tile_rep[t] || skip_uni[t] || few[t]) return;  // done by the kernels for one and few shifts
+  if (t >= tiles || !tile_rep[t] || skip_uni[t]) return;  // tiles of one shift: the group kernel's
   const int g = t * 32 + lane;
   const double sg = sigma[g];
   bool tiny = false;  // a value of this system too small for float pairs
@@ -887,153 +936,6 @@ __global__ void __launch_bounds__(BU * 32, 2)
         float2 a = df_axpy(sp.x, cp.x, sgp.x, sgp.y, sp.y, cp.y);  // S x + sigma M x
         emit(i, a.x, a.y, fmaf(sgp.x, b2, b1));
       }
-    }
-  }
-  block_reduce((double)acc, part, t);
-  __syncthreads();
-  block_reduce(tiny && mine ? HUGE_VAL : (double)accb, part_bound, t);  // +inf fails the caller's error check
-}
-
-// The same residual for a tile with a few distinct shifts (ragged sample counts of
-// eight or more pack two to four sinc nodes into a tile): the rows are combined
-// once per block for each of the shifts, A_d = S + sigma_d M, and a lane reads the
-// table of its own, so that one sum is formed instead of two.  The tables lie
-// 16 bytes apart modulo the banks: a warp's read of up to four of them costs no
-// more than one's.  Dynamic shared memory for `nd` shifts.
-template <int P>
-struct DfFewLayout {
-  static constexpr int BV = BvOf<P>::value;
-  static constexpr int CU = BU + 2 * P, CV = BV + 2 * P, NC = CU * CV, S2 = (2 * P + 1) * (2 * P + 1);
-  static constexpr int NPS = BU * (BV / 2) * S2;                            // row-pair entries of a table
-  static constexpr size_t win = (size_t)NC * 32 * sizeof(double);           // x window (raw rows at set-up)
-  static constexpr size_t ids = (size_t)(NC + BU * BV) * sizeof(int);
-  static constexpr size_t total(int nd) { return win + ids + (size_t)nd * (NPS + 1) * sizeof(float4); }
-  static_assert((size_t)BU * BV * S2 * sizeof(float4) <= win, "the raw rows are staged in the window area");
-  static_assert(win % 16 == 0 && ids % 16 == 0, "aligned tables");
-};
-
-template <int P>
-__global__ void __launch_bounds__(BU * 32, 2)
-    k_sten_trueres_df_few(StenGeo G, const float4* __restrict__ cdf, const double* __restrict__ x, int tiles,
-                          const int* __restrict__ tile_rep, const int* __restrict__ few, int nd,
-                          const int* __restrict__ sid, const double* __restrict__ sigma,
-                          const double* __restrict__ rhs, const int* __restrict__ src_of,
-                          const int* __restrict__ rep, float* __restrict__ r, double* __restrict__ part,
-                          double* __restrict__ part_bound) {
-  wm_wait_previous();
-  using LY = DfFewLayout<P>;
-  constexpr int BV = LY::BV, SW = 2 * P + 1, CU = LY::CU, NC = LY::NC, S2 = LY::S2, NPS = LY::NPS;
-  constexpr int NT = BU * 32;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  double* smd = reinterpret_cast<double*>(smraw);
-  float2* smf = reinterpret_cast<float2*>(smraw);  // the same cells after the split
-  float4* sraw = reinterpret_cast<float4*>(smraw);  // set-up only
-  int* scell = reinterpret_cast<int*>(smraw + LY::win);
-  int* srow = scell + NC;
-  float4* scf = reinterpret_cast<float4*>(smraw + LY::win + LY::ids);  // [nd][NPS + 1]
-  __shared__ int s_tiny[BU][32];
-  __shared__ float2 s_sg[kDfFew];
-  const int lane = threadIdx.x, w = threadIdx.y;
-  const int tid = w * 32 + lane;
-  int b = blockIdx.x;
-  const int bu = b % G.nbu;
-  b /= G.nbu;
-  const int bv = b % G.nbv;
-  const int m = b / G.nbv;
-  const int t = blockIdx.y;
-  if (t >= tiles || !few[t] || !tile_rep[t]) return;
-  const int g = t * 32 + lane;
-  // the tile's distinct shifts in order of their first lanes; d: this lane's
-  const unsigned same = __match_any_sync(0xffffffffu, sid[g]);
-  const int leader = __ffs(same) - 1;
-  const unsigned leaders = __ballot_sync(0xffffffffu, lane == leader);
-  const int d = min(__popc(leaders & ((1u << leader) - 1u)), nd - 1), D = min(__popc(leaders), nd);
-  bool tiny = false;
-  if (w == 0 && lane == leader) s_sg[d] = split_bits(sigma[g], tiny);  // (a tiny shift only loses itself)
-  tiny = false;
-  const bool mine = rep[g] != 0;
-  const int src = src_of[g];
-  // global DOF of every window cell and every output row
-  const int32_t* E = G.ext + (size_t)m * G.ELV * G.ELU;
-  const int32_t* OWN = G.own + (size_t)m * G.nlv * G.nlu;
-  for (int c = tid; c < NC + BU * BV; c += NT) {
-    int v = -1;
-    if (c < NC) {
-      int eu = bu * BU + c % CU, ev = bv * BV + c / CU;
-      if (eu < G.ELU && ev < G.ELV) v = E[(size_t)ev * G.ELU + eu];
-    } else {
-      int o = c - NC;
-      int iu = bu * BU + o % BU, iv = bv * BV + o / BU;
-      if (iu < G.nlu && iv < G.nlv) v = OWN[(size_t)iv * G.nlu + iu];
-    }
-    scell[c] = v;
-  }
-  __syncthreads();
-  for (int c = tid; c < BU * BV * S2; c += NT) {
-    const int gi = srow[c / S2];
-    cp_async16(sraw + c, gi >= 0 ? cdf + (size_t)gi * S2 + c % S2 : cdf, gi >= 0 ? 16 : 0);
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  // combined row pairs of every shift (rows 2jj and 2jj + 1 of a column side by side)
-  for (int c = tid; c < NPS; c += NT) {
-    const int pi = c / S2, sl = c - pi * S2;
-    const int o0 = (pi / BU) * 2 * BU + pi % BU;
-    const float4 q0 = sraw[o0 * S2 + sl], q1 = sraw[(o0 + BU) * S2 + sl];
-    for (int e = 0; e < D; ++e) {
-      const float2 sgp = s_sg[e];
-      const float2 a0 = df_axpy(q0.x, q0.y, sgp.x, sgp.y, q0.z, q0.w);
-      const float2 a1 = df_axpy(q1.x, q1.y, sgp.x, sgp.y, q1.z, q1.w);
-      scf[e * (NPS + 1) + c] = make_float4(a0.x, a1.x, a0.y, a1.y);
-    }
-  }
-  __syncthreads();  // the raw rows are dead: the window area is free
-  for (int c = tid; c < NC * 16; c += NT) {  // x window: 16 chunks of 16 bytes per cell
-    const int part16 = c % 16, cell = c / 16;
-    const int gi = scell[cell];
-    cp_async16(smd + (size_t)cell * 32 + part16 * 2, gi >= 0 ? x + ((size_t)t * G.N + gi) * 32 + part16 * 2 : x,
-               gi >= 0 ? 16 : 0);
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  for (int c = tid; c < NC * 32; c += NT) smf[c] = split_bits(smd[c], tiny);  // lane c % 32 == lane
-  s_tiny[w][lane] = tiny;
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < BU; ++k) tiny |= s_tiny[k][lane] != 0;
-  float acc = 0.f, accb = 0.f;
-  auto emit = [&](int i, float s, float c, float bnd) {
-    if (!mine) return;
-    const float2 bp = split_bits(src >= 0 ? rhs[((size_t)(src / 32) * G.N + i) * 32 + (src % 32)] : 0.0, tiny);
-    float e, de;
-    two_sum(bp.x, -s, e, de);
-    const float rt = __fadd_rn(e, __fadd_rn(de, __fsub_rn(bp.y, c)));
-    r[((size_t)t * G.N + i) * 32 + lane] = rt;
-    acc = fmaf(rt, rt, acc);
-    accb = fmaf(bnd, bnd, accb);
-  };
-  const int iu = bu * BU + w;
-  if (iu < G.nlu) {
-    const float4* const tab = scf + d * (NPS + 1);
-#pragma unroll 1
-    for (int j = 0; j < BV; j += 2) {
-      const int i0 = srow[j * BU + w], i1 = srow[(j + 1) * BU + w];
-      if (i0 < 0 && i1 < 0) continue;  // rows past the patch edge or owned by another patch
-      const float4* cf = tab + (size_t)((j / 2) * BU + w) * S2;  // row pair (j, j+1)
-      const float2* zw = smf + ((size_t)j * CU + w) * 32 + lane;
-      float2 sp = make_float2(0.f, 0.f), cp = make_float2(0.f, 0.f);
-      float b0 = 0.f, b1 = 0.f;
-#pragma unroll
-      for (int dv = 0; dv < SW; ++dv)
-#pragma unroll
-        for (int du = 0; du < SW; ++du) {
-          const float4 q = cf[dv * SW + du];
-          const float2 z0 = zw[(dv * CU + du) * 32], z1 = zw[((dv + 1) * CU + du) * 32];
-          df_acc2(sp, cp, b0, b1, make_float2(q.x, q.y), make_float2(q.z, q.w), make_float2(z0.x, z1.x),
-                  make_float2(z0.y, z1.y));
-        }
-      if (i0 >= 0) emit(i0, sp.x, cp.x, b0);
-      if (i1 >= 0) emit(i1, sp.y, cp.y, b1);
     }
   }
   block_reduce((double)acc, part, t);
@@ -1387,9 +1289,20 @@ int wm_sten_true_residual(const wm_level& L, int np, int p, int tiles, const dou
   return WM_OK;
 }
 
+int wm_sten_dots(const wm_level& L, int np, int p, const int* list, int n, const float* r, const float* z,
+                 const float* q, const int* tile_active, double* part_rz, double* part_zq, int stride,
+                 cudaStream_t s) {
+  for (int k = 0; k < n; k += 65535)  // grid.y limit
+    WM_DISPATCH_P(p, {
+      WM_TRY(wm_launch_next(WM_PC_CGVEC, k_sten_dots<PP>, dim3(np * L.nbu * L.nbv, std::min(65535, n - k)), dim3(32, BU),
+                            0, s, geo_of(L), list + k, r, z, q, tile_active, part_rz, part_zq, stride));
+    });
+  WM_CUDA(cudaGetLastError());
+  return WM_OK;
+}
+
 template <int P>
-static int launch_df(const wm_level& L, int np, int tiles, const UniTiles& ut, const int* sid, const double* sigma,
-                     const double* x,
+static int launch_df(const wm_level& L, int np, int tiles, const UniTiles& ut, const double* sigma, const double* x,
                      const double* rhs, const int* src_of, const int* rep, const int* tile_rep, float* r, double* part,
                      double* part_bound, cudaStream_t s) {
   constexpr size_t sm = DfLayout<P>::total;
@@ -1397,8 +1310,6 @@ static int launch_df(const wm_level& L, int np, int tiles, const UniTiles& ut, c
   static bool configured = false;
   if (!configured) {
     WM_CUDA(cudaFuncSetAttribute(k_sten_trueres_df<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    WM_CUDA(cudaFuncSetAttribute(k_sten_trueres_df_few<P>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)DfFewLayout<P>::total(kDfFew)));
     WM_CUDA(cudaFuncSetAttribute(k_sten_trueres_df_uni<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smu));
     configured = true;
   }
@@ -1417,26 +1328,19 @@ static int launch_df(const wm_level& L, int np, int tiles, const UniTiles& ut, c
       WM_CUDA(cudaGetLastError());
     }
   }
-  const dim3 grid(bx, tiles);
-  if (ut.n_few > 0) {
-    WM_TRY(wm_launch_next(WM_PC_TRUERES, k_sten_trueres_df_few<P>, grid, dim3(32, BU),
-        DfFewLayout<P>::total(ut.few_max), s, geo_of(L), L.d_csmdf.p, x, tiles, tile_rep, ut.few, ut.few_max, sid,
-        sigma, rhs, src_of, rep, r, part, part_bound));
-    WM_CUDA(cudaGetLastError());
-  }
-  if (ut.n + ut.n_few < tiles) {
-    WM_TRY(wm_launch_next(WM_PC_TRUERES, k_sten_trueres_df<P>, grid, dim3(32, BU), sm, s, geo_of(L), L.d_csmdf.p, x,
-        tiles, tile_rep, sigma, rhs, src_of, rep, r, part, part_bound, ut.flag, ut.few));
+  if (ut.n < tiles) {
+    WM_TRY(wm_launch_next(WM_PC_TRUERES, k_sten_trueres_df<P>, dim3(bx, tiles), dim3(32, BU), sm, s, geo_of(L), L.d_csmdf.p, x,
+        tiles, tile_rep, sigma, rhs, src_of, rep, r, part, part_bound, ut.flag));
     WM_CUDA(cudaGetLastError());
   }
   return WM_OK;
 }
 
-int wm_sten_true_residual_df(const wm_level& L, int np, int p, int tiles, const UniTiles& ut, const int* sid, const double* sigma,
+int wm_sten_true_residual_df(const wm_level& L, int np, int p, int tiles, const UniTiles& ut, const double* sigma,
                              const double* x, const double* rhs, const int* src_of, const int* rep,
                              const int* tile_rep, float* r, double* part, double* part_bound, cudaStream_t s) {
   WM_DISPATCH_P(p, {
-    return launch_df<PP>(L, np, tiles, ut, sid, sigma, x, rhs, src_of, rep, tile_rep, r, part, part_bound, s);
+    return launch_df<PP>(L, np, tiles, ut, sigma, x, rhs, src_of, rep, tile_rep, r, part, part_bound, s);
   });
   return WM_OK;
 }

@@ -13,14 +13,11 @@
 // consecutive such tiles with the same shift index, each (first tile, count).
 // A block of the one-shift kernel serves one group (or part of one).
 constexpr int kUniGroup = 8;
-constexpr int kDfFew = 4;
 struct UniTiles {
   const int* flag = nullptr;     // [tiles] 1 where the 32 shifts of the tile are equal
   int n = 0;                     // number of such tiles
   const int2* groups = nullptr;  // [n_groups] (first tile, count), count in 1..kUniGroup
   int n_groups = 0;
-  const int* few = nullptr;      // [tiles] 1 where a tile not of one shift has at most kDfFew shifts
-  int n_few = 0, few_max = 0;    // number of such tiles, most shifts of one
   int waves = 4;                 // grid target: runs are split until the grid has this many waves
 };
 
@@ -61,6 +58,11 @@ int wm_sten_residual(const wm_level& L, int np, int p, int tiles, const double* 
                      cudaStream_t s);
 int wm_sten_apply_pq(const wm_level& L, int np, int p, int tiles, const double* sigma, const double* pv, double* q,
                      const int* tile_active, const UniTiles& ut, double* part, cudaStream_t s);
+// partial sums (r, z) and (z, q) of the n tiles in `list` by the row blocks of the steps
+// above ([tile][stride][32], chunk = spatial block), with their float sums
+int wm_sten_dots(const wm_level& L, int np, int p, const int* list, int n, const float* r, const float* z,
+                 const float* q, const int* tile_active, double* part_rz, double* part_zq, int stride,
+                 cudaStream_t s);
 template <typename Tr>
 int wm_sten_true_residual(const wm_level& L, int np, int p, int tiles, const double* sigma, const double* x,
                           const double* rhs, const int* src_of, const int* rep, const int* tile_rep, Tr* r,
@@ -69,33 +71,35 @@ int wm_sten_true_residual(const wm_level& L, int np, int p, int tiles, const dou
 // arithmetic on the FP32 pipes; part_bound receives the per-block partial
 // sums of ||B||^2 with B_i = sum_j |a_ij| |x_j| (the rounding error of entry i
 // is below 2^-42 B_i), or +inf for a system with a value below 2^-102
-// (one-shift tiles of `ut` by groups, the others one tile per block: with the rows
-// combined for each shift where there are at most kDfFew)
-int wm_sten_true_residual_df(const wm_level& L, int np, int p, int tiles, const UniTiles& ut, const int* sid,
-                             const double* sigma,
-                             const double* x, const double* rhs, const int* src_of, const int* rep,
+// (one-shift tiles of `ut` by groups, the others one tile per block)
+int wm_sten_true_residual_df(const wm_level& L, int np, int p, int tiles, const UniTiles& ut,
+                             const double* sigma, const double* x, const double* rhs, const int* src_of, const int* rep,
                              const int* tile_rep, float* r, double* part, double* part_bound, cudaStream_t s);
 
 // ---- streaming kernels of the float solves (wm_stream.h): every tile, any shifts
 constexpr int kStreamTiles = 4;  // tiles of a block
-// The batch's tiles in groups of up to kStreamTiles consecutive ones, (first
-// tile, count): n[1] groups of one shift, then n[0] of any shifts.
+// The batch's tiles in groups of up to kStreamTiles (tile ids, -1: none): n[0] groups of
+// two pairs of tiles, each pair of one shift, n[1] of tiles of one shift each, then n[2]
+// of tiles of any shifts; `order`: the tiles one by one in the same order, the first n_pair
+// of the pairs, the first n_uni of one shift.
 struct StreamTiles {
-  const int2* groups = nullptr;
-  int n[2] = {0, 0};
-  int tiles = 0;
+  const int4* groups = nullptr;
+  const int* order = nullptr;
+  int n[3] = {0, 0, 0};
+  int tiles = 0, n_pair = 0, n_uni = 0;
 };
 // the grouping: `uni` flags the tiles of one shift, `shift` is its index
-void wm_stream_groups(const std::vector<int>& uni, const std::vector<int>& shift, std::vector<int2>& groups,
-                      int n[2]);
+void wm_stream_groups(const std::vector<int>& uni, const std::vector<int>& shift, std::vector<int4>& groups,
+                      std::vector<int>& order, StreamTiles* st);
 // ST_CHEB     three-term Chebyshev step out = z + c1 (z - prev) + c2 D^{-1} (r - A z)
 //             (c1 = 0 at kstep 0; prev = nullptr there; out may alias prev)
-// ST_CHEBDOT  the same, with the partial sums (r, out) in part and (out, q) in part2
+// ST_CHEBDOT  the same, with the partial sums (r, out) in part and (out, q) in part2 for
+//             the tiles that wm_stream_items counts
 // ST_CHEB1    the first two steps from z = 0 in one pass over z (which is r here):
 //             out1 = z1 = c2_0 D^{-1} r, out = z1 + c1_1 z1 + c2_1 D^{-1} (r - A z1)
 // ST_RESID    out = r - A z
 // ST_APPLY    out = A z, with the partial sums (z, out) in part
-// Partial sums: [tile][item][32], wm_stream_items() items.
+// Partial sums: [tile][item][32], wm_stream_items() items (rows of pstride items).
 enum { ST_CHEB = 0, ST_RESID = 1, ST_APPLY = 2, ST_CHEBDOT = 3, ST_CHEB1 = 4 };
 struct StreamArgs {
   const wm_level* L = nullptr;
@@ -109,12 +113,16 @@ struct StreamArgs {
   const float *z = nullptr, *r = nullptr, *prev = nullptr, *q = nullptr;
   float *out = nullptr, *out1 = nullptr;
   double *part = nullptr, *part2 = nullptr;
+  int pstride = 0;  // items of a tile's row of part (0: wm_stream_items())
   int cat = 0;
   cudaStream_t s = nullptr;
 };
 int wm_stream(int p, int mode, const StreamArgs& a);
 int wm_stream_build(int np, int p, wm_level& L, const std::vector<int32_t>& ext, cudaStream_t s);
-// partial sums per tile and system of the kernels that form dot products, and
-// the most that a solve of up to `tiles` tiles leaves over all its tiles
-int wm_stream_items(const wm_level& L, int np, int p, const StreamTiles& st);
+// whether a diagonal of S + sigma M on the level is beyond the kernels' quotients (wm_quotient.h):
+// the row kernels then do the float steps
+bool wm_stream_far(const wm_level& L, double sigma);
+// partial sums per tile and system of the kernels that form dot products (`fused`: of
+// how many of the first tiles of st.order ST_CHEBDOT forms them), and the most that a solve of up to `tiles` tiles leaves over all its tiles
+int wm_stream_items(const wm_level& L, int np, int p, const StreamTiles& st, int* fused = nullptr);
 size_t wm_stream_part_max(const wm_level& L, int np, int tiles);

@@ -28,7 +28,7 @@ __global__ void k_stream_cols(int64_t n, int nlu, int nlv, int ELV, const int32_
   out[b].coef[e] = v;
   if (e == 0) {
     const int o = row(s - 2 * P);
-    out[b].own = o >= 0 ? 32 * o : -1;
+    out[b].own = o;
     out[b].diag = o >= 0 ? make_float2(dS[o], dM[o]) : make_float2(1.f, 0.f);
   }
 }
@@ -54,6 +54,16 @@ __global__ void k_stream_done(int64_t n, int nlu, int nlv, int ELV, int EU, cons
   done[t] = i >= 0 ? 32 * i : 0;
 }
 
+// largest entry of each of two arrays of positive numbers (as their bits)
+__global__ void k_stream_max(int n, const float* __restrict__ a, const float* __restrict__ b, int* __restrict__ most) {
+  int ma = 0, mb = 0;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    ma = max(ma, __float_as_int(a[i]));
+    mb = max(mb, __float_as_int(b[i]));
+  }
+  atomicMax(most, __reduce_max_sync(0xffffffffu, ma));
+  atomicMax(most + 1, __reduce_max_sync(0xffffffffu, mb));
+}
 
 template <int P>
 int build(int np, wm_level& L, const std::vector<int32_t>& ext, cudaStream_t s) {
@@ -74,24 +84,36 @@ int build(int np, wm_level& L, const std::vector<int32_t>& ext, cudaStream_t s) 
                                    reinterpret_cast<ColRow<P>*>(L.d_st_cols.p)));
   WM_LAUNCH(WM_PC_ASSEMBLY, s, k_stream_diag<<<nb(ne), 256, 0, s>>>(ne, L.d_st_ext.p, L.d_dS32.p, L.d_dM32.p,
                                                                     L.d_st_dext.p));
+  DevBuf<int> most;
+  WM_TRY(most.alloc(2));
+  WM_CUDA(cudaMemsetAsync(most.p, 0, 2 * sizeof(int), s));
+  WM_LAUNCH(WM_PC_ASSEMBLY, s, k_stream_max<<<std::min(nb(L.N), 1024u), 256, 0, s>>>(L.N, L.d_dS32.p, L.d_dM32.p, most.p));
   WM_CUDA(cudaGetLastError());
-  WM_CUDA(cudaStreamSynchronize(s));  // the host table goes out of scope
+  WM_CUDA(cudaMemcpyAsync(L.diag_max, most.p, sizeof(L.diag_max), cudaMemcpyDeviceToHost, s));
+  WM_CUDA(cudaStreamSynchronize(s));  // (the host table goes out of scope)
+  most.release();
   return WM_OK;
 }
 
 }  // namespace
 
 int wm_stream_build(int np, int p, wm_level& L, const std::vector<int32_t>& ext, cudaStream_t s) {
-  if ((int64_t)L.N * 32 * kStreamTiles > INT32_MAX) {  // offsets within a block's tiles are 32-bit
+  if ((int64_t)L.N * 32 * kStreamTiles > INT32_MAX) {
     wm_set_error("level too large for the streaming kernels");
     return WM_ERR_UNSUPPORTED;
   }
   return p == 2 ? build<2>(np, L, ext, s) : build<3>(np, L, ext, s);
 }
 
-int wm_stream_items(const wm_level& L, int np, int p, const StreamTiles& st) {
+bool wm_stream_far(const wm_level& L, double sigma) {
+  return L.sten && !(sigma * L.diag_max[1] + L.diag_max[0] < 0x1p120);
+}
+
+int wm_stream_items(const wm_level& L, int np, int p, const StreamTiles& st, int* fused) {
   bool one = false;
-  return stream_geo(L, np, p, st, true, &one).items;
+  const StreamGeo G = stream_geo(L, np, p, st, true, &one);
+  if (fused) *fused = !one && stream_pairs(G, st) ? st.n_pair : 0;
+  return G.items;
 }
 
 size_t wm_stream_part_max(const wm_level& L, int np, int tiles) {
@@ -115,28 +137,28 @@ int wm_stream(int p, int mode, const StreamArgs& a) {
   return WM_ERR_UNSUPPORTED;
 }
 
-void wm_stream_groups(const std::vector<int>& uni, const std::vector<int>& shift, std::vector<int2>& groups,
-                      int n[2]) {
+void wm_stream_groups(const std::vector<int>& uni, const std::vector<int>& shift, std::vector<int4>& groups,
+                      std::vector<int>& order, StreamTiles* st) {
   const int tiles = (int)uni.size();
-  std::vector<int2> one, mixed;
-  auto same = [&](int a, int b) { return b < tiles && uni[a] && uni[b] && shift[a] == shift[b]; };
-  int t = 0;
-  while (t < tiles) {
-    int len = uni[t] ? 1 : 0;
-    while (len > 0 && len < kStreamTiles && same(t, t + len)) ++len;
-    if (len >= 3) {
-      one.push_back(make_int2(t, len));
-      t += len;
-    } else {
-      if (!mixed.empty() && mixed.back().x + mixed.back().y == t && mixed.back().y < kStreamTiles)
-        mixed.back().y += 1;
-      else
-        mixed.push_back(make_int2(t, 1));
-      t += 1;
+  std::vector<int> one, kinds[3];  // kinds[0]: pairs, two entries each
+  for (int t = 0; t < tiles; ++t) (uni[t] ? one : kinds[2]).push_back(t);
+  for (size_t k = 0; k < one.size(); ++k) {
+    const bool pair = k + 1 < one.size() && shift[one[k]] == shift[one[k + 1]];
+    kinds[pair ? 0 : 1].push_back(one[k]);
+    if (pair) kinds[0].push_back(one[++k]);
+  }
+  groups.clear();
+  order.clear();
+  for (int c = 0; c < 3; ++c) {
+    const std::vector<int>& v = kinds[c];
+    order.insert(order.end(), v.begin(), v.end());
+    st->n[c] = 0;
+    for (size_t k = 0; k < v.size(); k += kStreamTiles, ++st->n[c]) {
+      auto at = [&](size_t j) { return j < v.size() ? v[j] : -1; };
+      groups.push_back(make_int4(at(k), at(k + 1), at(k + 2), at(k + 3)));
     }
   }
-  n[0] = (int)mixed.size();
-  n[1] = (int)one.size();
-  groups = one;
-  groups.insert(groups.end(), mixed.begin(), mixed.end());
+  st->tiles = tiles;
+  st->n_uni = (int)one.size();
+  st->n_pair = (int)kinds[0].size();
 }

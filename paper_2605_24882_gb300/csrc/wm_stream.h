@@ -13,30 +13,37 @@
 // next to each other in a table made for this order; a load of a coefficient
 // serves the block's tiles.
 //
-// NSH = 0: the lanes of a tile may have any shifts.  S z and M z are summed as
-// one packed pair (FFMA2: one instruction per tap, tile and output, the
-// coefficient pair as it lies in memory); the shift enters once per output.
-// NSH = 1: the tiles of the block have one shift.  The warp combines
-// A = S + sigma M of its column one row ahead and one packed instruction serves
-// two tiles.
+// A tile's arithmetic depends on its shifts alone, not on the kernel, the block or the
+// tiles beside it: a solve stops at thresholds, and sums formed another way move a
+// system across one (a field of a batch by 1e-9 of its norm).  A tile of one shift has
+// its rows combined, A = S + sigma M, one sum per output and one weight c2 / diagonal; a
+// tile of several shifts sums S z and M z and divides c2 (r - A z) by the diagonal.  Taps
+// are added window row by window row, left to right.
+// NSH = 2: two pairs of tiles, each of one shift.  The warp combines its column's rows for
+// both shifts one row ahead; a packed instruction (FFMA2) per tap serves a tile of each.
+// NSH = 0: any tiles.  Several shifts: one FFMA2 per tap, tile and output on the pair
+// (S, M) as it lies in memory.  One shift each (`ones`): one FFMA2 for the rows of two
+// tiles, in registers, and one for their sums.
 //
-// What bounds it: the shared-memory pipe (72% busy; per output and tile 5 window
-// reads, 13 / 4 coefficient reads of two wavefronts each, the inputs' copies and
-// reads) and latency at 16 warps per SM, which the 128 registers of the running
-// sums of four tiles allow.  The tile-at-a-time kernel it replaces read every
-// window value 2p+1 times and the coefficients once per tile (26 load wavefronts
-// and 105 instructions per output against 16 and 60).  Chebyshev step, level 0 of
-// the 64 x 64 sphere (p = 2), 568 tiles in runs of eight of one shift: 1.83 -> 1.47 ms
-// (3.2 -> 4.0 TB/s); 256 x 256 torus (p = 3), 72 tiles in such runs 1.09 -> 0.66 ms.
-// Mixed shifts, rate of the level-0 smoothing: 213 systems on the 256 x 256 sphere
-// 1.2 -> 3.1 TB/s, 1136 on the 128 x 128 bicubic one 1.05 -> 1.95.
+// What bounds it: the shared-memory pipe (per output and tile 5 window reads, 13 / 4
+// coefficient reads of two wavefronts each, the inputs' copies and reads: 16 wavefronts
+// and 60 instructions where the tile-at-a-time kernel it replaces took 26 and 105) and
+// latency at 16 warps per SM, which the 128 registers of the running sums of four tiles
+// allow.  Chebyshev step (16 bytes per DOF and system; in brackets that kernel's time):
+// level 0 of the 64 x 64 sphere (p = 2), 568 tiles in runs of eight of one shift 1.52 ms
+// (1.86), 4.9 TB/s; 71 tiles of a shift each 0.26 ms (0.41); 256 x 256 torus (p = 3), 72
+// tiles in runs of two 0.63 ms (1.10), 3.8 TB/s.  Several shifts in a tile: 213 systems
+// on the 256 x 256 sphere 0.44 ms, 3.4 TB/s counted without the tiles' padding; 1152 on
+// the 128 x 128 bicubic sphere 0.73 ms, 2.6 TB/s.
 // Loads straight to registers a row ahead were slower (2.6 ms): the six load
 // scoreboards of a warp make the first use of any value wait for all of them.
 #pragma once
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
+#include "wm_quotient.h"
 #include "wm_solver.h"
 #include "wm_stencil.h"
 
@@ -45,10 +52,14 @@ namespace {
 constexpr int kBU = 8;      // columns of a block, one warp each
 constexpr int kD = 3;       // window rows on their way (two: 1-3% slower)
 constexpr int kNST = kD + 1;
-// Rows whose products a dot sums in float before it goes on in double.  The chunks of
-// the kernels that form dots are multiples of it, so that a system's float sums do not
-// depend on the launch's shape, that is, on how many tiles share the batch.
-constexpr int kGrp = 8;
+// Rows whose products a dot sums in float before it goes on in double: the row blocks of
+// wm_stencil.cu.  The chunks of the kernels that form dots are multiples of it, so that a
+// system's float sums do not depend on the launch's shape, that is, on how many tiles
+// share the batch.
+template <int P>
+struct StGrp {
+  static constexpr int value = P == 2 ? 6 : 8;
+};
 constexpr int kBlocks = 2, kBlocks1 = 4;  // blocks per SM of four tiles and of one (register budgets 128 and 64)
 
 // what a window row holds for one column: the coefficients (S, M) of every
@@ -92,25 +103,18 @@ __device__ __forceinline__ void cp_wait() {
 struct FAcc {
   double d = 0.0;
   float f = 0.f;
-  __device__ __forceinline__ void add(float v) { f += v; }
+  __device__ __forceinline__ void add(float a, float b) { f = fmaf(a, b, f); }
   __device__ __forceinline__ void flush() {
     d += (double)f;
     f = 0.f;
   }
 };
 
-// 1 / d: the hardware's approximation improved by one Newton step
-// x (2 - d x), which leaves it within an ulp (d > 0, a diagonal of S + sigma M)
-__device__ __forceinline__ float recip(float d) {
-  float x;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(x) : "f"(d));
-  return fmaf(x, fmaf(-d, x, 1.f), x);
-}
-
 // rows of an output that the epilogue reads besides the window
-template <int MODE>
+template <int MODE, int NSH>
 struct StIn {
-  static constexpr int value = MODE == ST_CHEBDOT ? 3 : MODE == ST_CHEB ? 2 : MODE == ST_RESID ? 1 : 0;
+  static constexpr int value =
+      MODE == ST_CHEBDOT ? 3 : MODE == ST_CHEB ? 2 : MODE == ST_RESID || (MODE == ST_CHEB1 && NSH == 0) ? 1 : 0;
 };
 // shared memory: kNST stages (a window row and what its step needs, byte
 // offsets within a stage), combined rows, ids
@@ -119,83 +123,133 @@ struct StreamLayout {
   static constexpr int CW = kBU + 2 * P;                 // cells of a window row
   static constexpr int NCELL = (CW + kBU - 1) / kBU;     // cells a warp copies
   static constexpr int CELL = TPB * 32 * (int)sizeof(float);  // bytes of a cell
-  static constexpr int NIN = StIn<MODE>::value;
+  static constexpr int NIN = StIn<MODE, NSH>::value;
   static constexpr int ORW = CW * CELL;                  // inputs of the output rows, by warp
   static constexpr int COL = ORW + NIN * kBU * CELL;     // ColRow of the columns
   static constexpr int DCL = COL + kBU * (int)sizeof(ColRow<P>);  // ST_CHEB1: diagonals of the cells
   static constexpr int STAGE = DCL + (MODE == ST_CHEB1 ? kBU * NCELL * (int)sizeof(float2) : 0);
   static constexpr int NID = 8;                          // rows of ids (at least 2 kD + 1, a power of two)
   static_assert(NID >= 2 * kD + 1, "ring of ids");
-  static constexpr int CU = ColRow<P>::S2 + 1;           // combined row: A of every tap, Chebyshev weight
+  // combined row: A of every tap, then two weights of the completed output, each for NSH shifts
+  static constexpr int CU = (ColRow<P>::S2 + 2 + 3) / 4 * 4;
   static constexpr int COMB = kNST * STAGE;
-  static constexpr int CHALF = NSH * kBU * CU * (int)sizeof(float2);  // one of two
-  static constexpr int IDS = COMB + 2 * CHALF;           // [NID][kBU] int4
+  static constexpr int CHALF = NSH * kBU * CU * (int)sizeof(float);  // one of two
+  static constexpr int FACT = COMB + 2 * CHALF;  // ST_CHEB1, NSH = 0: [2][kBU * NCELL][TPB] c2_0 / the cells' diagonals
+  static constexpr int FHALF = MODE == ST_CHEB1 && NSH == 0 ? kBU * NCELL * TPB * (int)sizeof(float) : 0;
+  // shifts and Chebyshev coefficients by tile and lane, where there are no registers for them
+  static constexpr bool SPAR = P == 3 && TPB == 4 && NSH == 0;
+  static constexpr int PAR = FACT + 2 * FHALF;
+  // and the double sums of the dot products by tile, warp and lane
+  static constexpr bool SDOT = SPAR && MODE == ST_APPLY;
+  static constexpr int DOTS = PAR + (SPAR ? TPB * 32 * (int)sizeof(float4) : 0);
+  static constexpr int IDS = DOTS + (SDOT ? TPB * kBU * 32 * (int)sizeof(double) : 0);  // [NID][kBU] int4
   static constexpr size_t total = (size_t)IDS + (size_t)NID * kBU * 4 * sizeof(int);
-  static_assert(STAGE % 16 == 0 && CHALF % 16 == 0 && COL % 16 == 0 && DCL % 16 == 0, "aligned regions");
+  static_assert(STAGE % 16 == 0 && CHALF % 16 == 0 && FHALF % 16 == 0 && COL % 16 == 0 && DCL % 16 == 0,
+                "aligned regions");
 };
+
+// what a launch takes besides the level's tables
+struct StreamIo {
+  const double* sigma;
+  const float2* ctab;
+  const int *sid, *tile_active;
+  const float *z, *r, *prev, *q;
+  float *out, *out1;
+  double *part, *part2;
+  const int4* groups;
+  const int* order;
+  int n_one;  // groups [0, n_one) (TPB = 1: tiles) have one shift per tile
+  int g0, kstep, pstride;
+};
+
+// the tiles of group y (-1: none)
+template <int TPB>
+__device__ __forceinline__ void stream_tiles_of(const StreamIo& io, int y, int (&tile)[TPB]) {
+  if constexpr (TPB == 1) {
+    tile[0] = io.order[y];
+  } else {
+    const int4 g = io.groups[y];
+    tile[0] = g.x;
+    tile[1] = g.y;
+    tile[2] = g.z;
+    tile[3] = g.w;
+  }
+}
+
+// A block's work: one spatial chunk of group y.  ones (NSH = 0): the tiles have one shift each.
 template <int P, int MODE, int NSH, int TPB>
-__global__ void __launch_bounds__(kBU * 32, TPB == 1 ? kBlocks1 : kBlocks)
-    k_stream(const StreamGeo G, const double* __restrict__ sigma, const float2* __restrict__ ctab,
-             const int* __restrict__ sid, int kstep, const float* __restrict__ z, const float* __restrict__ r,
-             const float* prev, const float* __restrict__ q, float* out, float* __restrict__ out1,
-             const int2* __restrict__ groups, int g0, const int* __restrict__ tile_active, double* __restrict__ part,
-             double* __restrict__ part2) {
-  wm_wait_previous();
+__device__ __forceinline__ void stream_block(const StreamGeo& G, const StreamIo& io, int y, bool ones) {
   using LY = StreamLayout<P, MODE, NSH, TPB>;
   using CR = ColRow<P>;
   constexpr int SW = CR::SW, S2 = CR::S2, CW = LY::CW, NIN = LY::NIN, STAGE = LY::STAGE, CELL = LY::CELL;
   constexpr bool CHEB = MODE == ST_CHEB || MODE == ST_CHEBDOT;
   constexpr bool CENTRE = MODE != ST_RESID;       // the input at the output row is needed
   constexpr bool DOT = MODE == ST_APPLY || MODE == ST_CHEBDOT;
-  constexpr int NCELL = LY::NCELL, NID = LY::NID, CU = LY::CU;
-  constexpr int NS = NSH == 0 ? TPB : 1;       // shifts that a lane keeps
-  static_assert((TPB == 4 || (TPB == 1 && NSH == 0)) && NCELL == 2, "the copies and the ids per row and warp below");
+  constexpr int NCELL = LY::NCELL, NID = LY::NID, CU = LY::CU, GRP = StGrp<P>::value;
+  constexpr int NS = NSH == 0 ? TPB : NSH;        // shifts that a lane keeps
+  static_assert((TPB == 4 || (TPB == 1 && NSH == 0)) && (NSH == 0 || NSH == 2) && NCELL == 2,
+                "the copies and the ids per row and warp below");
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lane = threadIdx.x, w = __shfl_sync(0xffffffffu, (int)threadIdx.y, 0);
   const int item = blockIdx.x;
   const int bu = item % G.nbu;
   const int vc = (item / G.nbu) % G.nvc, m = item / (G.nbu * G.nvc);
-  const int2 grp = TPB == 1 ? make_int2(g0 + blockIdx.y, 1) : groups[g0 + blockIdx.y];  // (first tile, count)
-  const int t0 = grp.x;
   // src: a tile that is not to be computed stands in for one that is: the same
-  // inputs, shift and stores
-  int src[TPB];
+  // inputs, shift and stores (NSH = 2: for the other one of its shift first)
+  int src[TPB], tile[TPB];
+  stream_tiles_of(io, y, tile);
+  unsigned act = 0;
+#pragma unroll
+  for (int k = 0; k < TPB; ++k)
+    if (tile[k] >= 0 && io.tile_active[tile[k]]) act |= 1u << k;
+  if (act == 0) return;
   {
-    unsigned act = 0;
+    int first = tile[0];
+#pragma unroll
+    for (int k = TPB - 1; k >= 0; --k)
+      if (act >> k & 1) first = tile[k];
 #pragma unroll
     for (int k = 0; k < TPB; ++k)
-      if (k < grp.y && tile_active[t0 + k]) act |= 1u << k;
-    if (act == 0) return;
-    const int first = __ffs(act) - 1;
-#pragma unroll
-    for (int k = 0; k < TPB; ++k) src[k] = act >> k & 1 ? k : first;
+      src[k] = act >> k & 1 ? tile[k] : NSH == 2 && (act >> (k ^ 1) & 1) ? tile[(k ^ 1) % TPB] : first;
   }
   const int v0 = vc * G.VH;
   const int steps = min(G.nlv - v0, G.VH) + 2 * P;  // window rows
   const int col = bu * kBU + w;
   const bool mine = col < G.ncol;                   // this warp's column exists
-  // shift of lane and tile (NSH = 0) or of the block
+  // the shift of tile k: its lane's (NSH = 0) or one of the block's
+  auto sh = [](int k) { return NSH == 2 ? k / 2 : k; };
   float sg[NS], c1[NS], c2[NS], c0[NS];
 #pragma unroll
   for (int k = 0; k < NS; ++k) {
-    const int g = (t0 + src[k]) * 32 + lane;
-    sg[k] = (float)sigma[g];
+    const int g = src[NSH == 2 ? (2 * k) % TPB : k] * 32 + (NSH == 0 ? lane : 0);
+    sg[k] = (float)io.sigma[g];
     c1[k] = c2[k] = c0[k] = 0.f;
     if constexpr (CHEB) {
-      const float2 c = ctab[sid[g] * WM_MAX_CHEB + kstep];
-      c1[k] = kstep == 0 ? 0.f : c.x;
+      const float2 c = io.ctab[io.sid[g] * WM_MAX_CHEB + io.kstep];
+      c1[k] = io.kstep == 0 ? 0.f : c.x;
       c2[k] = c.y;
     }
-    if constexpr (MODE == ST_CHEB1) {
-      // steps 0 and 1 from z = 0: with z1 = c20 Dinv r the second step is
-      // z1 (1 + c1 + c2 / c20) - c2 Dinv A z1
-      c0[k] = ctab[sid[g] * WM_MAX_CHEB].y;
-      const float2 c = ctab[sid[g] * WM_MAX_CHEB + 1];
-      c1[k] = 1.f + c.x + c.y / c0[k];
+    if constexpr (MODE == ST_CHEB1) {  // steps 0 and 1
+      c0[k] = io.ctab[io.sid[g] * WM_MAX_CHEB].y;
+      const float2 c = io.ctab[io.sid[g] * WM_MAX_CHEB + 1];
+      c1[k] = c.x;
       c2[k] = c.y;
     }
   }
-  auto sh = [](int k) { return NSH == 0 ? k : 0; };  // shift of tile k
+  // the parameters of tile k
+  float4* const spar = reinterpret_cast<float4*>(smraw + LY::PAR) + lane;  // SPAR: {sg, c1, c2, c0}
+  if constexpr (LY::SPAR) {
+    if (w == 0)
+#pragma unroll
+      for (int k = 0; k < TPB; ++k) spar[k * 32] = make_float4(sg[k], c1[k], c2[k], c0[k]);
+    __syncthreads();
+  }
+  auto par = [&](int k) {
+    if constexpr (LY::SPAR)
+      return spar[k * 32];
+    else
+      return make_float4(sg[sh(k)], c1[sh(k)], c2[sh(k)], c0[sh(k)]);
+  };
   // running pointers: ids of the row to copy next (4 bytes by each of four
   // lanes: the warp's cells w, w + kBU, .. < CW, others repeating the first, and
   // the row that the window row completes), the column's ColRow, the cells' diagonals
@@ -205,30 +259,24 @@ __global__ void __launch_bounds__(kBU * 32, TPB == 1 ? kBlocks1 : kBlocks)
   const char* cp = reinterpret_cast<const char*>(reinterpret_cast<const CR*>(G.cols) +
                                                  ((size_t)m * G.ELV + v0) * G.ncol + col) + lane * 16;
   const unsigned cstep = (unsigned)G.ncol * (unsigned)sizeof(CR);
-  const size_t tb = (size_t)t0 * G.N * 32;
-  const unsigned ts = (unsigned)G.N * 32u;  // tile stride
+  const size_t ts = (size_t)G.N * 32;  // tile stride
   // this lane's part of a row of 32 systems: 16-byte chunk lane % 8; with four
   // tiles of tile lane / 8, with one of the cells (0, 1), r (2) and prev (3)
-  size_t cofs = tb + (size_t)((lane % 8) * 4);
   const int lq = lane / 8;
+  size_t cofs = (size_t)src[0] * ts;
   if constexpr (TPB == 4) {
 #pragma unroll
-    for (int k = 0; k < TPB; ++k)
-      if (lq == k) cofs += (unsigned)src[k] * ts;
+    for (int k = 1; k < TPB; ++k)
+      if (lq == k) cofs = (size_t)src[k] * ts;
   }
-  z += cofs;
-  if constexpr (NIN > 0) r += cofs;
-  if constexpr (NIN > 1) prev += cofs;
-  if constexpr (NIN > 2) q += cofs;
-  const float* one = lq < 2 || NIN == 0 ? z : lq == 2 || NIN == 1 ? r : prev;  // TPB = 1: this lane's source
+  cofs += (lane % 8) * 4;
+  const float* const one =  // TPB = 1: this lane's source
+      (lq < 2 || NIN == 0 ? io.z : lq == 2 || NIN == 1 ? io.r : io.prev) + cofs;
   const bool one_on = lq == 0 || (lq == 1 && w + kBU < CW) || (lq == 2 && NIN > 0 && mine) || (lq == 3 && NIN > 1 && mine);
   const unsigned one_to = lq < 2 ? (w + lq * kBU) * CELL : LY::ORW + (w * NIN + lq - 2) * CELL;
-  float *ot[TPB], *ot1[TPB];
+  unsigned row0[TPB];  // first row of 32 systems of the tile stored to
 #pragma unroll
-  for (int k = 0; k < TPB; ++k) {
-    ot[k] = out + tb + (unsigned)src[k] * ts + lane;
-    ot1[k] = MODE == ST_CHEB1 ? out1 + tb + (unsigned)src[k] * ts + lane : nullptr;
-  }
+  for (int k = 0; k < TPB; ++k) row0[k] = (unsigned)src[k] * (unsigned)G.N;
   const unsigned sbase = (unsigned)__cvta_generic_to_shared(smraw);
   const unsigned sid_ = sbase + LY::IDS + w * 16;
 
@@ -243,18 +291,18 @@ __global__ void __launch_bounds__(kBU * 32, TPB == 1 ? kBlocks1 : kBlocks)
       const uint4 id = *reinterpret_cast<const uint4*>(smraw + LY::IDS + ((s & (NID - 1)) * kBU + w) * 16);
       if constexpr (TPB == 4) {
         const unsigned st = sbase + so + lane * 16;
-        cp16(st + w * CELL, z + id.x);
-        if (w + kBU < CW) cp16(st + (w + kBU) * CELL, z + id.y);
+        cp16(st + w * CELL, io.z + (cofs + id.x));
+        if (w + kBU < CW) cp16(st + (w + kBU) * CELL, io.z + (cofs + id.y));
         if (mine) {
-          if constexpr (NIN > 0) cp16(st + LY::ORW + w * (NIN * CELL), r + id.w);
-          if constexpr (NIN > 1) cp16(st + LY::ORW + w * (NIN * CELL) + CELL, prev + id.w);
-          if constexpr (NIN > 2) cp16(st + LY::ORW + w * (NIN * CELL) + 2 * CELL, q + id.w);
+          if constexpr (NIN > 0) cp16(st + LY::ORW + w * (NIN * CELL), io.r + (cofs + id.w));
+          if constexpr (NIN > 1) cp16(st + LY::ORW + w * (NIN * CELL) + CELL, io.prev + (cofs + id.w));
+          if constexpr (NIN > 2) cp16(st + LY::ORW + w * (NIN * CELL) + 2 * CELL, io.q + (cofs + id.w));
         }
       } else {
         const unsigned st = sbase + so + (lane % 8) * 16;
         if (one_on) cp16(st + one_to, one + (lq == 0 ? id.x : lq == 1 ? id.y : id.w));
         if constexpr (NIN > 2)
-          if (lane < 8 && mine) cp16(st + LY::ORW + (w * NIN + 2) * CELL, q + id.w);
+          if (lane < 8 && mine) cp16(st + LY::ORW + (w * NIN + 2) * CELL, io.q + (cofs + id.w));
       }
       if (mine) {
         const unsigned st = sbase + so + lane * 16;
@@ -269,18 +317,55 @@ __global__ void __launch_bounds__(kBU * 32, TPB == 1 ? kBlocks1 : kBlocks)
     copy_ids(s + kD);
     cp_commit();
   };
-  // A = S + sigma M of this warp's column in the stage at so, and the Chebyshev weight
+  auto of_shift = [](const float (&v)[NS], int k) {
+    float a = v[0];
+#pragma unroll
+    for (int j = 1; j < NS; ++j)
+      if (k == j) a = v[j];
+    return a;
+  };
+  // NSH = 2: A = S + sigma M of this warp's column in the stage at so for both shifts
+  // of the block, and the weights of the output that the row completes: c2 / diagonal
+  // (ST_CHEB1: c2_0 / diagonal and c2 / diagonal; A times c2_0 / the cell's diagonal).
+  // A lane does one division at most.
   auto combine = [&](unsigned so, int half) {
     if constexpr (NSH > 0) {
+      float* const tab = reinterpret_cast<float*>(smraw + LY::COMB + half * LY::CHALF) + w * (CU * NSH);
+      const float2* const cd = reinterpret_cast<const float2*>(smraw + so + LY::COL + w * (int)sizeof(CR));
+      float f0 = 0.f, f1 = 0.f;  // ST_CHEB1: by lane cell (SW: the output) x shift
+      if constexpr (MODE == ST_CHEB1) {
+        static_assert((SW + 1) * NSH <= 32, "lanes");
+        const int i = min(lane / NSH, SW), k = lane % NSH, c = w + i;
+        const float2 d = i < SW ? reinterpret_cast<const float2*>(smraw + so + LY::DCL)[(c % kBU) * NCELL + c / kBU]
+                                : cd[S2];
+        const float dinv = wm_quotient(1.f, fmaf(of_shift(sg, k), d.y, d.x));
+        f0 = of_shift(c0, k) * dinv;
+        f1 = of_shift(c2, k) * dinv;
+      }
 #pragma unroll
-      for (int e0 = 0; e0 < CU; e0 += 32) {
+      for (int e0 = 0; e0 < S2; e0 += 32) {
         const int e = e0 + lane;
-        if (e < CU) {
-          // (entry S2: the diagonal)
-          const float2 v = reinterpret_cast<const float2*>(smraw + so + LY::COL + w * (int)sizeof(CR))[e];
-          float a = v.x + sg[0] * v.y;
-          if ((CHEB || MODE == ST_CHEB1) && e == S2) a = c2[0] * recip(a);
-          reinterpret_cast<float2*>(smraw + LY::COMB + half * LY::CHALF)[w * CU + e] = make_float2(a, a);
+        const float2 v = cd[min(e, S2 - 1)];
+        float a[NS];
+#pragma unroll
+        for (int k = 0; k < NSH; ++k) {
+          a[k] = fmaf(sg[k], v.y, v.x);
+          if constexpr (MODE == ST_CHEB1) a[k] *= __shfl_sync(0xffffffffu, f0, min(e, S2 - 1) / SW * NSH + k);
+        }
+        if (e < S2) reinterpret_cast<float2*>(tab)[e] = make_float2(a[0], a[NS - 1]);
+      }
+      if constexpr (CHEB) {
+        const int k = lane - (32 - NSH);  // the last lanes have no entry (p = 3: of the second pass)
+        if (k >= 0) {
+          const float2 d = cd[S2];
+          tab[S2 * NSH + k] = wm_quotient(of_shift(c2, k), fmaf(of_shift(sg, k), d.y, d.x));
+        }
+      }
+      if constexpr (MODE == ST_CHEB1) {
+        const int k = lane - SW * NSH;
+        if (k >= 0 && k < NSH) {
+          tab[S2 * NSH + k] = f0;
+          tab[(S2 + 1) * NSH + k] = f1;
         }
       }
     }
@@ -294,19 +379,33 @@ __global__ void __launch_bounds__(kBU * 32, TPB == 1 ? kBlocks1 : kBlocks)
   for (int s = 0; s < kD; ++s) copy_row(s, s * STAGE);
   if constexpr (NSH > 0) {
     cp_wait<kD - 1>();
-    __syncwarp();
+    if constexpr (MODE == ST_CHEB1)
+      __syncthreads();  // (diagonals of other warps' cells)
+    else
+      __syncwarp();
     if (mine) combine(0, 0);
   }
 
-  // running sums: (S z, M z) per tile, or two tiles' A z
-  float2 acc[SW][NSH == 0 ? TPB : TPB / 2];
+  // running sums: (S z, M z) per tile, or A z of two tiles (NSH = 2: k and k + 2; ones:
+  // 2k and 2k + 1) or one
+  float2 acc[SW][NSH == 0 ? TPB : 2];
   float zr[SW][TPB];  // the input at the column, a window row per slot
   FAcc dot[TPB], dot2[TPB];
   unsigned so = 0, sprev = kD * STAGE;  // stages of rows s and s - 1
+  double* const sdot = reinterpret_cast<double*>(smraw + LY::DOTS) + w * 32 + lane;
+  if constexpr (LY::SDOT) {
+#pragma unroll
+    for (int k = 0; k < TPB; ++k) sdot[k * (kBU * 32)] = 0.0;
+  }
   auto flush = [&]() {
 #pragma unroll
     for (int k = 0; k < TPB; ++k) {
-      dot[k].flush();
+      if constexpr (LY::SDOT) {
+        sdot[k * (kBU * 32)] += (double)dot[k].f;
+        dot[k].f = 0.f;
+      } else {
+        dot[k].flush();
+      }
       if constexpr (MODE == ST_CHEBDOT) dot2[k].flush();
     }
   };
@@ -318,19 +417,37 @@ __global__ void __launch_bounds__(kBU * 32, TPB == 1 ? kBlocks1 : kBlocks)
       if (s >= steps) break;
       // this thread's copies of row s (NSH > 0: and of row s + 1), ids of row s + kD
       cp_wait<NSH == 0 ? kD - 1 : kD - 2>();
-      if constexpr (MODE == ST_CHEB1) {  // r of this warp's cells becomes z1 = c20 Dinv r
+      if constexpr (MODE == ST_CHEB1 && NSH == 0) {
         __syncwarp();
+        const float2* const dcl = reinterpret_cast<const float2*>(smraw + so + LY::DCL) + w * NCELL;
+        if (ones) {  // c2_0 / diagonal of this warp's cells
+          if (lane < NCELL * TPB) {
+            const int k = lane % TPB;
+            const float2 d = dcl[lane / TPB];
+            float4 pk = par(0);
+            if constexpr (LY::SPAR) {
+              pk = par(k);
+            } else {
 #pragma unroll
-        for (int i = 0; i < NCELL; ++i)
-          if (w + i * kBU < CW) {
-            const float2 d = *reinterpret_cast<const float2*>(smraw + so + LY::DCL + (w * NCELL + i) * 8);
-            float f[NS];
-#pragma unroll
-            for (int k = 0; k < NS; ++k) f[k] = c0[k] * recip(d.x + sg[k] * d.y);
-            float* p = reinterpret_cast<float*>(smraw + so + (w + i * kBU) * CELL) + lane;
-#pragma unroll
-            for (int k = 0; k < TPB; ++k) p[k * 32] *= f[sh(k)];
+              for (int j = 1; j < TPB; ++j)
+                if (k == j) pk = par(j);
+            }
+            reinterpret_cast<float*>(smraw + LY::FACT + (s & 1) * LY::FHALF)[w * (NCELL * TPB) + lane] =
+                pk.w * wm_quotient(1.f, fmaf(pk.x, d.y, d.x));
           }
+        } else {  // their r becomes z1 = c2_0 r / diagonal
+#pragma unroll
+          for (int i = 0; i < NCELL; ++i)
+            if (w + i * kBU < CW) {
+              const float2 d = dcl[i];
+              float* p = reinterpret_cast<float*>(smraw + so + (w + i * kBU) * CELL) + lane;
+#pragma unroll
+              for (int k = 0; k < TPB; ++k) {
+                const float4 pk = par(k);
+                p[k * 32] = wm_quotient(pk.w * p[k * 32], fmaf(pk.x, d.y, d.x));
+              }
+            }
+        }
       }
       __syncthreads();  // row s is there, row s - 1 is no longer read
       copy_row(s + kD, sprev);
@@ -338,79 +455,128 @@ __global__ void __launch_bounds__(kBU * 32, TPB == 1 ? kBlocks1 : kBlocks)
       sprev = so;
       so = so == kD * STAGE ? 0 : so + STAGE;
       if (!mine) continue;
-      if (DOT && s > 2 * P && (s - 2 * P) % kGrp == 0) flush();  // the last kGrp output rows' products
+      if (DOT && s > 2 * P && (s - 2 * P) % GRP == 0) flush();  // the last GRP output rows' products
       if (NSH > 0 && s + 1 < steps) combine(so, (s + 1) & 1);
       const float* zw = reinterpret_cast<const float*>(smraw + sc_ + w * CELL) + lane;
       const CR& R = *reinterpret_cast<const CR*>(smraw + sc_ + LY::COL + w * (int)sizeof(CR));
       const float4* cf = NSH == 0 ? reinterpret_cast<const float4*>(R.coef)
                                   : reinterpret_cast<const float4*>(smraw + LY::COMB + (s & 1) * LY::CHALF) +
-                                        w * (CU / 2);
+                                        w * (CU * NSH / 4);
       float4 c4 = make_float4(0.f, 0.f, 0.f, 0.f);  // the last one holds the diagonal or the weight too
+      // e: tap, k: sum, a z + sum
+      auto add2 = [&](int e, int sl, int k, float2 a, float2 zz) {
+        acc[sl][k] = e == 0 ? __fmul2_rn(a, zz) : __ffma2_rn(a, zz, acc[sl][k]);
+      };
+      auto taps = [&](auto one) {
+        constexpr bool ONE = decltype(one)::value;
+        float sgt[TPB];  // ONE: the tiles' shifts
+        if constexpr (ONE) {
 #pragma unroll
-      for (int du = 0; du < SW; ++du) {
-        float zv[TPB];
-#pragma unroll
-        for (int k = 0; k < TPB; ++k) {
-          zv[k] = zw[(du * TPB + k) * 32];
-          if (CENTRE && du == P) zr[u][k] = zv[k];
+          for (int k = 0; k < TPB; ++k) sgt[k] = par(k).x;
         }
 #pragma unroll
-        for (int dv = 0; dv < SW; ++dv) {
-          const int sl = (u - dv + SW) % SW;  // slot of output row s - dv
-          const int e = du * SW + dv;
-          if (e % 2 == 0) c4 = cf[e / 2];
-          const float2 a = e % 2 == 0 ? make_float2(c4.x, c4.y) : make_float2(c4.z, c4.w);
-          if constexpr (NSH == 0) {
+        for (int du = 0; du < SW; ++du) {
+          float zv[TPB], f[TPB];
 #pragma unroll
-            for (int k = 0; k < TPB; ++k) {
-              const float2 zz = make_float2(zv[k], zv[k]);
-              acc[sl][k] = e == 0 ? __fmul2_rn(a, zz) : __ffma2_rn(a, zz, acc[sl][k]);
-            }
-          } else {
+          for (int k = 0; k < TPB; ++k) {
+            zv[k] = zw[(du * TPB + k) * 32];
+            if (CENTRE && du == P) zr[u][k] = zv[k];
+          }
+          if constexpr (ONE && MODE == ST_CHEB1) {
+            const int c = w + du;
+            const float* const fc = reinterpret_cast<const float*>(smraw + LY::FACT + (s & 1) * LY::FHALF) +
+                                    ((c % kBU) * NCELL + c / kBU) * TPB;
 #pragma unroll
-            for (int k = 0; k < TPB / 2; ++k) {
-              const float2 zz = make_float2(zv[2 * k], zv[2 * k + 1]);
-              acc[sl][k] = e == 0 ? __fmul2_rn(a, zz) : __ffma2_rn(a, zz, acc[sl][k]);
+            for (int k = 0; k < TPB; ++k) f[k] = fc[k];
+          }
+#pragma unroll
+          for (int dv = 0; dv < SW; ++dv) {
+            const int sl = (u - dv + SW) % SW;  // slot of output row s - dv
+            const int e = du * SW + dv;
+            if (e % 2 == 0) c4 = cf[e / 2];
+            const float2 a = e % 2 == 0 ? make_float2(c4.x, c4.y) : make_float2(c4.z, c4.w);
+            if constexpr (NSH == 2) {
+              add2(e, sl, 0, a, make_float2(zv[0], zv[2 % TPB]));
+              add2(e, sl, 1, a, make_float2(zv[1 % TPB], zv[3 % TPB]));
+            } else if constexpr (!ONE) {
+#pragma unroll
+              for (int k = 0; k < TPB; ++k) add2(e, sl, k, a, make_float2(zv[k], zv[k]));
+            } else if constexpr (TPB == 1) {
+              float A = fmaf(sgt[0], a.y, a.x);
+              if constexpr (MODE == ST_CHEB1) A *= f[0];
+              acc[sl][0].x = e == 0 ? A * zv[0] : fmaf(A, zv[0], acc[sl][0].x);
+            } else {
+#pragma unroll
+              for (int k = 0; k < TPB / 2; ++k) {
+                float2 A = __ffma2_rn(make_float2(sgt[2 * k], sgt[2 * k + 1]), make_float2(a.y, a.y),
+                                      make_float2(a.x, a.x));
+                if constexpr (MODE == ST_CHEB1) A = __fmul2_rn(A, make_float2(f[2 * k], f[2 * k + 1]));
+                add2(e, sl, k, A, make_float2(zv[2 * k], zv[2 * k + 1]));
+              }
             }
           }
         }
+      };
+      if constexpr (NSH == 0) {
+        if (ones)
+          taps(std::true_type{});
+        else
+          taps(std::false_type{});
+      } else {
+        taps(std::false_type{});
       }
       const int own = s >= 2 * P ? R.own : -1;  // the output row that row s completes
       if (own < 0) continue;
       const int sl = (u + 1) % SW;              // output row s - 2p
       const int sc = (u - P + SW) % SW;         // its centre row
       const float* orr = reinterpret_cast<const float*>(smraw + sc_ + LY::ORW + w * (NIN * CELL)) + lane;
+      float2 w2 = make_float2(0.f, 0.f);  // NSH = 2, ST_CHEB1: the second weights
+      if constexpr (NSH == 2 && MODE == ST_CHEB1) w2 = reinterpret_cast<const float2*>(cf)[S2 + 1];
 #pragma unroll
       for (int k = 0; k < TPB; ++k) {
-        float az, wt;  // A z and c2 / diagonal
-        if constexpr (NSH == 0) {
-          az = acc[sl][k].x + sg[k] * acc[sl][k].y;
-          wt = CHEB || MODE == ST_CHEB1 ? c2[k] * recip(c4.z + sg[k] * c4.w) : 0.f;
+        const float4 pk = par(k);  // sg, c1, c2, c0
+        float az;
+        if constexpr (NSH == 2) {
+          az = k < 2 ? acc[sl][k % 2].x : acc[sl][k % 2].y;
         } else {
-          az = k % 2 == 0 ? acc[sl][k / 2].x : acc[sl][k / 2].y;
-          wt = c4.z;
+          const float one = TPB == 1 ? acc[sl][0].x : k % 2 == 0 ? acc[sl][k / 2].x : acc[sl][k / 2].y;
+          az = ones ? one : fmaf(pk.x, acc[sl][k].y, acc[sl][k].x);
         }
+        const float diag = NSH == 0 ? fmaf(pk.x, c4.w, c4.z) : 1.f;
         const float rv = NIN > 0 ? orr[k * 32] : 0.f;
         float res;
         if constexpr (CHEB) {
           const float zc = zr[sc][k];
-          const float pv = orr[(TPB + k) * 32];
-          res = zc + c1[sh(k)] * (zc - pv) + wt * (rv - az);
+          const float mom = fmaf(pk.y, zc - orr[(TPB + k) * 32], zc);
+          const float d = rv - az;
+          if constexpr (NSH == 0)  // ones: (c2 / diagonal) d, else (c2 d) / diagonal
+            res = fmaf(wm_quotient(pk.z * (ones ? 1.f : d), diag), ones ? d : 1.f, mom);
+          else
+            res = fmaf(k < 2 ? c4.z : c4.w, d, mom);
           if constexpr (MODE == ST_CHEBDOT) {
-            dot[k].add(rv * res);
-            dot2[k].add(res * orr[(2 * TPB + k) * 32]);
+            dot[k].add(rv, res);
+            dot2[k].add(res, orr[(2 * TPB + k) * 32]);
           }
         } else if constexpr (MODE == ST_CHEB1) {
-          const float z1 = zr[sc][k];
-          ot1[k][(unsigned)own] = z1;
-          res = c1[sh(k)] * z1 - wt * az;
+          const float zc = zr[sc][k];  // NSH = 2, ones: r, else z1
+          float z1, wt;
+          if constexpr (NSH == 2) {
+            z1 = (k < 2 ? c4.z : c4.w) * zc;
+            wt = k < 2 ? w2.x : w2.y;
+          } else {
+            const float q = wm_quotient(ones ? 1.f : pk.z * (rv - az), diag);
+            z1 = ones ? pk.w * q * zc : zc;
+            wt = ones ? pk.z * q : q;
+          }
+          io.out1[(size_t)(row0[k] + own) * 32 + lane] = z1;
+          res = fmaf(wt, NSH == 2 || ones ? zc - az : 1.f, fmaf(pk.y, z1, z1));
         } else if constexpr (MODE == ST_RESID) {
           res = rv - az;
         } else {
           res = az;
-          dot[k].add(zr[sc][k] * az);
+          dot[k].add(zr[sc][k], az);
         }
-        ot[k][(unsigned)own] = res;
+        io.out[(size_t)(row0[k] + own) * 32 + lane] = res;
       }
     }
   }
@@ -419,20 +585,35 @@ __global__ void __launch_bounds__(kBU * 32, TPB == 1 ? kBlocks1 : kBlocks)
     double* red = reinterpret_cast<double*>(smraw);  // [TPB][kBU][32]
     static_assert(LY::total >= sizeof(double) * TPB * kBU * 32, "reduction buffer");
     cp_wait<0>();
+    stream_tiles_of(io, y, tile);  // (again: the registers are short in the loop)
     for (int h = 0; h < (MODE == ST_CHEBDOT ? 2 : 1); ++h) {
       __syncthreads();
 #pragma unroll
-      for (int k = 0; k < TPB; ++k) red[(k * kBU + w) * 32 + lane] = h == 0 ? dot[k].d : dot2[k].d;
+      for (int k = 0; k < TPB; ++k)
+        red[(k * kBU + w) * 32 + lane] = LY::SDOT ? sdot[k * (kBU * 32)] : h == 0 ? dot[k].d : dot2[k].d;
       __syncthreads();
-      for (int k = w; k < TPB; k += kBU) {
-        if (!(k < grp.y && tile_active[t0 + k])) continue;
+#pragma unroll
+      for (int k = 0; k < TPB; ++k) {
+        if (w != k || tile[k] < 0 || !io.tile_active[tile[k]]) continue;
         double a = 0.0;
 #pragma unroll
         for (int y = 0; y < kBU; ++y) a += red[(k * kBU + y) * 32 + lane];
-        (h == 0 ? part : part2)[((size_t)(t0 + k) * G.items + item) * 32 + lane] = a;
+        (h == 0 ? io.part : io.part2)[((size_t)tile[k] * io.pstride + item) * 32 + lane] = a;
       }
     }
   }
+}
+
+// The groups of a launch: pairs of tiles of one shift, two to a block (NSH = 2), or
+// (NSH = 0) tiles of one shift each, then tiles of any shifts, four or one to a block.
+// The dot products at a V-cycle's end of the tiles of NSH = 0 are other kernels'
+// (wm_sten_dots, k_dots_rz_zq).
+template <int P, int MODE, int NSH, int TPB>
+__global__ void __launch_bounds__(kBU * 32, TPB == 1 ? kBlocks1 : kBlocks)
+    k_stream(const __grid_constant__ StreamGeo G, const __grid_constant__ StreamIo io) {
+  wm_wait_previous();
+  const int y = io.g0 + blockIdx.y;
+  stream_block<P, MODE, NSH, TPB>(G, io, y, y < io.n_one);
 }
 
 // Shape of a launch.  Where the strips x groups of four tiles give every SM a block,
@@ -468,11 +649,12 @@ StreamGeo stream_geo(const wm_level& L, int np, int p, const StreamTiles& st, bo
   G.ncol = L.nlu;
   G.nbu = strips(L);
   G.EU = G.nbu * kBU + 2 * p;
-  const int64_t strip = (int64_t)np * G.nbu, base4 = strip * std::max(1, st.n[0] + st.n[1]);
+  const int64_t strip = (int64_t)np * G.nbu, base4 = strip * std::max(1, st.n[0] + st.n[1] + st.n[2]);
+  const int grp = p == 2 ? StGrp<2>::value : StGrp<3>::value;
   *one = false;
   auto split = [&](int chunks) {
     G.VH = (L.nlv + chunks - 1) / chunks;
-    if (dot) G.VH = (G.VH + kGrp - 1) / kGrp * kGrp;
+    if (dot) G.VH = (G.VH + grp - 1) / grp * grp;
     G.nvc = (L.nlv + G.VH - 1) / G.VH;
   };
   if (base4 >= kSMs) {
@@ -501,8 +683,17 @@ StreamGeo stream_geo(const wm_level& L, int np, int p, const StreamTiles& st, bo
   return G;
 }
 
+// Whether the pairs of tiles of one shift have a launch of their own: always without
+// other tiles, else where it has four waves of blocks (a launch waits for its longest block:
+// 100 samples on the 128 x 64 bicubic torus 101 ms a call, with a launch at any number of
+// blocks 117; on the 128 x 128 sphere 229 ms, never with one 244)
+bool stream_pairs(const StreamGeo& G, const StreamTiles& st) {
+  return st.n[0] > 0 && (st.n[1] + st.n[2] == 0 || (int64_t)st.n[0] * G.items >= 4 * kSMs * kBlocks);
+}
+
+// groups [g0, g0 + n)
 template <int P, int MODE, int NSH, int TPB>
-int launch_stream_n(const StreamArgs& a, const StreamGeo& G, const int2* groups, int n) {
+int launch_stream_n(const StreamArgs& a, const StreamGeo& G, StreamIo io, int g0, int n) {
   if (n <= 0) return WM_OK;
   constexpr size_t sm = StreamLayout<P, MODE, NSH, TPB>::total;
   static bool configured = false;
@@ -510,22 +701,43 @@ int launch_stream_n(const StreamArgs& a, const StreamGeo& G, const int2* groups,
     WM_CUDA(cudaFuncSetAttribute(k_stream<P, MODE, NSH, TPB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     configured = true;
   }
-  for (int g0 = 0; g0 < n; g0 += 65535) {  // grid.y limit
-    WM_TRY(wm_launch_next(a.cat, (k_stream<P, MODE, NSH, TPB>), dim3(G.items, std::min(65535, n - g0)), dim3(32,
-        kBU), sm, a.s, G, a.sigma, a.ctab, a.sid, a.kstep, a.z, a.r, a.prev, a.q, a.out, a.out1, groups, g0,
-        a.tile_active, a.part, a.part2));
+  for (int k = 0; k < n; k += 65535) {  // grid.y limit
+    io.g0 = g0 + k;
+    WM_TRY(wm_launch_next(a.cat, (k_stream<P, MODE, NSH, TPB>), dim3(G.items, std::min(65535, n - k)), dim3(32, kBU), sm,
+                          a.s, G, io));
     WM_CUDA(cudaGetLastError());
   }
   return WM_OK;
 }
 template <int P, int MODE>
 int launch_stream(const StreamArgs& a) {
-  const int* n = a.st.n;
   bool one = false;
   const StreamGeo G = stream_geo(*a.L, a.np, P, a.st, MODE == ST_APPLY || MODE == ST_CHEBDOT, &one);
-  if (one) return launch_stream_n<P, MODE, 0, 1>(a, G, nullptr, a.st.tiles);
-  WM_TRY((launch_stream_n<P, MODE, 1, kStreamTiles>(a, G, a.st.groups, n[1])));
-  return launch_stream_n<P, MODE, 0, kStreamTiles>(a, G, a.st.groups + n[1], n[0]);
+  StreamIo io;
+  io.sigma = a.sigma;
+  io.ctab = a.ctab;
+  io.sid = a.sid;
+  io.tile_active = a.tile_active;
+  io.z = a.z;
+  io.r = a.r;
+  io.prev = a.prev;
+  io.q = a.q;
+  io.out = a.out;
+  io.out1 = a.out1;
+  io.part = a.part;
+  io.part2 = a.part2;
+  io.groups = a.st.groups;
+  io.order = a.st.order;
+  io.g0 = 0;
+  io.kstep = a.kstep;
+  io.pstride = a.pstride > 0 ? a.pstride : G.items;
+  constexpr int REST = MODE == ST_CHEBDOT ? ST_CHEB : MODE;
+  const int* n = a.st.n;
+  io.n_one = one ? a.st.n_uni : n[0] + n[1];
+  if (one) return launch_stream_n<P, REST, 0, 1>(a, G, io, 0, a.st.tiles);
+  const int pairs = stream_pairs(G, a.st) ? n[0] : 0;  // in a launch of their own
+  WM_TRY((launch_stream_n<P, MODE, 2, kStreamTiles>(a, G, io, 0, pairs)));
+  return launch_stream_n<P, REST, 0, kStreamTiles>(a, G, io, pairs, n[0] + n[1] + n[2] - pairs);
 }
 
 }  // namespace
