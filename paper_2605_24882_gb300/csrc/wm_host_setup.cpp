@@ -887,6 +887,8 @@ int wm_host_stencil(const wm_geom_desc& g, int np, const wm_level& L, std::vecto
   const int nlu = L.nlu, nlv = L.nlv;
   const int ELU = nlu + 2 * p, ELV = nlv + 2 * p;
   const int SW = 2 * p + 1;
+  // offsets within a tile (32 per DOF) are 32-bit in the stencil kernels
+  if ((int64_t)L.N * WM_LANES > INT32_MAX) return WM_ERR_UNSUPPORTED;
   ext.assign((size_t)np * ELV * ELU, -1);
   own.assign((size_t)np * nlv * nlu, -1);
   if (wm_periodic(g.kind)) {

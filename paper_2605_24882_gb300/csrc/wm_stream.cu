@@ -98,10 +98,6 @@ int build(int np, wm_level& L, const std::vector<int32_t>& ext, cudaStream_t s) 
 }  // namespace
 
 int wm_stream_build(int np, int p, wm_level& L, const std::vector<int32_t>& ext, cudaStream_t s) {
-  if ((int64_t)L.N * 32 * kStreamTiles > INT32_MAX) {
-    wm_set_error("level too large for the streaming kernels");
-    return WM_ERR_UNSUPPORTED;
-  }
   return p == 2 ? build<2>(np, L, ext, s) : build<3>(np, L, ext, s);
 }
 
