@@ -686,12 +686,12 @@ __global__ void __launch_bounds__(BU * 32)
 //    (FMA) plus the two cross terms; the rounded products are summed with
 //    Knuth's two-sum and all errors gathered in a float tail (about 48
 //    significant bits for the stencil sum);
-//  * where the 32 shifts of a tile are equal (sample-major packing) each
-//    coefficient row is combined once per block into A = S + sigma M in the
-//    same arithmetic and one sum is formed, two output rows at a time on the
-//    packed FP32 instructions (FMUL2/FFMA2/FADD2, rounding per component as
-//    the scalar ones); otherwise S x and M x are the two packed sums and are
-//    combined per output.
+//  * where the 32 shifts of a tile are equal (sample-major packing;
+//    k_sten_trueres_df_uni) each coefficient row is combined once per block
+//    into A = S + sigma M in the same arithmetic and one sum is formed, two
+//    output rows at a time on the packed FP32 instructions (FMUL2/FFMA2/FADD2,
+//    rounding per component as the scalar ones); otherwise (k_sten_trueres_df)
+//    S x and M x are the two packed sums and are combined per output.
 // Each output also accumulates B_i = sum_j |a_ij x_j| (float, from the rounded
 // hi products, within a factor 1 + 2^-22 of the exact sum): the entry's
 // rounding error stays below 2^-42 B_i (operand splits 2^-47 and 2^-48,
@@ -841,42 +841,10 @@ __global__ void __launch_bounds__(BU * 32, 2)
   }
   cp_async_wait_all();
   __syncthreads();
-  // split x in place; combine the rows when the tile's shifts are equal
+  // split x in place
   __shared__ int s_tiny[BU][32];
   for (int c = tid; c < NC * 32; c += BU * 32) smf[c] = split_bits(smd[c], tiny);  // lane c % 32 == lane
   s_tiny[w][lane] = tiny;
-  // equal shifts compared bit for bit (the same answer in every warp of the
-  // block); both shuffles run on all 32 lanes before any comparison
-  const int sgh = __double2hiint(sg), sgl = __double2loint(sg);
-  const int sgh0 = __shfl_sync(0xffffffffu, sgh, 0);
-  const int sgl0 = __shfl_sync(0xffffffffu, sgl, 0);
-  const bool uni = __all_sync(0xffffffffu, (sgh == sgh0) & (sgl == sgl0));
-  if (uni) {
-    // combined rows A = S + sigma M, rewritten in place as row pairs: entry
-    // (pair jj*BU + w, slot) = (A_hi of rows 2jj and 2jj+1, A_lo of both), the
-    // operand layout of the packed two-row loop below
-    constexpr int NPS = BU * (BV / 2) * S2;            // pair-slot entries
-    constexpr int KPT = (NPS + BU * 32 - 1) / (BU * 32);  // per thread
-    float4 pv[KPT];
-#pragma unroll
-    for (int k = 0; k < KPT; ++k) {
-      const int c = tid + k * BU * 32;
-      if (c < NPS) {
-        const int pi = c / S2, sl = c - pi * S2;
-        const int o0 = (pi / BU) * 2 * BU + pi % BU;  // rows 2jj and 2jj+1 of column w
-        const float4 q0 = scf[o0 * S2 + sl], q1 = scf[(o0 + BU) * S2 + sl];
-        const float2 a0 = df_axpy(q0.x, q0.y, sgp.x, sgp.y, q0.z, q0.w);
-        const float2 a1 = df_axpy(q1.x, q1.y, sgp.x, sgp.y, q1.z, q1.w);
-        pv[k] = make_float4(a0.x, a1.x, a0.y, a1.y);
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < KPT; ++k) {
-      const int c = tid + k * BU * 32;
-      if (c < NPS) scf[c] = pv[k];
-    }
-  }
   __syncthreads();
 #pragma unroll
   for (int k = 0; k < BU; ++k) tiny |= s_tiny[k][lane] != 0;
@@ -892,28 +860,7 @@ __global__ void __launch_bounds__(BU * 32, 2)
     acc = fmaf(rt, rt, acc);
     accb = fmaf(bnd, bnd, accb);
   };
-  if (iu < G.nlu && uni) {
-#pragma unroll 1
-    for (int j = 0; j < BV; j += 2) {
-      const int i0 = srow[j * BU + w], i1 = srow[(j + 1) * BU + w];
-      if (i0 < 0 && i1 < 0) continue;  // rows past the patch edge or owned by another patch
-      const float4* cf = scf + (size_t)((j / 2) * BU + w) * S2;  // row pair (j, j+1)
-      const float2* zw = smf + ((size_t)j * CU + w) * 32 + lane;
-      float2 sp = make_float2(0.f, 0.f), cp = make_float2(0.f, 0.f);
-      float b0 = 0.f, b1 = 0.f;
-#pragma unroll
-      for (int dv = 0; dv < SW; ++dv)
-#pragma unroll
-        for (int du = 0; du < SW; ++du) {
-          const float4 q = cf[dv * SW + du];
-          const float2 z0 = zw[(dv * CU + du) * 32], z1 = zw[((dv + 1) * CU + du) * 32];
-          df_acc2(sp, cp, b0, b1, make_float2(q.x, q.y), make_float2(q.z, q.w), make_float2(z0.x, z1.x),
-                  make_float2(z0.y, z1.y));
-        }
-      if (i0 >= 0) emit(i0, sp.x, cp.x, b0);
-      if (i1 >= 0) emit(i1, sp.y, cp.y, b1);
-    }
-  } else if (iu < G.nlu) {
+  if (iu < G.nlu) {
 #pragma unroll 1
     for (int j = 0; j < BV; ++j) {
       const int i = srow[j * BU + w];
@@ -923,7 +870,7 @@ __global__ void __launch_bounds__(BU * 32, 2)
       // S x and M x side by side on the packed instructions
       float2 sp = make_float2(0.f, 0.f), cp = make_float2(0.f, 0.f);
       float b1 = 0.f, b2 = 0.f;
-#pragma unroll 1  // a full unroll makes the scheduler hoist every operand load (spills)
+#pragma unroll 4  // (residuals of the 128 x 128 bicubic sphere, 1136 systems: 727 us a launch, unroll 1: 797)
       for (int dv = 0; dv < SW; ++dv)
 #pragma unroll
         for (int du = 0; du < SW; ++du) {
@@ -1107,9 +1054,9 @@ __global__ void k_build_csm(int N, int W, int S2, const int16_t* __restrict__ sl
 }  // namespace
 
 // ====================================================================== host
-// levels whose patches have fewer local DOFs per side keep the row kernels
-// (moving the 10- and 18-wide levels of the sphere to the row kernels was slower:
-// 174.5 and 184.0 against 172.5 ms per bench step)
+// levels whose patches have fewer local DOFs per side keep the row kernels (with the
+// tile-at-a-time kernels, moving the 10- and 18-wide levels of the sphere to the row
+// kernels was slower: 174.5 and 184.0 against 172.5 ms per bench step)
 #ifndef WM_STEN_MIN_NL
 #define WM_STEN_MIN_NL 8
 #endif
