@@ -5,7 +5,7 @@ pre- and post-smoothing sweep) on the finest level and on the coarser ones,
 and the ratio r of its interval [lambda_max / r, 1.1 lambda_max].  A higher degree costs more per V-cycle but
 saves outer iterations; the best pair depends on the spline degree, the mesh
 and the shifts.  The kernel schedule of a hierarchy (wm_schedule: tiles per
-run of the one-shift stencil kernels, their grid target in waves, rows per
+run of the float64 stencil and the true-residual kernels, their grid target in waves, rows per
 block of the vector and coarse-level kernels, the fused coarse end of the
 V-cycle) changes how the batched solves
 map onto the SMs, not their results beyond rounding order.

@@ -218,8 +218,8 @@ int wm_k_mass_rows(const wm_level& L, int n, const double* x, double* y, cudaStr
   if (n <= 0 || L.N <= 0) return WM_OK;
   const size_t sm = (size_t)L.W * 33 * (sizeof(double) + sizeof(int32_t));
   constexpr int per = kRowsPerBlock * kMassVec;
-  for (int v0 = 0; v0 < n; v0 += 65535 * per) {  // grid.y limit
-    const int nv = std::min(n - v0, 65535 * per);
+  for (int64_t v0 = 0; v0 < n; v0 += 65535 * per) {  // grid.y limit
+    const int nv = (int)std::min<int64_t>(n - v0, 65535 * per);
     WM_LAUNCH(WM_PC_SINC, s, k_mass_rows<<<dim3((L.N + 31) / 32, (nv + per - 1) / per), kBlock, sm, s>>>(
                                  L.N, L.W, L.d_col.p, L.d_M64.p, x + (size_t)v0 * L.N, y + (size_t)v0 * L.N, nv));
     WM_CUDA(cudaGetLastError());

@@ -1495,6 +1495,8 @@ void WorkSpace::release() {
   prep_shifts.clear();
   prep_lmax = prep_ainv = nullptr;
   n_uni_tiles = n_uni_groups = 0;
+  st = StreamTiles();
+  dots_sten = far = false;
 }
 
 // lambda_max(D^{-1}(S + sigma M)) on every non-coarsest level for each shift,
