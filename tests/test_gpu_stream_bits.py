@@ -89,6 +89,34 @@ def test_dots_of_pairs_singles_and_remainders(split):
     assert float((u - v).norm() / u.norm()) < 1e-11
 
 
+@pytest.mark.parametrize("cap", [499, 500, 501])
+def test_caps_about_the_number_of_systems(cap):
+    """500 systems of 20 samples: one solve from a cap of 500 on, below it whole tiles and a
+    remainder tile of one shift.  The remainder's company does not enter the fields."""
+    hier = wm.Hierarchy(wm.Geometry("sphere", 2, 16), 5)
+    b = torch.randn((20, hier.num_dofs(0)), dtype=torch.float64, device="cuda",
+                    generator=torch.Generator(device="cuda").manual_seed(4))
+    kw = dict(b=b, kappa=3.0, beta=0.7, sinc_k=0.5, l_lo=-12, l_hi=12, n_samples=20, precision="mixed")
+    u, st = hier.sample_fields(**kw)
+    v, sv = hier.sample_fields(max_systems=cap, **kw)
+    assert st["n_batches"] == 1 and sv["n_batches"] == (1 if cap >= 500 else 2)
+    assert float((u - v).norm() / u.norm()) < 1e-11
+
+
+@pytest.mark.parametrize("surf", [("sphere", 2, 8, 4), ("sphere", 3, 16, 5)])
+def test_thin_float64_row_blocks_keep_the_arithmetic(surf):
+    """Levels of 152 and 218 rows: two tiles take blocks of two warps and two rows, 80 tiles
+    (20 groups) blocks of 16 rows; the same float64 V-cycle bit for bit."""
+    kind, p, nu, levels = surf
+    hier = wm.Hierarchy(wm.Geometry(kind, p, nu), levels)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    r = torch.randn((80 * 32, hier.num_dofs(0)), dtype=torch.float64, device="cuda", generator=g)
+    sg = np.geomspace(1.0, 1e4, len(r))
+    z = hier.vcycle(r, sg, precision="fp64", smoother_degree=3)
+    few = hier.vcycle(r[:64], sg[:64], precision="fp64", smoother_degree=3)
+    assert torch.equal(z[:64], few)
+
+
 @pytest.mark.parametrize("shift", [1e30, 3e37])
 def test_vcycle_at_the_end_of_the_float_range(shift):
     """Diagonals beyond 2^120, which the kernels' quotients do not take (elements of area 3)."""
