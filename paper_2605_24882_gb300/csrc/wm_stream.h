@@ -27,14 +27,14 @@
 //
 // What bounds it: the shared-memory pipe (per output and tile 5 window reads, 13 / 4
 // coefficient reads of two wavefronts each, the inputs' copies and reads: 16 wavefronts
-// and 60 instructions where the tile-at-a-time kernel it replaces took 26 and 105) and
+// and 67 instructions where the tile-at-a-time kernel it replaces took 26 and 105) and
 // latency at 16 warps per SM, which the 128 registers of the running sums of four tiles
 // allow.  Chebyshev step (16 bytes per DOF and system; in brackets that kernel's time):
 // level 0 of the 64 x 64 sphere (p = 2), 568 tiles in runs of eight of one shift 1.52 ms
 // (1.86), 4.9 TB/s; 71 tiles of a shift each 0.26 ms (0.41); 256 x 256 torus (p = 3), 72
 // tiles in runs of two 0.63 ms (1.10), 3.8 TB/s.  Several shifts in a tile: 213 systems
-// on the 256 x 256 sphere 0.44 ms, 3.4 TB/s counted without the tiles' padding; 1152 on
-// the 128 x 128 bicubic sphere 0.73 ms, 2.6 TB/s.
+// on the 256 x 256 sphere 0.44 ms, 3.0 TB/s; 1152 on the 128 x 128 bicubic sphere
+// 0.73 ms, 2.6 TB/s.
 // Loads straight to registers a row ahead were slower (2.6 ms): the six load
 // scoreboards of a warp make the first use of any value wait for all of them.
 #pragma once
