@@ -19,12 +19,13 @@ int main() {
   long bad = 0;
   for (long i = 0; i < 3000000; ++i) {
     s ^= s << 13, s ^= s >> 7, s ^= s << 17;
-    const uint32_t e = 64 + (uint32_t)((s >> 50) % 128);  // exponents 2^(+-63)
+    const uint32_t e = 64 + (uint32_t)((s >> 50) % 183);  // d from 2^-63 to 2^120
+    const uint32_t ea = 27 + (uint32_t)((s >> 40) % 130);  // |a| from 2^-100 to 2^30
     uint32_t m = (uint32_t)s & 0x7fffff, k = (uint32_t)(s >> 23) & 0x7fffff;
     if (i % 7 == 0) m = 0x7fffff - m % 4;  // mantissas at both ends
     if (i % 11 == 0) k = k % 4;
     if (i % 13 == 0) k = 0x7fffff - k % 4;
-    const float a = (i & 1 ? -1.f : 1.f) * f(0x3f800000u | m), d = f(e << 23 | k);
+    const float a = (i & 1 ? -1.f : 1.f) * f(ea << 23 | m), d = f(e << 23 | k);
     const float y = (float)(1.0 / (double)d);
     for (int o = -1; o <= 1; ++o) bad += wm_quotient_from(a, d, f(u(y) + o)) != a / d;
   }
