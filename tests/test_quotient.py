@@ -1,5 +1,5 @@
 """csrc/wm_quotient.h on the host: the quotient equals IEEE division for every reciprocal
-within an ulp that the device may start from."""
+within an ulp that the device may start from (a subnormal quotient within its last bit)."""
 import os
 import shutil
 import subprocess
@@ -27,7 +27,10 @@ int main() {
     if (i % 13 == 0) k = 0x7fffff - k % 4;
     const float a = (i & 1 ? -1.f : 1.f) * f(ea << 23 | m), d = f(e << 23 | k);
     const float y = (float)(1.0 / (double)d);
-    for (int o = -1; o <= 1; ++o) bad += wm_quotient_from(a, d, f(u(y) + o)) != a / d;
+    for (int o = -1; o <= 1; ++o) {
+      const float q = wm_quotient_from(a, d, f(u(y) + o)), t = a / d;
+      bad += std::fabs(t) >= 0x1p-126f ? q != t : !(std::fabs(q - t) <= 0x1p-149f);
+    }
   }
   bad += wm_quotient_from(0.f, 3.f, 1.f / 3.f) != 0.f;
   std::printf("%ld\n", bad);
